@@ -346,6 +346,7 @@ static void run_sigma_tc(Context& c, Problem& p, const double* d_psi, double* d_
   r.items = reinterpret_cast<const Item*>(p.d_tc_items.p);
   r.groups = p.d_tc_groups.as<Group>();
   r.n_groups = (int)p.tc.groups.size();
+  r.max_tile = p.tc.max_tile;
   r.blocks = p.d_blocks.as<PsiBlock>();
   r.scratch = p.d_tc_scratch.as<double>();
   {
@@ -410,6 +411,7 @@ void run_sigma_f64(Context& c, Problem& p, const double* d_psi, double* d_sigma)
   a.n_items = (int)p.wl.items.size();
   a.groups = p.d_groups.as<Group>();
   a.n_groups = (int)p.wl.groups.size();
+  a.max_tile = p.wl.max_tile;
   a.blocks = p.d_blocks.as<PsiBlock>();
   a.scratch = p.d_scratch.as<double>();
   a.counter = p.d_counter.as<unsigned int>();
@@ -458,6 +460,7 @@ void run_sigma_part(Context& c, Problem& p, int rank, int n_ranks, const double*
   a.n_items = (int)w.wl.items.size();
   a.groups = w.d_groups.as<Group>();
   a.n_groups = (int)w.wl.groups.size();
+  a.max_tile = w.wl.max_tile;
   a.blocks = p.d_blocks.as<PsiBlock>();
   a.scratch = w.d_scratch.as<double>();
   a.counter = w.d_counter.as<unsigned int>();

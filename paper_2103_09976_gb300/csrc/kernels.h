@@ -44,8 +44,9 @@ struct SigmaDev {
   int n_items;
   const Group* groups;
   int n_groups;
+  int max_tile;               // elements of the largest group's tile
   const PsiBlock* blocks;
-  double* scratch;
+  double* scratch;            // partial tiles; the items of a group have consecutive slots
   unsigned int* counter;      // must be zero at launch (the caller clears it)
 };
 void launch_sigma_f64(const SigmaDev& a, int n_sm, cudaStream_t st);

@@ -360,6 +360,12 @@ static double tile_cost(const Task& k, const PsiBlock& in, int nr, int nc, doubl
   return c;
 }
 
+int largest_tile(const std::vector<Group>& groups) {
+  int n = 0;
+  for (const Group& g : groups) n = std::max(n, g.nrows * g.ncols);
+  return n;
+}
+
 void build_items(const std::vector<PsiBlock>& blocks, WorkList& wl, const TileShape& ts,
                  int want_items, int n_out) {
   // output blocks are blocks[0, n_out); inputs may follow them
@@ -416,6 +422,7 @@ void build_items(const std::vector<PsiBlock>& blocks, WorkList& wl, const TileSh
       }
     }
   }
+  wl.max_tile = largest_tile(wl.groups);
   wl.schedule.resize(wl.items.size());
   std::iota(wl.schedule.begin(), wl.schedule.end(), 0);
   std::stable_sort(wl.schedule.begin(), wl.schedule.end(),
@@ -783,6 +790,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
       plan.groups[G[j] + k] = g;
     }
   });
+  plan.max_tile = largest_tile(plan.groups);
   for (const Part& P : parts) plan.n_units += (long long)P.units.size();
   std::vector<int> small1;
   for (size_t i = 0; i < plan.items.size(); ++i) {

@@ -201,6 +201,7 @@ struct WorkList {
   std::vector<Group> groups;
   std::vector<int> schedule;      // item indices, most expensive first
   long long scratch_elems = 0;
+  int max_tile = 0;          // elements of the largest group's tile
   double flops = 0;          // algorithmic (min order)
   double bytes_ops = 0;      // operator bytes read (FP64), each product reading its two blocks
   // host only, parallel to tasks: index of each task's left / right stored
@@ -215,6 +216,7 @@ struct TileShape {
   double per_task = 16384.0;  // fixed latency term of one task in the item cost
 };
 
+int largest_tile(const std::vector<Group>& groups);
 void build_tasks(const std::vector<PsiBlock>& blocks, const OpSet& L, const OpSet& R,
                  const std::vector<Term>& terms, WorkList& wl);
 // Split every output block into tm x tn tiles and each tile's task list into
@@ -336,6 +338,7 @@ struct TcPlan {
   std::vector<int> schedule;            // kind-0 items, most expensive first
   std::vector<Group> groups;
   long long scratch_elems = 0;
+  int max_tile = 0;                     // elements of the largest group's tile
   std::vector<TcUnitRec, NoInit<TcUnitRec>> recs;  // kind-0 item i: records [items[i].r_begin, items[i].r_end)
   std::vector<SmallTerm> small;         // kind-1/2 item i: terms [items[i].r_begin, items[i].r_end)
   // per record and term slot (record * TC_MAX_G + q): split-block indices of

@@ -20,6 +20,7 @@
 // (rows, columns) and 4 (k), instead of to whole register micro-tiles.
 // Each warp owns a set of 8x8 sub-tiles of the output tile and of the
 // intermediate chunk; fragments come from shared memory.
+#include <algorithm>
 #include <mutex>
 #include <set>
 #include <string>
@@ -228,17 +229,36 @@ sigma_f64_kernel(SigmaDev a) {
   }
 }
 
-__global__ void reduce_kernel(SigmaDev a) {
-  for (int gi = blockIdx.x; gi < a.n_groups; gi += gridDim.x) {
-    const Group g = a.groups[gi];
-    const PsiBlock ob = a.blocks[g.out];
-    const int n = g.nrows * g.ncols;
-    for (int e = threadIdx.x; e < n; e += blockDim.x) {
-      double acc = 0.0;
-      for (int i = g.i_begin; i < g.i_end; ++i) acc += a.scratch[a.items[i].slot + e];
-      int r = e / g.ncols, c = e % g.ncols;
-      a.sigma[ob.off + (long long)(g.r0 + r) * ob.mR + g.c0 + c] = acc;
+// Sum of every output tile's partial tiles, in item order: blockIdx.x the
+// group, blockIdx.y a run of RED_THREADS elements of its tile (the work lists
+// give the items of a group consecutive slots of one tile each, so element e
+// of the k-th item is at slot + k * n + e). Bound by latency: a tile has 5-30
+// partials of a few thousand elements. One CTA per group walking its items
+// one load at a time took 402 us at K=76, M=2000 (104 groups, BF16X3) and
+// 292 us at K=16, M=150 (31 groups); spreading the elements over CTAs, with
+// RED_UNROLL loads in flight per thread and the same order of additions,
+// takes 21 us and 19 us.
+constexpr int RED_THREADS = 128;
+constexpr int RED_UNROLL = 8;
+__global__ void __launch_bounds__(RED_THREADS) reduce_kernel(SigmaDev a) {
+  const Group g = a.groups[blockIdx.x];
+  const int n = g.nrows * g.ncols, ni = g.i_end - g.i_begin;
+  const PsiBlock ob = a.blocks[g.out];
+  const double* __restrict__ part = a.scratch + a.items[g.i_begin].slot;
+  for (int e = blockIdx.y * RED_THREADS + threadIdx.x; e < n; e += gridDim.y * RED_THREADS) {
+    const double* __restrict__ src = part + e;
+    double acc = 0.0;
+    int k = 0;
+    for (; k + RED_UNROLL <= ni; k += RED_UNROLL) {
+      double v[RED_UNROLL];
+#pragma unroll
+      for (int u = 0; u < RED_UNROLL; ++u) v[u] = src[(long long)(k + u) * n];
+#pragma unroll
+      for (int u = 0; u < RED_UNROLL; ++u) acc += v[u];
     }
+    for (; k < ni; ++k) acc += src[(long long)k * n];
+    const int r = e / g.ncols, c = e - r * g.ncols;
+    a.sigma[ob.off + (long long)(g.r0 + r) * ob.mR + g.c0 + c] = acc;
   }
 }
 
@@ -268,9 +288,13 @@ void launch_sigma_f64(const SigmaDev& a, int n_sm, cudaStream_t st) {
 }
 
 void launch_reduce(const SigmaDev& a, cudaStream_t st) {
-  int grid = a.n_groups < 152 * 8 ? a.n_groups : 152 * 8;
-  if (grid < 1) grid = 1;
-  reduce_kernel<<<grid, 256, 0, st>>>(a);
+  if (a.n_groups < 1 || a.max_tile < 1) return;
+  // a CTA per run of elements until that fills the GPU many times over (a
+  // transformation has one group per operator block, 1e5 and more)
+  int ny = (a.max_tile + RED_THREADS - 1) / RED_THREADS;
+  ny = std::min(ny, std::max(1, 152 * 64 / a.n_groups));
+  const dim3 grid((unsigned)a.n_groups, (unsigned)ny);
+  reduce_kernel<<<grid, RED_THREADS, 0, st>>>(a);
 }
 
 }  // namespace dmrg

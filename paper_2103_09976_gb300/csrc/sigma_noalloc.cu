@@ -89,6 +89,7 @@ void sigma_noalloc(Context& c, Problem& p, const double* psi, double* sigma) {
   a.n_items = (int)p.wl.items.size();
   a.groups = p.d_groups.as<Group>();
   a.n_groups = (int)p.wl.groups.size();
+  a.max_tile = p.wl.max_tile;
   a.blocks = p.d_blocks.as<PsiBlock>();
   a.scratch = s.scratch;
   a.counter = s.counter;

@@ -320,6 +320,7 @@ void transform(Context& c, const OpSet& EO, const double* enl_store, const Basis
   a.n_items = (int)wl.items.size();
   a.groups = d_groups.as<Group>();
   a.n_groups = (int)wl.groups.size();
+  a.max_tile = wl.max_tile;
   a.blocks = d_blocks.as<PsiBlock>();
   a.scratch = d_scratch.as<double>();
   a.counter = d_counter.as<unsigned int>();
