@@ -122,7 +122,7 @@ static_assert(sizeof(TcItem) == sizeof(Item), "reduction reads TcItem as Item");
 // operator store is unchanged by it).
 static void prepare_tc_plan(Context& c, Problem& p) {
   cudaStream_t st = c.stream;
-  build_tc_plan(p.blocks, p.L, p.R, p.wl, p.tc, TcShape{c.n_sm * p.tc_items_per_sm, p.tc_unit_cost});
+  build_tc_plan(p.blocks, p.L, p.R, p.wl, p.tc, TcShape{c.n_sm * p.tc_items_per_sm, p.tc_unit_cost, c.n_sm});
   p.tc_producers[0] = tc_default_producers(p.tc, false);
   p.tc_producers[1] = tc_default_producers(p.tc, true);
   p.d_tc_recs.upload(p.tc.recs, st);

@@ -559,8 +559,15 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
   };
   const double unit_overhead = shape.unit_cost;  // fixed cost of a unit in the item split
   double total = 0;
+  long long n_small[2] = {0, 0};  // CUDA-core terms: all blocks <= TC_SMALL_MID, the rest
   for (size_t b = 0; b < nblk; ++b) {
     const PsiBlock& ob = blocks[b];
+    if (std::max(ob.mL, ob.mR) <= TC_SMALL_MAX)
+      for (int t = wl.out_start[b]; t < wl.out_start[b + 1]; ++t) {
+        const PsiBlock& ib = blocks[base[t].in_blk];
+        const int wmax = std::max(std::max(ob.mL, ob.mR), std::max(ib.mL, ib.mR));
+        if (wmax <= TC_SMALL_MAX) ++n_small[wmax <= TC_SMALL_MID ? 0 : 1];
+      }
     for (int r0 = 0; r0 < ob.mL; r0 += 128)
       for (int c0 = 0; c0 < ob.mR; c0 += 128) {
         const int tm = std::min(128, ob.mL - r0), tn = std::min(128, ob.mR - c0);
@@ -588,7 +595,15 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
     long long n_terms = 0;
     double macs = 0;
   };
-  constexpr int SMALL_ITEM = 512;        // small terms per CUDA-core item
+  // Terms per CUDA-core item: enough items to fill the resident CTAs several
+  // times over (3 per SM of the <= 16 class, 2 of the rest), at least 8 terms
+  // per warp of a CTA (8 or 4 warps) against the cost of an item's final sum
+  // and its partial tile. Against 512 terms always, per kernel of one sigma:
+  // <= 32 class 222 -> 45 us at K=16, M=150 (22 items before), 857 -> 520 us at
+  // K=54, M=1000; <= 16 class 136 -> 67 us at K=24, M=250.
+  int small_item[2];
+  small_item[0] = (int)std::min<long long>(512, std::max<long long>(64, n_small[0] / (shape.n_sm * 12)));
+  small_item[1] = (int)std::min<long long>(512, std::max<long long>(32, n_small[1] / (shape.n_sm * 8)));
   std::vector<Part> parts(nparts);
   in_parallel([&](int j) {
     Part& P = parts[j];
@@ -672,8 +687,8 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
             const size_t base0 = P.small.size();
             P.small.insert(P.small.end(), sm[cls].begin(), sm[cls].end());
             P.small_blk.insert(P.small_blk.end(), smb[cls].begin(), smb[cls].end());
-            for (size_t s0 = base0; s0 < P.small.size(); s0 += SMALL_ITEM) {
-              const size_t s1 = std::min(P.small.size(), s0 + SMALL_ITEM);
+            for (size_t s0 = base0; s0 < P.small.size(); s0 += small_item[cls]) {
+              const size_t s1 = std::min(P.small.size(), s0 + small_item[cls]);
               double c = 0;
               for (size_t q = s0; q < s1; ++q) {
                 const PsiBlock& ib = blocks[P.small[q].in_blk];
