@@ -87,10 +87,21 @@ Problem& need_problem(Context& c, int site) {
 
 namespace dmrg {
 
+// Items of an FP64 sigma: want_items of them, but none below a minimum cost.
+// The minimum of ITEM_MIN (about ten tasks) lets small problems use every SM
+// (K=8, M=64: 34 items of 2e6 took 34 us alone on the same kernel's rate); where that many partial tiles
+// would not fit the fixed scratch of dmrg_sigma_noalloc and larger items do,
+// the larger minimum is kept, so that every problem that call can take it takes.
+static void build_sigma_items(const std::vector<PsiBlock>& blocks, WorkList& wl, int want_items, double per_task) {
+  constexpr double ITEM_MIN = 2e5, ITEM_MIN_LARGE = 2e6;
+  build_items(blocks, wl, TileShape{F64_TM, F64_TN, ITEM_MIN, per_task}, want_items);
+  if (wl.scratch_elems > NOALLOC_DOUBLES)
+    build_items(blocks, wl, TileShape{F64_TM, F64_TN, ITEM_MIN_LARGE, per_task}, want_items);
+}
+
 // Items, groups and scratch of the FP64 work list for the problem's tuning.
 static void prepare_items(Context& c, Problem& p) {
-  TileShape ts{F64_TM, F64_TN, 2e6, p.per_task_cost};
-  build_items(p.blocks, p.wl, ts, c.n_sm * p.items_per_sm);
+  build_sigma_items(p.blocks, p.wl, c.n_sm * p.items_per_sm, p.per_task_cost);
   cudaStream_t st = c.stream;
   p.d_items.upload(p.wl.items, st);
   p.d_groups.upload(p.wl.groups, st);
@@ -102,8 +113,7 @@ static void prepare_items(Context& c, Problem& p) {
 
 void prepare_worklist(Context& c, Problem& p) {
   build_tasks(p.blocks, p.L, p.R, p.terms, p.wl);
-  TileShape ts{F64_TM, F64_TN, 2e6, p.per_task_cost};
-  build_items(p.blocks, p.wl, ts, c.n_sm * p.items_per_sm);
+  build_sigma_items(p.blocks, p.wl, c.n_sm * p.items_per_sm, p.per_task_cost);
   cudaStream_t st = c.stream;
   p.d_tasks.upload(p.wl.tasks, st);
   p.d_items.upload(p.wl.items, st);
@@ -439,7 +449,7 @@ void run_sigma_part(Context& c, Problem& p, int rank, int n_ranks, const double*
     for (size_t t = 0; t < p.terms.size(); ++t)
       if (ranks[t] == rank) mine.push_back(p.terms[t]);
     build_tasks(p.blocks, p.L, p.R, mine, w->wl);
-    build_items(p.blocks, w->wl, TileShape{F64_TM, F64_TN, 2e6}, c.n_sm * 8);
+    build_sigma_items(p.blocks, w->wl, c.n_sm * 8, 16384.0);
     w->d_tasks.upload(w->wl.tasks, st);
     w->d_items.upload(w->wl.items, st);
     w->d_groups.upload(w->wl.groups, st);

@@ -34,6 +34,9 @@ void launch_gen_vector(double* x, long long n, uint64_t key, unsigned long long 
 constexpr int F64_TM = 32;    // output rows per tile
 constexpr int F64_TN = 256;   // output columns per tile (32 groups of 8)
 
+// Partial-tile doubles that dmrg_sigma_noalloc's fixed scratch holds (32 MiB).
+constexpr long long NOALLOC_DOUBLES = 4ll << 20;
+
 struct SigmaDev {
   const double* store;        // operator store (FP64)
   const double* psi;
@@ -50,6 +53,9 @@ struct SigmaDev {
   unsigned int* counter;      // must be zero at launch (the caller clears it)
 };
 void launch_sigma_f64(const SigmaDev& a, int n_sm, cudaStream_t st);
+// The same for a work list with one item per output tile: each item is
+// written straight to a.sigma (scratch and groups unused).
+void launch_sigma_f64_direct(const SigmaDev& a, int n_sm, cudaStream_t st);
 void launch_reduce(const SigmaDev& a, cudaStream_t st);
 
 // ------------------------------------------------------------ tensor cores

@@ -6,20 +6,29 @@
 // persistent CTA takes one work item = (output block tile, run of tasks) and
 // accumulates, for every task,
 //     S[r0:r0+32, c0:c0+nc] += scale * (X_L[r0:, :] psi_b) X_R[c0:, :]^T
-// chunk by chunk (64 columns of the intermediate at a time, the intermediate
-// never leaves shared memory), then writes its partial tile to a private
+// chunk by chunk (32 columns of the intermediate at a time, the intermediate
+// never leaves a warp's registers), then writes its partial tile to a private
 // scratch slot. A second kernel sums each output tile's slots in fixed order
 // (Sec. II.D's final reduction), so sigma is bitwise deterministic whatever
 // the schedule of the items.
 //
 // The FP64 path is bound by the FP64 multiply-add rate, which on this GPU
 // is the same for the FP64 tensor instruction (mma.sync m8n8k4 .f64: 256
-// multiply-adds per warp instruction) and for scalar FMAs. The tensor form
-// is used because its 8x8x4 granularity keeps padding small: every output
-// tile, intermediate chunk and contraction is padded only to multiples of 8
-// (rows, columns) and 4 (k), instead of to whole register micro-tiles.
-// Each warp owns a set of 8x8 sub-tiles of the output tile and of the
-// intermediate chunk; fragments come from shared memory.
+// multiply-adds per warp instruction) and for scalar FMAs: about 1.9 FMAs per
+// cycle and SM, so one such instruction occupies its SM sub-partition for
+// about 540 cycles. The tensor form is used because its 8x8x4 granularity keeps
+// padding small: every output tile, intermediate chunk and contraction is
+// padded only to multiples of 8 (rows, columns) and 4 (k). At that rate a load
+// straight from global memory (L1 / L2) into a fragment is never the limit, so
+// nothing is staged in shared memory and no barrier stands between the warps:
+// a warp owns rows of the tile and a share of the item's tasks, computes the
+// intermediate of 32 columns in registers and feeds it to the second product
+// from the registers it is in (below). Per sigma, against 8 warps sharing
+// operands staged in shared memory with 4 barriers per 32 k steps: 9.6 us
+// (before: 74) at K=8, M=64; 1.92 ms (2.84) at K=36, M=501, with the FP64 pipe
+// busy 75% of one launch (blocks of 1-30 rows, padded to twice their
+// multiply-adds); 22.9 ms (26.3) at K=54, M=1000; 635 ms (658) at K=108,
+// M=2000.
 #include <algorithm>
 #include <mutex>
 #include <set>
@@ -33,31 +42,17 @@ namespace dmrg {
 
 namespace {
 
-constexpr int TM = F64_TM;    // 32 output rows (4 row groups of 8)
-constexpr int TN = F64_TN;    // up to 256 output columns (32 column groups)
-constexpr int NCH = 64;       // intermediate columns per chunk
-constexpr int KC = 32;        // k staging depth of the first product
-constexpr int KC2 = 16;       // k staging depth of the second product
-constexpr int NT = 256;       // threads (8 warps)
-constexpr int NW = NT / 32;
-constexpr int XS = (TM / 8) * (NCH / 8) / NW;  // intermediate sub-tiles per warp (4)
-constexpr int SS = (TM / 8) * (TN / 8) / NW;   // output sub-tiles per warp (16)
+constexpr int NW = 4;             // warps per CTA
+constexpr int NT = 32 * NW;
+constexpr int CTAS_PER_SM = 2;
+constexpr int NX = 4;             // 8-column groups of the intermediate per chunk
+constexpr int WARP_ELEMS = 2048;  // output elements of a warp: 16 x 128 or 8 x 256
+static_assert(F64_TM == 32 && F64_TN == 256, "warp layouts of a tile");
 
-// Row strides = 4 (mod 16) doubles: a fragment load (8 rows x 4 k, or 4 k x
-// 8 columns) then touches every bank pair exactly twice.
 struct Smem {
-  double A[TM][KC + 4];       // left operator rows x k
-  double B[KC][NCH + 4];      // psi k x chunk columns
-  double X[TM][NCH + 4];      // intermediate rows x chunk columns
-  double C[KC2][TN + 4];      // right operator, k-major: C[k][j] = X_R(c0 + j, k)
+  double part[NW][WARP_ELEMS];  // the warps' sums of an item
   int item;
 };
-
-__device__ __forceinline__ double ld_op(const double* __restrict__ base, long long aoff, bool trans,
-                                        int rows, int cols, int i, int k) {
-  // element (i, k) of the used matrix (rows x cols); stored transposed when trans
-  return trans ? base[aoff + (long long)k * rows + i] : base[aoff + (long long)i * cols + k];
-}
 
 // D = A(8x4) B(4x8) + D; lane (g = lane/4, c = lane%4) holds A[g][c],
 // B[c][g] and D[g][2c], D[g][2c+1].
@@ -67,164 +62,289 @@ __device__ __forceinline__ void dmma(double (&d)[2], double a, double b) {
                : "d"(a), "d"(b));
 }
 
-__device__ __forceinline__ int up8(int x) { return (x + 7) & ~7; }
-__device__ __forceinline__ int up4(int x) { return (x + 3) & ~3; }
+// s += sum of the tasks t0, t0 + step, ... < t1 on rows r0 .. r0 + 8 nrs - 1
+// (nrs <= RG groups of 8) and columns c0 .. c0 + 8 ncs - 1 (ncs <= CG groups)
+// of output block ob. Rows and columns past the block are computed from its
+// last row or column (never stored, so only finite or not matters to
+// themselves); contraction indices past the end enter as zeros on both sides.
+//
+// The second product contracts the columns of X. Its A fragment wants X[g][k]
+// for four k in lane order c = 0..3, and the lane already holds X[g][2c] and
+// X[g][2c + 1] of every 8-column group: the order of a contraction is free, so
+// one instruction takes the columns 2c and the next the columns 2c + 1, with
+// the right operator's columns loaded in the same order, and X never moves.
+// Only a last group of 2-4 valid columns is brought into natural order by
+// shuffles, where one instruction then replaces two.
+template <int RG, int CG>
+__device__ __forceinline__ void run_tasks(const SigmaDev& a, const PsiBlock& ob, int r0, int nrs, int c0, int ncs,
+                                          int t0, int t1, int step, int lane, double (&s)[RG][CG][2]) {
+  const int g = lane >> 2, c = lane & 3;
+  const int mo = ob.mL, no = ob.mR;
+  int row[RG];
+#pragma unroll
+  for (int r = 0; r < RG; ++r) row[r] = min(r0 + 8 * r + g, mo - 1);
+  const int col_first = min(c0 + g, no - 1), col_last = min(c0 + 8 * (ncs - 1) + g, no - 1);
+  Task nx{};
+  if (t0 < t1) nx = a.tasks[t0];
+  for (int t = t0; t < t1; t += step) {
+    const Task tk = nx;
+    if (t + step < t1) nx = a.tasks[t + step];  // in flight during this task
+    const PsiBlock ib = a.blocks[tk.in_blk];
+    const int m = ib.mL, n = ib.mR;
+    const double* __restrict__ psib = a.psi + ib.off;
+    const bool tA = tk.flags & 1, tB = tk.flags & 2;
+    // element (i, k) of the left block used: la[i * ars + k * aks]; of the right one likewise
+    const long long ars = tA ? 1 : m, aks = tA ? mo : 1, rrs = tB ? 1 : n, rks = tB ? no : 1;
+    const double* __restrict__ la = a.store + (tk.aoff < 0 ? 0 : tk.aoff);
+    const double* __restrict__ lr = a.store + (tk.boff < 0 ? 0 : tk.boff);
+    for (int nc0 = 0; nc0 < n; nc0 += 8 * NX) {
+      const int nleft = n - nc0, nxs = min(NX, (nleft + 7) >> 3);
+      // ---- X = scale * L[rows, :] psi_b[:, nc0 .. nc0 + 8 nxs)
+      double x[RG][NX][2];
+      if (tk.aoff < 0) {
+#pragma unroll
+        for (int r = 0; r < RG; ++r)
+#pragma unroll
+          for (int q = 0; q < NX; ++q)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              x[r][q][h] = psib[(long long)row[r] * n + min(nc0 + 8 * q + 2 * c + h, n - 1)];
+      } else {
+#pragma unroll
+        for (int r = 0; r < RG; ++r)
+#pragma unroll
+          for (int q = 0; q < NX; ++q) x[r][q][0] = x[r][q][1] = 0.0;
+        const double* pa[RG];
+#pragma unroll
+        for (int r = 0; r < RG; ++r) pa[r] = la + row[r] * ars + c * aks;
+        const double* pb = psib + (long long)c * n;
+        int ob_[NX];
+#pragma unroll
+        for (int q = 0; q < NX; ++q) ob_[q] = min(nc0 + 8 * q + g, n - 1);
+        auto kstep = [&](bool valid) {
+          double av[RG], bv[NX];
+#pragma unroll
+          for (int r = 0; r < RG; ++r) av[r] = (valid && r < nrs) ? __ldg(pa[r]) : 0.0;
+#pragma unroll
+          for (int q = 0; q < NX; ++q) bv[q] = (valid && q < nxs) ? __ldg(pb + ob_[q]) : 0.0;
+#pragma unroll
+          for (int q = 0; q < NX; ++q)
+            if (q < nxs)
+#pragma unroll
+              for (int r = 0; r < RG; ++r)
+                if (r < nrs) dmma(x[r][q], av[r], bv[q]);
+        };
+        for (int k = 0; k + 4 <= m; k += 4) {
+          kstep(true);
+#pragma unroll
+          for (int r = 0; r < RG; ++r) pa[r] += 4 * aks;
+          pb += 4ll * n;
+        }
+        if (m & 3) kstep(c < (m & 3));
+      }
+      if (tk.scale != 1.0) {
+#pragma unroll
+        for (int r = 0; r < RG; ++r)
+#pragma unroll
+          for (int q = 0; q < NX; ++q)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) x[r][q][h] *= tk.scale;
+      }
+      if (nleft < 8 * NX) {  // columns past the block
+#pragma unroll
+        for (int r = 0; r < RG; ++r)
+#pragma unroll
+          for (int q = 0; q < NX; ++q)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              if (8 * q + 2 * c + h >= nleft) x[r][q][h] = 0.0;
+      }
+      // ---- S += X R[columns, nc0 ..]^T
+      if (tk.boff < 0) {  // identity: output column j is intermediate column j
+#pragma unroll
+        for (int j = 0; j < CG; ++j)
+#pragma unroll
+          for (int q = 0; q < NX; ++q)
+            if (c0 + 8 * j == nc0 + 8 * q) {
+#pragma unroll
+              for (int r = 0; r < RG; ++r)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) s[r][j][h] += x[r][q][h];
+            }
+        continue;
+      }
+#pragma unroll
+      for (int q = 0; q < NX; ++q) {
+        if (q >= nxs) break;
+        const int left = nleft - 8 * q;        // valid columns of this group
+        const bool natural = left >= 2 && left <= 4;
+        double a0[RG], a1[RG];
+        if (natural) {
+#pragma unroll
+          for (int r = 0; r < RG; ++r) {
+            const int src = (lane & ~3) | (c >> 1);
+            const double u = __shfl_sync(0xffffffffu, x[r][q][0], src), v = __shfl_sync(0xffffffffu, x[r][q][1], src);
+            a0[r] = (c & 1) ? v : u;
+            a1[r] = 0.0;
+          }
+        } else {
+#pragma unroll
+          for (int r = 0; r < RG; ++r) {
+            a0[r] = x[r][q][0];
+            a1[r] = x[r][q][1];
+          }
+        }
+        const int k0 = nc0 + 8 * q + (natural ? c : 2 * c);  // this lane's first contraction column
+        const bool two = !natural && left > 1;               // the columns 2c + 1 hold something
+        const bool v0 = k0 < n, v1 = two && k0 + 1 < n;
+        const double* p0 = lr + col_first * rrs + k0 * rks;
+        const double* pl = lr + col_last * rrs + k0 * rks;
+#pragma unroll
+        for (int j = 0; j < CG; ++j) {
+          if (j >= ncs) break;
+          const double* p = j == ncs - 1 ? pl : p0 + 8ll * j * rrs;
+          const double b0 = v0 ? __ldg(p) : 0.0, b1 = v1 ? __ldg(p + rks) : 0.0;
+#pragma unroll
+          for (int r = 0; r < RG; ++r)
+            if (r < nrs) dmma(s[r][j], a0[r], b0);
+          if (two) {
+#pragma unroll
+            for (int r = 0; r < RG; ++r)
+              if (r < nrs) dmma(s[r][j], a1[r], b1);
+          }
+        }
+      }
+    }
+  }
+}
 
-__global__ void __launch_bounds__(NT, 2)
+// One item on one CTA: RG x CG register tiles, rows [8 RG i, ..) of the tile
+// on row slice i, and the item's tasks shared by NW / n_rows warps per row
+// slice. `flip` swaps the row slices between the two resident CTAs, so that a
+// short last slice does not leave the same SM sub-partitions idle in both.
+template <int RG, int CG>
+__device__ __forceinline__ void run_item(const SigmaDev& a, const Item& it, const PsiBlock& ob, bool flip, Smem& sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int g = lane >> 2, c = lane & 3;
+  int n_rows = (it.nrows + 8 * RG - 1) / (8 * RG);  // 1, 2 or 4 (3 leaves a warp idle)
+  if (n_rows == 3) n_rows = 4;
+  const int n_slices = NW / n_rows;
+  const int w = flip ? NW - 1 - warp : warp;
+  const int rs = w / n_slices, sl = w - rs * n_slices;
+  const int r0 = 8 * RG * rs, nr = min(8 * RG, it.nrows - r0);
+  double s[RG][CG][2];
+#pragma unroll
+  for (int r = 0; r < RG; ++r)
+#pragma unroll
+    for (int j = 0; j < CG; ++j) s[r][j][0] = s[r][j][1] = 0.0;
+  if (nr > 0)
+    run_tasks<RG, CG>(a, ob, it.r0 + r0, (nr + 7) >> 3, it.c0, (it.ncols + 7) >> 3, it.t_begin + sl, it.t_end,
+                      n_slices, lane, s);
+  double* out = a.scratch + it.slot;
+  if (n_slices == 1) {  // the warp holds its rows' sums
+#pragma unroll
+    for (int r = 0; r < RG; ++r)
+#pragma unroll
+      for (int j = 0; j < CG; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int row = 8 * r + g, col = 8 * j + 2 * c + h;
+          if (row < nr && col < it.ncols) out[(long long)(r0 + row) * it.ncols + col] = s[r][j][h];
+        }
+    return;
+  }
+  // add the slices of every row slice in order
+  double* mine = sm.part[rs * n_slices + sl];
+#pragma unroll
+  for (int r = 0; r < RG; ++r)
+#pragma unroll
+    for (int j = 0; j < CG; ++j)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int row = 8 * r + g, col = 8 * j + 2 * c + h;
+        if (row < nr && col < it.ncols) mine[row * it.ncols + col] = s[r][j][h];
+      }
+  __syncthreads();
+  for (int e = threadIdx.x; e < it.nrows * it.ncols; e += NT) {
+    const int i = e / (8 * RG * it.ncols), le = e - i * (8 * RG * it.ncols);
+    double v = sm.part[i * n_slices][le];
+    for (int k = 1; k < n_slices; ++k) v += sm.part[i * n_slices + k][le];
+    out[e] = v;
+  }
+}
+
+__global__ void __launch_bounds__(NT, CTAS_PER_SM)
 sigma_f64_kernel(SigmaDev a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
-  const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  const int g = lane >> 2, c = lane & 3;
-
+  const bool flip = blockIdx.x >= gridDim.x / 2;
   for (;;) {
-    if (tid == 0) {
+    if (threadIdx.x == 0) {
       unsigned k = atomicAdd(a.counter, 1u);
       sm.item = (k < (unsigned)a.n_items) ? a.schedule[k] : -1;
     }
     __syncthreads();
     const int it_idx = sm.item;
-    __syncthreads();
+    __syncthreads();  // the slot and sm.part are rewritten from here on
     if (it_idx < 0) return;
     const Item it = a.items[it_idx];
     const PsiBlock ob = a.blocks[it.out];
-    const int nr = it.nrows, ncol = it.ncols;
-    const int nr8 = up8(nr), nrg = nr8 >> 3, ncg = up8(ncol) >> 3;
-    const int n_s = nrg * ncg;  // output sub-tiles of this item
+    // tiles up to 128 columns: 16 x 128 per warp; wider: 8 x 256, so that the
+    // intermediate is still computed once per row
+    if (it.ncols <= 128)
+      run_item<2, 16>(a, it, ob, flip, sm);
+    else
+      run_item<1, 32>(a, it, ob, flip, sm);
+  }
+}
 
-    double s[SS][2];
+// Work lists whose output tiles are one item of one task each (the
+// transformation of Eq. op-trans: 1e3-1e6 tiles): the warps of a CTA share the
+// 16 x 128 pieces of NW items at a time (each piece one warp's register tile)
+// and write them straight into sigma: no partial tiles, no reduction pass, one
+// counter access per NW items. (An item per warp, whatever its size, left a
+// tail of single warps on the widest sectors.) The transformations of two
+// sweeps at K=24, M=300 take 87 ms, mostly host lists (90 ms with partial tiles
+// as large as the store written and reduced).
+__global__ void __launch_bounds__(NT, CTAS_PER_SM)
+sigma_f64_direct_kernel(SigmaDev a) {
+  __shared__ int next;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+  for (;;) {
+    if (threadIdx.x == 0) next = (int)min(atomicAdd(a.counter, (unsigned)NW), 0x7ffffff0u);
+    __syncthreads();
+    const int q0 = next;
+    __syncthreads();
+    if (q0 >= a.n_items) return;
+    int p = warp;  // this warp's next piece, counted from the current item's first
+    for (int q = q0; q < min(q0 + NW, a.n_items); ++q) {
+      const Item it = a.items[a.schedule[q]];
+      const int n_cols = (it.ncols + 127) >> 7, n_pieces = ((it.nrows + 15) >> 4) * n_cols;
+      if (p < n_pieces) {
+        const PsiBlock ob = a.blocks[it.out];
+        double* out = a.sigma + ob.off + (long long)it.r0 * ob.mR + it.c0;
+        for (; p < n_pieces; p += NW) {
+          const int r0 = 16 * (p / n_cols), c0 = 128 * (p % n_cols);
+          const int nr = min(16, it.nrows - r0), nc = min(128, it.ncols - c0);
+          double s[2][16][2];
 #pragma unroll
-    for (int q = 0; q < SS; ++q) s[q][0] = s[q][1] = 0.0;
-
-    for (int t = it.t_begin; t < it.t_end; ++t) {
-      const Task tk = a.tasks[t];
-      const PsiBlock ib = a.blocks[tk.in_blk];
-      const int m = ib.mL, n = ib.mR;        // input block
-      const int mo = ob.mL, no = ob.mR;      // output block
-      const bool tA = tk.flags & 1, tB = tk.flags & 2;
-      const double* __restrict__ psib = a.psi + ib.off;
-
-      for (int nc0 = 0; nc0 < n; nc0 += NCH) {
-        const int nch = min(NCH, n - nc0), nch8 = up8(nch), nch4 = up4(nch);
-        const int xcg = nch8 >> 3, n_x = nrg * xcg;
-        // ---- step 1: X = scale * X_L[r0:r0+nr, :] psi_b[:, nc0:nc0+nch]
-        if (tk.aoff < 0) {
-          for (int e = tid; e < nr8 * nch8; e += NT) {
-            const int i = e / nch8, j = e % nch8;
-            double v = 0.0;
-            if (i < nr && j < nch) v = psib[(long long)(it.r0 + i) * n + nc0 + j];
-            sm.X[i][j] = tk.scale * v;
-          }
-        } else {
-          double x[XS][2];
+          for (int r = 0; r < 2; ++r)
 #pragma unroll
-          for (int p = 0; p < XS; ++p) x[p][0] = x[p][1] = 0.0;
-          for (int k0 = 0; k0 < m; k0 += KC) {
-            const int kc = min(KC, m - k0), kc4 = up4(kc);
-            if (!tA) {
-              for (int e = tid; e < nr8 * kc4; e += NT) {
-                const int i = e / kc4, kk = e % kc4;
-                sm.A[i][kk] = (i < nr && kk < kc) ? ld_op(a.store, tk.aoff, false, mo, m, it.r0 + i, k0 + kk) : 0.0;
-              }
-            } else {
-              for (int e = tid; e < nr8 * kc4; e += NT) {
-                const int kk = e / nr8, i = e % nr8;
-                sm.A[i][kk] = (i < nr && kk < kc) ? ld_op(a.store, tk.aoff, true, mo, m, it.r0 + i, k0 + kk) : 0.0;
-              }
-            }
-            for (int e = tid; e < kc4 * nch8; e += NT) {
-              const int kk = e / nch8, j = e % nch8;
-              sm.B[kk][j] = (kk < kc && j < nch) ? psib[(long long)(k0 + kk) * n + nc0 + j] : 0.0;
-            }
-            __syncthreads();
-            for (int kk = 0; kk < kc4; kk += 4) {
+            for (int j = 0; j < 16; ++j) s[r][j][0] = s[r][j][1] = 0.0;
+          run_tasks<2, 16>(a, ob, it.r0 + r0, (nr + 7) >> 3, it.c0 + c0, (nc + 7) >> 3, it.t_begin, it.t_end, 1, lane,
+                           s);
 #pragma unroll
-              for (int p = 0; p < XS; ++p) {
-                const int sx = warp + NW * p;
-                if (sx < n_x) {
-                  const int rg = sx / xcg, cg = sx - rg * xcg;
-                  dmma(x[p], sm.A[rg * 8 + g][kk + c], sm.B[kk + c][cg * 8 + g]);
-                }
-              }
-            }
-            __syncthreads();
-          }
+          for (int r = 0; r < 2; ++r)
 #pragma unroll
-          for (int p = 0; p < XS; ++p) {
-            const int sx = warp + NW * p;
-            if (sx < n_x) {
-              const int rg = sx / xcg, cg = sx - rg * xcg;
-              sm.X[rg * 8 + g][cg * 8 + 2 * c] = tk.scale * x[p][0];
-              sm.X[rg * 8 + g][cg * 8 + 2 * c + 1] = tk.scale * x[p][1];
-            }
-          }
-        }
-        __syncthreads();
-
-        // ---- step 2: S += X X_R[c0:c0+ncol, nc0:nc0+nch]^T
-        if (tk.boff < 0) {
-          // identity on the right: output column j reads intermediate column j
-#pragma unroll
-          for (int q = 0; q < SS; ++q) {
-            const int ss = warp + NW * q;
-            if (ss < n_s) {
-              const int rg = ss / ncg, cg = ss - rg * ncg;
+            for (int j = 0; j < 16; ++j)
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
-                const int col = it.c0 + cg * 8 + 2 * c + h - nc0;
-                if (col >= 0 && col < nch) s[q][h] += sm.X[rg * 8 + g][col];
+                const int row = 8 * r + g, col = 8 * j + 2 * c + h;
+                if (row < nr && col < nc) out[(long long)(r0 + row) * ob.mR + c0 + col] = s[r][j][h];
               }
-            }
-          }
-        } else {
-          const int nc8 = ncg * 8;
-          for (int k0 = 0; k0 < nch4; k0 += KC2) {
-            const int kc4 = min(KC2, nch4 - k0);
-            if (!tB) {
-              for (int e = tid; e < nc8 * kc4; e += NT) {
-                const int j = e / kc4, kk = e % kc4;
-                const int k = nc0 + k0 + kk;
-                sm.C[kk][j] = (j < ncol && k0 + kk < nch) ? ld_op(a.store, tk.boff, false, no, n, it.c0 + j, k) : 0.0;
-              }
-            } else {
-              for (int e = tid; e < nc8 * kc4; e += NT) {
-                const int kk = e / nc8, j = e % nc8;
-                const int k = nc0 + k0 + kk;
-                sm.C[kk][j] = (j < ncol && k0 + kk < nch) ? ld_op(a.store, tk.boff, true, no, n, it.c0 + j, k) : 0.0;
-              }
-            }
-            __syncthreads();
-            for (int kk = 0; kk < kc4; kk += 4) {
-#pragma unroll
-              for (int q = 0; q < SS; ++q) {
-                const int ss = warp + NW * q;
-                if (ss < n_s) {
-                  const int rg = ss / ncg, cg = ss - rg * ncg;
-                  dmma(s[q], sm.X[rg * 8 + g][k0 + kk + c], sm.C[kk + c][cg * 8 + g]);
-                }
-              }
-            }
-            __syncthreads();
-          }
-        }
-        __syncthreads();
-      }
-    }
-    // partial tile -> private scratch slot
-    double* out = a.scratch + it.slot;
-#pragma unroll
-    for (int q = 0; q < SS; ++q) {
-      const int ss = warp + NW * q;
-      if (ss < n_s) {
-        const int rg = ss / ncg, cg = ss - rg * ncg;
-        const int r = rg * 8 + g;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int col = cg * 8 + 2 * c + h;
-          if (r < nr && col < ncol) out[(long long)r * ncol + col] = s[q][h];
         }
       }
+      p -= n_pieces;
     }
   }
 }
@@ -278,10 +398,17 @@ void set_max_dynamic_smem(const void* fn, int bytes) {
   done.insert({fn, dev, bytes});
 }
 
+void launch_sigma_f64_direct(const SigmaDev& a, int n_sm, cudaStream_t st) {
+  if (a.n_items < 1) return;
+  int grid = CTAS_PER_SM * n_sm;
+  if (grid > (a.n_items + NW - 1) / NW) grid = (a.n_items + NW - 1) / NW;
+  sigma_f64_direct_kernel<<<grid, NT, 0, st>>>(a);
+}
+
 void launch_sigma_f64(const SigmaDev& a, int n_sm, cudaStream_t st) {
   const int smem = (int)sizeof(Smem);
   set_max_dynamic_smem((const void*)sigma_f64_kernel, smem);
-  int grid = 2 * n_sm;  // two resident CTAs per SM overlap one's loads with the other's products
+  int grid = CTAS_PER_SM * n_sm;
   if (grid > a.n_items) grid = a.n_items;
   if (grid < 1) grid = 1;
   sigma_f64_kernel<<<grid, NT, smem, st>>>(a);

@@ -24,7 +24,7 @@
 
 namespace dmrg {
 
-constexpr long long kScratchDoubles = 4ll << 20;  // 32 MiB of FP64 partial tiles
+constexpr long long kScratchDoubles = NOALLOC_DOUBLES;  // FP64 partial tiles
 
 static __device__ __align__(256) double g_sigma_scratch[kScratchDoubles];
 static __device__ __align__(256) unsigned int g_sigma_counter[64];

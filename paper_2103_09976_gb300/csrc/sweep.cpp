@@ -300,17 +300,15 @@ void transform(Context& c, const OpSet& EO, const double* enl_store, const Basis
   }
   wl.tasks = tasks;
   build_items(blocks, wl, TileShape{F64_TM, F64_TN, 2e6}, c.n_sm * 8, nout);
-  DevBuf d_tasks, d_items, d_groups, d_sched, d_blocks, d_scratch, d_counter;
+  DevBuf d_tasks, d_items, d_sched, d_blocks, d_counter;
   cudaStream_t st = c.stream;
   d_tasks.upload(wl.tasks, st);
   d_items.upload(wl.items, st);
-  d_groups.upload(wl.groups, st);
   d_sched.upload(wl.schedule, st);
   d_blocks.upload(blocks, st);
-  d_scratch.alloc(std::max<long long>(1, wl.scratch_elems) * sizeof(double));
   d_counter.alloc(16);
   DMRG_CUDA(cudaMemsetAsync(d_counter.p, 0, sizeof(unsigned int), st));
-  SigmaDev a;
+  SigmaDev a{};
   a.store = u_store;
   a.psi = enl_store;
   a.sigma = out.store.as<double>();
@@ -318,16 +316,11 @@ void transform(Context& c, const OpSet& EO, const double* enl_store, const Basis
   a.items = d_items.as<Item>();
   a.schedule = d_sched.as<int>();
   a.n_items = (int)wl.items.size();
-  a.groups = d_groups.as<Group>();
-  a.n_groups = (int)wl.groups.size();
-  a.max_tile = wl.max_tile;
   a.blocks = d_blocks.as<PsiBlock>();
-  a.scratch = d_scratch.as<double>();
   a.counter = d_counter.as<unsigned int>();
   if (a.n_items > 0) {
     ProfScope ps(c.prof, 3, st);
-    launch_sigma_f64(a, c.n_sm, st);
-    launch_reduce(a, st);
+    launch_sigma_f64_direct(a, c.n_sm, st);  // one task, so one item, per output tile
   }
   DMRG_CUDA(cudaGetLastError());
   DMRG_CUDA(cudaStreamSynchronize(st));
