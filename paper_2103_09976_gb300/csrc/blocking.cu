@@ -358,81 +358,197 @@ __global__ void svd_norm_kernel(const SvdBlock* __restrict__ sb, int nb, const d
   }
 }
 
-// A pair is rotated while its cosine |a_p . a_q| / (|a_p| |a_q|) exceeds
+// A pair is rotated while its cosine |a_p . a_q| / (|a_p| |a_q|) is at least
 // tol = max(1e-15, eps sqrt(m)) (the rounding floor of an m-term dot
 // product), and only if both vectors exceed 1e-15 |A|_F: vectors below that
 // are numerical zeros (a block with more rows than columns has them), whose
 // mutual cosines are rounding noise and would never settle. Sweeps stop when
 // no pair of any block is above its tolerance (at most 30).
-__global__ void svd_jacobi_kernel(const SvdBlock* __restrict__ sb, int nb, int total_pairs, int max_rounds,
-                                  double* __restrict__ work, const double* __restrict__ fro,
-                                  unsigned long long* __restrict__ off_max) {
+//
+// Bound by the latency of a round (one pair per warp, then a grid barrier),
+// and on this GPU mostly by the FP64 pipe within it: a warp instruction takes
+// about 67 cycles of its SM sub-partition, so the two divisions and three square
+// roots of the rotation, a few dozen instructions each, cost more than the
+// vectors. Hence: the rotation's tangent is computed in FP32 (an angle off
+// by 1e-7 leaves 1e-7 of the product, which later sweeps remove) and only its
+// cosine, which keeps the rotation orthogonal, in FP64 by Newton steps; the
+// squared column norms are carried along (al - t ga, be + t ga; exact to
+// second order in the angle) and recomputed at the start of every sweep; both
+// vectors and their columns of V are loaded once, before the angle is known;
+// every warp keeps its pair's block description for all rounds; and one CTA per
+// SM takes part in the barrier, consecutive pairs on different SMs. Decimations
+// of two sweeps, against three full dot products per pair, a plain FP64
+// rotation and 608 CTAs: 474 -> 112 ms at K=16, M=150 (30 steps), 1771 -> 449 ms
+// at K=24, M=300 (46 steps).
+constexpr int SVD_THREADS = 256;
+constexpr int SVD_REG = 8;         // vectors up to 32 * SVD_REG long stay in registers
+
+// Tangent of the rotation that makes two columns of squared norms al, be and
+// product ga orthogonal (|t| <= 1), to FP32 accuracy.
+__device__ __forceinline__ double jacobi_tangent(double al, double be, double ga) {
+  const double hi = fmax(al, be);
+  const int e = (__double2hiint(hi) >> 20) & 0x7ff;
+  if (e < 64 || e > 1980) {  // 2^-e out of range: plain FP64
+    const double zeta = (be - al) / (2.0 * ga);
+    return (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+  }
+  const double sc = __hiloint2double((2046 - e) << 20, 0);  // brings hi into [1, 2)
+  const float d = (float)((be - al) * sc), g = (float)(ga * sc);
+  const float z = d / (2.0f * g);
+  const float az = fabsf(z);
+  const float t = az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az));
+  return z >= 0.0f ? (double)t : -(double)t;
+}
+
+// 1 / sqrt(u), u in [1, 2], by Newton's iteration from an FP32 start
+__device__ __forceinline__ double newton_rsqrt(double u) {
+  double r = (double)rsqrtf((float)u);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) r = fma(0.5 * r, fma(-u * r, r, 1.0), r);
+  return r;
+}
+
+// Round `r` of block s, pair i: true when the pair was above its tolerance.
+// fresh: the norms are recomputed (first round of a sweep).
+__device__ bool svd_pair(const SvdBlock& s, int i, int r, bool fresh, double* __restrict__ work,
+                         double* __restrict__ nrm, double floor2, int lane) {
+  const int dp = s.d + (s.d & 1);
+  auto player = [&](int x) { return x == 0 ? 0 : 1 + (x - 1 + r) % (dp - 1); };
+  int p = player(i), q = player(dp - 1 - i);
+  if (p > q) { const int t = p; p = q; q = t; }
+  double* ap = work + s.a_off + (long long)p * s.m;
+  if (q >= s.d) {  // p sits this round out
+    if (fresh) {
+      double al = 0.0;
+      for (int e = lane; e < s.m; e += 32) al = fma(ap[e], ap[e], al);
+      al = warp_sum(al);
+      if (lane == 0) nrm[s.q_off + p] = al;
+    }
+    return false;
+  }
+  double* aq = work + s.a_off + (long long)q * s.m;
+  double* vp = work + s.v_off + (long long)p * s.d;
+  double* vq = work + s.v_off + (long long)q * s.d;
+  const bool in_regs = s.m <= 32 * SVD_REG && s.d <= 32 * SVD_REG;
+  double x[SVD_REG], y[SVD_REG], vx[SVD_REG], vy[SVD_REG];
+  double al = 0.0, be = 0.0, ga = 0.0;
+  if (!fresh) {
+    al = nrm[s.q_off + p];
+    be = nrm[s.q_off + q];
+  }
+  if (in_regs) {
+#pragma unroll
+    for (int k = 0; k < SVD_REG; ++k) {
+      const int e = lane + 32 * k;
+      if (32 * k < s.m) {
+        x[k] = e < s.m ? ap[e] : 0.0;
+        y[k] = e < s.m ? aq[e] : 0.0;
+      }
+      if (32 * k < s.d) {
+        vx[k] = e < s.d ? vp[e] : 0.0;
+        vy[k] = e < s.d ? vq[e] : 0.0;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < SVD_REG; ++k)
+      if (32 * k < s.m) {
+        ga = fma(x[k], y[k], ga);
+        if (fresh) {
+          al = fma(x[k], x[k], al);
+          be = fma(y[k], y[k], be);
+        }
+      }
+  } else {
+    for (int e = lane; e < s.m; e += 32) {
+      const double u = ap[e], v = aq[e];
+      ga = fma(u, v, ga);
+      if (fresh) {
+        al = fma(u, u, al);
+        be = fma(v, v, be);
+      }
+    }
+  }
+  ga = warp_sum(ga);
+  if (fresh) {
+    al = warp_sum(al);
+    be = warp_sum(be);
+  }
+  const double tol2 = fmax(1e-30, 4.930380657631324e-32 * (double)s.m);
+  const bool rotate = ga != 0.0 && al > floor2 && be > floor2 && ga * ga >= tol2 * (al * be);
+  double t = 0.0;
+  if (rotate) {
+    t = jacobi_tangent(al, be, ga);
+    const double c = newton_rsqrt(fma(t, t, 1.0)), sn = c * t;
+    if (in_regs) {
+#pragma unroll
+      for (int k = 0; k < SVD_REG; ++k) {
+        const int e = lane + 32 * k;
+        if (32 * k < s.m && e < s.m) {
+          ap[e] = fma(c, x[k], -sn * y[k]);
+          aq[e] = fma(sn, x[k], c * y[k]);
+        }
+        if (32 * k < s.d && e < s.d) {
+          vp[e] = fma(c, vx[k], -sn * vy[k]);
+          vq[e] = fma(sn, vx[k], c * vy[k]);
+        }
+      }
+    } else {
+      for (int e = lane; e < s.m; e += 32) {
+        const double u = ap[e], v = aq[e];
+        ap[e] = fma(c, u, -sn * v);
+        aq[e] = fma(sn, u, c * v);
+      }
+      for (int e = lane; e < s.d; e += 32) {
+        const double u = vp[e], v = vq[e];
+        vp[e] = fma(c, u, -sn * v);
+        vq[e] = fma(sn, u, c * v);
+      }
+    }
+  }
+  if (lane == 0 && (rotate || fresh)) {
+    nrm[s.q_off + p] = fma(-t, ga, al);
+    nrm[s.q_off + q] = fma(t, ga, be);
+  }
+  return rotate;
+}
+
+__global__ void __launch_bounds__(SVD_THREADS, 1)
+svd_jacobi_kernel(const SvdBlock* __restrict__ sb, int nb, int total_pairs, int max_rounds, double* __restrict__ work,
+                  double* __restrict__ nrm, const double* __restrict__ fro, unsigned int* __restrict__ above) {
   namespace cgp = cooperative_groups;
   cgp::grid_group grid = cgp::this_grid();
   const int lane = threadIdx.x & 31;
-  const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+  const int warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;  // consecutive pairs on different SMs
+  const int nwarps = (blockDim.x >> 5) * gridDim.x;
+  auto block_of = [&](int pid) {  // last b with pair0 <= pid
+    int lo = 0, hi = nb - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (sb[mid].pair0 <= pid) lo = mid;
+      else hi = mid - 1;
+    }
+    return sb[lo];
+  };
+  const SvdBlock first = block_of(min(warp, total_pairs - 1));
+  const double floor_first = 1e-30 * fro[first.w_off];
   for (int sweep = 0; sweep < 30; ++sweep) {
-    const int slot = sweep & 1;
-    double local = 0.0;
+    bool any = false;
     for (int round = 0; round < max_rounds; ++round) {
-      for (long long pid = warp; pid < total_pairs; pid += nwarps) {
-        int lo = 0, hi = nb - 1;  // block of pair pid: last b with pair0 <= pid
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (sb[mid].pair0 <= pid) lo = mid;
-          else hi = mid - 1;
-        }
-        const SvdBlock s = sb[lo];
-        const int i = (int)(pid - s.pair0);
+      for (int pid = warp; pid < total_pairs; pid += nwarps) {
+        const SvdBlock s = pid == warp ? first : block_of(pid);
+        const int i = pid - s.pair0;
         if (i >= s.npairs || s.rounds <= 0) continue;
-        const int dp = s.d + (s.d & 1), r = round % s.rounds;
-        auto player = [&](int x) { return x == 0 ? 0 : 1 + (x - 1 + r) % (dp - 1); };
-        int p = player(i), q = player(dp - 1 - i);
-        if (p > q) { const int t = p; p = q; q = t; }
-        if (q >= s.d) continue;
-        double* ap = work + s.a_off + (long long)p * s.m;
-        double* aq = work + s.a_off + (long long)q * s.m;
-        double al = 0.0, be = 0.0, ga = 0.0;
-        for (int e = lane; e < s.m; e += 32) {
-          const double x = ap[e], y = aq[e];
-          al = fma(x, x, al);
-          be = fma(y, y, be);
-          ga = fma(x, y, ga);
-        }
-        al = warp_sum(al);
-        be = warp_sum(be);
-        ga = warp_sum(ga);
-        const double floor2 = 1e-30 * fro[s.w_off];
-        if (ga == 0.0 || al <= floor2 || be <= floor2) continue;
-        const double tol = fmax(1e-15, 2.220446049250313e-16 * sqrt((double)s.m));
-        const double cosv = fabs(ga) / sqrt(al * be);
-        local = fmax(local, cosv / tol);
-        if (cosv < tol) continue;
-        const double zeta = (be - al) / (2.0 * ga);
-        const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double c = 1.0 / sqrt(1.0 + t * t), sn = c * t;
-        for (int e = lane; e < s.m; e += 32) {
-          const double x = ap[e], y = aq[e];
-          ap[e] = c * x - sn * y;
-          aq[e] = sn * x + c * y;
-        }
-        double* vp = work + s.v_off + (long long)p * s.d;
-        double* vq = work + s.v_off + (long long)q * s.d;
-        for (int e = lane; e < s.d; e += 32) {
-          const double x = vp[e], y = vq[e];
-          vp[e] = c * x - sn * y;
-          vq[e] = sn * x + c * y;
-        }
+        const double floor2 = pid == warp ? floor_first : 1e-30 * fro[s.w_off];
+        any |= svd_pair(s, i, round % s.rounds, round == 0, work, nrm, floor2, lane);
       }
       grid.sync();
     }
-    if (lane == 0 && local > 0.0) atomicMax(off_max + slot, (unsigned long long)__double_as_longlong(local));
+    // above[sweep % 3]: raised in this sweep, read after the barrier, cleared for reuse two sweeps later
+    if (lane == 0 && any) atomicOr(above + sweep % 3, 1u);
     grid.sync();
-    const double worst = __longlong_as_double((long long)off_max[slot]);
-    if (blockIdx.x == 0 && threadIdx.x == 0) off_max[slot ^ 1] = 0ull;
-    grid.sync();
-    if (worst < 1.0) break;
+    const bool more = *(volatile unsigned int*)(above + sweep % 3) != 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) above[(sweep + 2) % 3] = 0u;
+    if (!more) break;
   }
 }
 
@@ -508,18 +624,14 @@ void launch_svd_blocks(const double* psi, const SvdBlock* sb, int nb, int total_
     svd_setup_kernel<<<grid, 256, 0, st>>>(psi, sb, nb, work, left ? 1 : 0);
   }
   if (total_pairs > 0 && max_rounds > 0) {
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, svd_jacobi_kernel, 256, 0);
-    if (per_sm < 1) per_sm = 1;
-    if (per_sm > 4) per_sm = 4;
-    int grid = n_sm * per_sm;
-    unsigned long long* off_max = reinterpret_cast<unsigned long long*>(work);  // first 2 words of work
-    cudaMemsetAsync(off_max, 0, 2 * sizeof(unsigned long long), st);
+    unsigned int* above = reinterpret_cast<unsigned int*>(work);  // first words of work
+    cudaMemsetAsync(above, 0, 4 * sizeof(unsigned int), st);
     svd_norm_kernel<<<nb < 65535 ? nb : 65535, 256, 0, st>>>(sb, nb, work, w);
     const double* fro = w;
+    double* nrm = Q;  // Q is written by the finish kernel: until then the squared column norms, d per block
     void* args[] = {(void*)&sb,   (void*)&nb,  (void*)&total_pairs, (void*)&max_rounds,
-                    (void*)&work, (void*)&fro, (void*)&off_max};
-    const cudaError_t e = cudaLaunchCooperativeKernel((void*)svd_jacobi_kernel, dim3(grid), dim3(256), args, 0, st);
+                    (void*)&work, (void*)&nrm, (void*)&fro,         (void*)&above};
+    const cudaError_t e = cudaLaunchCooperativeKernel((void*)svd_jacobi_kernel, dim3(n_sm), dim3(SVD_THREADS), args, 0, st);
     if (e != cudaSuccess) return;  // the caller's cudaGetLastError reports it
   }
   svd_finish_kernel<<<nb < 65535 ? nb : 65535, 256, (size_t)max_d_hint * sizeof(double), st>>>(sb, nb, work, Q, w);

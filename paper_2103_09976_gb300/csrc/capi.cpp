@@ -88,10 +88,10 @@ Problem& need_problem(Context& c, int site) {
 namespace dmrg {
 
 // Items of an FP64 sigma: want_items of them, but none below a minimum cost.
-// The minimum of ITEM_MIN (about ten tasks) lets small problems use every SM
-// (K=8, M=64: 34 items of 2e6 took 34 us alone on the same kernel's rate); where that many partial tiles
-// would not fit the fixed scratch of dmrg_sigma_noalloc and larger items do,
-// the larger minimum is kept, so that every problem that call can take it takes.
+// ITEM_MIN is about ten tasks of small blocks (two or three per warp), so that
+// small problems use every SM. Where that many partial tiles would not fit the
+// fixed scratch of dmrg_sigma_noalloc, the larger minimum is kept, so that
+// every problem that call could take with it is still taken.
 static void build_sigma_items(const std::vector<PsiBlock>& blocks, WorkList& wl, int want_items, double per_task) {
   constexpr double ITEM_MIN = 2e5, ITEM_MIN_LARGE = 2e6;
   build_items(blocks, wl, TileShape{F64_TM, F64_TN, ITEM_MIN, per_task}, want_items);
