@@ -151,8 +151,10 @@ struct Problem {
   // Davidson workspace (built on first use)
   bool dav_ready = false;
   int dav_space = 0;
-  DevBuf dav_V, dav_AV, dav_diag, dav_x, dav_ax, dav_r, dav_t, dav_partial, dav_H, dav_w, dav_Y, dav_s;
+  DevBuf dav_V, dav_AV, dav_diag, dav_x, dav_ax, dav_r, dav_t, dav_x2, dav_partial, dav_cnt, dav_H, dav_w, dav_Y, dav_Yf,
+      dav_s;
   DevBuf d_dstart, d_dtask;
+  DavScratch dav_scratch() const { return {dav_partial.as<double>(), dav_cnt.as<unsigned int>()}; }
   DevBuf split, psi_split;         // slice-interleaved bf16 tiles of the operators / of psi
   DevBuf split16, psi_split16;     // FP16X2: slice-interleaved fp16 tiles of the scaled operators / psi
   DevBuf d_exps, d_psi_exp;        // FP16X2: block exponents (per split job), exponent of max |psi|

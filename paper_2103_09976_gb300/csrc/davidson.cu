@@ -1,66 +1,251 @@
 // Davidson eigensolver on the device (FP64 control path).
 //
 // Appendix A (solving step, Eq. eff-eigsh) names the Davidson method. The
-// steps here: projected matrix V^T H V, its eigenpairs (one-warp cyclic
-// Jacobi), Ritz vector and residual, diagonal preconditioner clamped at
-// 1e-8, classical Gram-Schmidt twice, thick restart from the two lowest Ritz
-// vectors. Only two scalars per iteration (Ritz value, squared residual
-// norm) and the new direction's norm cross to the host. All reductions are
-// two-stage with a fixed order, so results are deterministic.
+// steps here: projected matrix V^T H V, its lowest eigenpair, Ritz vector and
+// residual, diagonal preconditioner clamped at 1e-8, classical Gram-Schmidt
+// twice, thick restart from the two lowest Ritz vectors. Three scalars per
+// iteration (Ritz value, squared residual norm, squared norm of the previous
+// new direction) cross to the host. All reductions have a fixed order, so
+// results are deterministic.
+//
+// The vectors of a solve are short (1e3 - 1e6) and the FP64 pipe takes about
+// 67 cycles per warp instruction and SM sub-partition, so an iteration is
+// bound by launches and by the instructions of its reductions, not by memory.
+// Hence a few kernels that each do all that one pass over the subspace can
+// (Ritz vector, residual, preconditioner and the first Gram-Schmidt products
+// in one), sums of up to 32 products over a warp that halve the number of
+// values with the number of lanes (31 additions instead of 160), and the last
+// block of a grid summing the blocks' partial results instead of a second
+// launch. An iteration took 28 launches and, without its sigma, 390 us at
+// K=16, M=150 (224 us of them the eigenproblem, 98 us dot products); now 8
+// launches and 140 us.
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace dmrg {
 
 namespace {
 
-constexpr int RED_BLOCKS = 256;   // partial sums per dot product
-constexpr int RED_THREADS = 256;
+constexpr int KMAX = DAV_KMAX;     // vectors per call (subspace size limit)
+constexpr int DT = 128;            // threads of a vector kernel
+constexpr int PSTRIDE = DAV_PSTRIDE;  // partial results per block: two sets of KMAX, or one and a scalar
+static_assert(PSTRIDE >= 2 * KMAX, "two sets of partial results");
 
-constexpr int KMAX = 32;           // vectors per dot-product call (subspace size limit)
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 
-// partial[i * RED_BLOCKS + b] = sum over block b's elements of V[i][e] * w[e],
-// for all i < k in one pass: each thread keeps k running sums, then the block
-// reduces them (warp shuffles, then across warps) in a fixed order.
-__global__ void dots_partial(const double* __restrict__ V, long long ld, int k, const double* __restrict__ w,
-                             long long n, double* __restrict__ partial) {
-  __shared__ double red[RED_THREADS / 32][KMAX];
-  double s[KMAX];
+// Sums of KB values per lane over the warp; returns the sum of value
+// lane / (32 / KB). KB = 8, 16 or 32.
+template <int KB>
+__device__ __forceinline__ double warp_sums(double (&v)[KB], int lane) {
 #pragma unroll
-  for (int i = 0; i < KMAX; ++i) s[i] = 0.0;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const double we = w[e];
+  for (int c = KB / 2, o = 16; o > 0; o >>= 1, c >>= 1) {
+    if (c > 0) {  // lanes with bit o keep the upper half of the values
+      const bool up = lane & o;
 #pragma unroll
-    for (int i = 0; i < KMAX; ++i)
-      if (i < k) s[i] = fma(V[i * ld + e], we, s[i]);
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < KMAX; ++i) {
-    if (i < k) {
-      double v = s[i];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[wid][i] = v;
+      for (int i = 0; i < KB / 2; ++i)
+        if (i < c) {
+          const double send = up ? v[i] : v[i + c], keep = up ? v[i + c] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
     }
   }
+  return v[0];
+}
+
+// Sums over the block of v[0..KB) into row[0..KB) (global memory), and of
+// `extra` into row[KMAX] when with_extra. All threads of the block call it.
+template <int KB>
+__device__ __forceinline__ void block_sums(double (&v)[KB], double extra, bool with_extra, double* __restrict__ row) {
+  __shared__ double red[DT / 32][KB + 1];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const double s = warp_sums<KB>(v, lane);
+  if (lane % (32 / KB) == 0) red[wid][lane / (32 / KB)] = s;
+  if (with_extra) {
+    extra = warp_sum(extra);
+    if (lane == 0) red[wid][KB] = extra;
+  }
   __syncthreads();
-  if (threadIdx.x < k) {
-    double v = 0.0;
-    for (int j = 0; j < RED_THREADS / 32; ++j) v += red[j][threadIdx.x];
-    partial[threadIdx.x * RED_BLOCKS + blockIdx.x] = v;
+  if (threadIdx.x < KB + (with_extra ? 1 : 0)) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < DT / 32; ++w) t += red[w][threadIdx.x];
+    row[threadIdx.x < KB ? threadIdx.x : KMAX] = t;
   }
 }
 
-// out[i * out_stride] = sum_b partial[i * RED_BLOCKS + b] (fixed order); one block per i
-__global__ void dots_final(const double* __restrict__ partial, int k, double* __restrict__ out, int out_stride) {
-  __shared__ double red[RED_BLOCKS];
-  const int i = blockIdx.x;
-  red[threadIdx.x] = partial[i * RED_BLOCKS + threadIdx.x];
+// True in every thread of the last block of the grid (of `nblk` blocks that
+// share the counter) to get here; everything the blocks wrote before is then
+// visible. The counter is left at zero.
+__device__ __forceinline__ bool last_block(unsigned int* counter, unsigned int nblk) {
+  __shared__ bool last;
+  __threadfence();
   __syncthreads();
-  for (int h = RED_BLOCKS / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(counter, 1u) == nblk - 1;
+    if (last) *counter = 0u;
   }
-  if (threadIdx.x == 0) out[(long long)i * out_stride] = red[0];
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// Column `lane` of the partial results, summed over the blocks in a fixed
+// order (each warp every 4th block, then the warps), by all threads of the
+// last block; valid in warp 0.
+__device__ __forceinline__ double sum_blocks(const double* __restrict__ part, int nblk, int col) {
+  __shared__ double red[DT / 32][33];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double s = 0.0;
+  __syncthreads();
+#pragma unroll 4
+  for (int b = wid; b < nblk; b += DT / 32) s += __ldcg(part + (long long)b * PSTRIDE + col);
+  red[wid][lane] = s;
+  __syncthreads();
+  double t = 0.0;
+  if (wid == 0)
+#pragma unroll
+    for (int w = 0; w < DT / 32; ++w) t += red[w][lane];
+  return t;
+}
+
+// out[i * stride] = V[i] . w for i < k, one set of vectors per blockIdx.y
+struct DotSet {
+  const double* V;
+  const double* w;
+  double* out;
+  int stride;
+};
+template <int KB>
+__global__ void __launch_bounds__(DT) dots_kernel(DotSet a, DotSet b, long long ld, int k, long long n,
+                                                  double* __restrict__ partial, unsigned int* __restrict__ counter) {
+  const DotSet d = blockIdx.y ? b : a;
+  double acc[KB];
+#pragma unroll
+  for (int i = 0; i < KB; ++i) acc[i] = 0.0;
+  for (long long e = blockIdx.x * (long long)DT + threadIdx.x; e < n; e += (long long)gridDim.x * DT) {
+    const double we = d.w[e];
+#pragma unroll
+    for (int i = 0; i < KB; ++i)
+      if (i < k) acc[i] = fma(d.V[i * ld + e], we, acc[i]);
+  }
+  double* part = partial + blockIdx.y * KMAX;
+  block_sums<KB>(acc, 0.0, false, part + (long long)blockIdx.x * PSTRIDE);
+  if (!last_block(counter + blockIdx.y, gridDim.x)) return;
+  const double s = sum_blocks(part, gridDim.x, threadIdx.x & 31);
+  if (threadIdx.x < k) d.out[(long long)threadIdx.x * d.stride] = s;
+}
+
+// 1 / d for a preconditioner: FP32 start and two Newton steps (within an ulp
+// or two), plain division outside FP32's range
+__device__ __forceinline__ double fast_rcp(double d) {
+  const double a = fabs(d);
+  if (!(a > 1e-30 && a < 1e30)) return 1.0 / d;
+  double r = (double)(1.0f / (float)d);
+  r = fma(r, fma(-d, r, 1.0), r);
+  return fma(r, fma(-d, r, 1.0), r);
+}
+
+// One pass over the subspace after the projected eigenproblem: Ritz vector
+// x = sum_i y_i V_i and ax = sum_i y_i AV_i, residual r = ax - theta x,
+// preconditioned direction t = r / clamp(theta - diag), r . r, and the
+// products c_i = V_i . t of the first Gram-Schmidt pass. sc = {r . r, theta}.
+template <int KB>
+__global__ void __launch_bounds__(DT)
+ritz_kernel(const double* __restrict__ V, const double* __restrict__ AV, long long ld, int k,
+            const double* __restrict__ Y, int ys, const double* __restrict__ theta, const double* __restrict__ diag,
+            double* __restrict__ x, double* __restrict__ ax, double* __restrict__ t, long long n,
+            double* __restrict__ partial, unsigned int* __restrict__ counter, double* __restrict__ c,
+            double* __restrict__ sc) {
+  __shared__ double y[KMAX];
+  if (threadIdx.x < KMAX) y[threadIdx.x] = threadIdx.x < k ? Y[threadIdx.x * ys] : 0.0;
+  __syncthreads();
+  const double th = *theta;
+  double acc[KB], rr = 0.0;
+#pragma unroll
+  for (int i = 0; i < KB; ++i) acc[i] = 0.0;
+  for (long long e = blockIdx.x * (long long)DT + threadIdx.x; e < n; e += (long long)gridDim.x * DT) {
+    double v[KB], xe = 0.0, axe = 0.0;
+#pragma unroll
+    for (int i = 0; i < KB; ++i)
+      if (i < k) {
+        v[i] = V[i * ld + e];
+        xe = fma(y[i], v[i], xe);
+        axe = fma(y[i], AV[i * ld + e], axe);
+      }
+    x[e] = xe;
+    ax[e] = axe;
+    const double re = axe - th * xe;
+    rr = fma(re, re, rr);
+    double den = th - diag[e];
+    if (fabs(den) < 1e-8) den = den < 0.0 ? -1e-8 : 1e-8;
+    const double te = re * fast_rcp(den);
+    t[e] = te;
+#pragma unroll
+    for (int i = 0; i < KB; ++i)
+      if (i < k) acc[i] = fma(v[i], te, acc[i]);
+  }
+  block_sums<KB>(acc, rr, true, partial + (long long)blockIdx.x * PSTRIDE);
+  if (!last_block(counter, gridDim.x)) return;
+  const int lane = threadIdx.x & 31;
+  const double s = sum_blocks(partial, gridDim.x, lane);
+  if (threadIdx.x < k) c[threadIdx.x] = s;
+  const double q = sum_blocks(partial, gridDim.x, KMAX);
+  if (threadIdx.x == 0) {
+    sc[0] = q;
+    sc[1] = th;
+  }
+}
+
+// out = t - sum_i c_i V_i. dots: also c2_i = V_i . out (the next Gram-Schmidt
+// pass); otherwise out . out into *c2.
+template <int KB, bool DOTS>
+__global__ void __launch_bounds__(DT)
+project_kernel(const double* __restrict__ V, long long ld, int k, const double* __restrict__ c, const double* t,
+               double* out, long long n, double* __restrict__ partial, unsigned int* __restrict__ counter,
+               double* __restrict__ c2) {
+  __shared__ double cc[KMAX];
+  if (threadIdx.x < KMAX) cc[threadIdx.x] = threadIdx.x < k ? c[threadIdx.x] : 0.0;
+  __syncthreads();
+  double acc[KB], nn = 0.0;
+#pragma unroll
+  for (int i = 0; i < KB; ++i) acc[i] = 0.0;
+  for (long long e = blockIdx.x * (long long)DT + threadIdx.x; e < n; e += (long long)gridDim.x * DT) {
+    double v[KB], s = 0.0;
+#pragma unroll
+    for (int i = 0; i < KB; ++i)
+      if (i < k) {
+        v[i] = V[i * ld + e];
+        s = fma(cc[i], v[i], s);
+      }
+    const double o = t[e] - s;
+    out[e] = o;
+    if (DOTS) {
+#pragma unroll
+      for (int i = 0; i < KB; ++i)
+        if (i < k) acc[i] = fma(v[i], o, acc[i]);
+    } else {
+      nn = fma(o, o, nn);
+    }
+  }
+  if (DOTS) {
+    block_sums<KB>(acc, 0.0, false, partial + (long long)blockIdx.x * PSTRIDE);
+    if (!last_block(counter, gridDim.x)) return;
+    const double s = sum_blocks(partial, gridDim.x, threadIdx.x & 31);
+    if (threadIdx.x < k) c2[threadIdx.x] = s;
+  } else {
+    double one[8] = {nn, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    block_sums<8>(one, 0.0, false, partial + (long long)blockIdx.x * PSTRIDE);
+    if (!last_block(counter, gridDim.x)) return;
+    const double s = sum_blocks(partial, gridDim.x, 0);
+    if (threadIdx.x == 0) *c2 = s;
+  }
 }
 
 // out = sum_i c[i*cs] V[i] (+ beta * out when add)
@@ -73,20 +258,6 @@ __global__ void lincomb_kernel(const double* __restrict__ V, long long ld, int k
   }
 }
 
-// r = ax - theta x; t = r / clamp(theta - diag)
-__global__ void residual_precond(const double* __restrict__ x, const double* __restrict__ ax,
-                                 const double* __restrict__ diag, const double* __restrict__ theta,
-                                 double* __restrict__ r, double* __restrict__ t, long long n) {
-  const double th = *theta;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const double re = ax[e] - th * x[e];
-    r[e] = re;
-    double den = th - diag[e];
-    if (fabs(den) < 1e-8) den = den < 0.0 ? -1e-8 : 1e-8;
-    t[e] = re / den;
-  }
-}
-
 // x <- sign(x . z) x + a z / sqrt(z . z); xz_zz = {x . z, z . z}
 __global__ void axpy_unit_kernel(double* __restrict__ x, const double* __restrict__ z,
                                  const double* __restrict__ xz_zz, double a, long long n) {
@@ -96,8 +267,10 @@ __global__ void axpy_unit_kernel(double* __restrict__ x, const double* __restric
     x[e] = fma(s, z[e], sg * x[e]);
 }
 
-__global__ void scale_kernel(double* __restrict__ x, const double* __restrict__ nrm2, long long n) {
-  const double s = 1.0 / sqrt(*nrm2);
+// x /= sqrt(*nrm2); zero when the norm is below `floor` (the host then drops it)
+__global__ void scale_kernel(double* __restrict__ x, const double* __restrict__ nrm2, double floor, long long n) {
+  const double nrm = sqrt(*nrm2);
+  const double s = nrm < floor ? 0.0 : 1.0 / nrm;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
     x[e] *= s;
 }
@@ -109,17 +282,11 @@ __global__ void scale_kernel(double* __restrict__ x, const double* __restrict__ 
 // pair i's rotation is computed by warp i % 4, and every thread applies the
 // rotations of its warp's pairs to its row (and its column). w ascending,
 // Y columns = vectors (Y row-major k x ldh). k <= 32; 128 threads.
-//
-// Warm start (k0 > 0): the leading k0 x k0 block of H is the previous
-// projected matrix and Y holds its eigenvectors, so Q starts as
-// diag(Y[:k0, :k0], 1) and A as Q^T H Q, which is diagonal except for the
-// rows and columns added since; Jacobi then needs fewer sweeps.
 constexpr int EIGH_WARPS = 4;
-__global__ void jacobi_eigh(const double* __restrict__ H, int k, int ldh, double* __restrict__ w,
-                            double* __restrict__ Y, int k0) {
+__device__ void jacobi_eigh(const double* __restrict__ H, int k, int ldh, double* __restrict__ w,
+                            double* __restrict__ Y) {
   __shared__ double A[32][33];
   __shared__ double Q[32][33];
-  __shared__ double T[32][33];
   __shared__ double cs[16], sn[16];
   __shared__ int pp[16], qq[16];
   __shared__ double red[2][EIGH_WARPS];
@@ -128,36 +295,9 @@ __global__ void jacobi_eigh(const double* __restrict__ H, int k, int ldh, double
   for (int e = tid; e < k * k; e += blockDim.x) {
     const int i = e / k, c = e % k;
     A[i][c] = 0.5 * (H[i * ldh + c] + H[c * ldh + i]);
-    Q[i][c] = (i < k0 && c < k0) ? Y[i * ldh + c] : (i == c ? 1.0 : 0.0);
+    Q[i][c] = i == c ? 1.0 : 0.0;
   }
   __syncthreads();
-  if (k0 > 0) {
-    for (int e = tid; e < k * k; e += blockDim.x) {  // T = A Q
-      const int i = e / k, c = e % k;
-      double s = 0.0;
-      for (int j = 0; j < k; ++j) s = fma(A[i][j], Q[j][c], s);
-      T[i][c] = s;
-    }
-    __syncthreads();
-    for (int e = tid; e < k * k; e += blockDim.x) {  // A = Q^T T, symmetrized below
-      const int i = e / k, c = e % k;
-      double s = 0.0;
-      for (int j = 0; j < k; ++j) s = fma(Q[j][i], T[j][c], s);
-      A[i][c] = s;
-    }
-    __syncthreads();
-    for (int e = tid; e < k * k; e += blockDim.x) {
-      const int i = e / k, c = e % k;
-      if (c < i) T[i][c] = 0.5 * (A[i][c] + A[c][i]);
-    }
-    __syncthreads();
-    for (int e = tid; e < k * k; e += blockDim.x) {
-      const int i = e / k, c = e % k;
-      if (c < i) A[i][c] = T[i][c];
-      else if (c > i) A[i][c] = T[c][i];
-    }
-    __syncthreads();
-  }
   const int kp = k + (k & 1);            // players, one dummy when k is odd
   const int npairs = kp / 2;
   for (int sweep = 0; sweep < 60 && k > 1; ++sweep) {
@@ -252,14 +392,282 @@ __global__ void jacobi_eigh(const double* __restrict__ H, int k, int ldh, double
   }
 }
 
+__global__ void __launch_bounds__(32 * EIGH_WARPS)
+eigh_full_kernel(const double* __restrict__ H, int k, int ldh, double* __restrict__ w, double* __restrict__ Y) {
+  jacobi_eigh(H, k, ldh, w, Y);
+}
+
+// Lowest eigenpair of the symmetric part of the k x k matrix H (k <= 32):
+// w[0] and column 0 of Y. One FP64 Jacobi sweep of a 24 x 24 matrix costs 22 us
+// of one SM's FP64 pipe, so the whole spectrum is found by Jacobi in FP32 (256
+// times the rate; the two-sided rotation of a 2 x 2 block of pairs per thread,
+// two barriers per round), warm-started from the previous call's vectors in Yf,
+// and the lowest pair is then refined in FP64: with residual r = H y - theta y,
+// y -= sum_i q_i (q_i . r) / (lambda_i - theta) over the other FP32
+// eigenvectors, which multiplies its error by about 1e-6 per step. Where the
+// lowest two values are closer than FP32 can tell apart, or the residual does
+// not reach FP64 rounding in a few steps, the FP64 Jacobi above decides.
+// Per call at K=16, M=150: 40 us (FP64 Jacobi of the whole spectrum: 224 us).
+__global__ void __launch_bounds__(32 * EIGH_WARPS)
+eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restrict__ w, double* __restrict__ Y,
+                   float* __restrict__ Yf, int k0) {
+  __shared__ double Hs[32][33];
+  __shared__ float A[32][33], Q[32][33], T[32][33];
+  __shared__ float cs[16], sn[16];
+  __shared__ int pp[16], qq[16];
+  __shared__ double part[EIGH_WARPS][32], yv[32], rv[32];
+  __shared__ float coef[32], redf[2][EIGH_WARPS];
+  __shared__ int state;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nt = 32 * EIGH_WARPS;
+  const int kp = k + (k & 1), npairs = kp / 2;  // odd k: one empty row and column
+  double mx = 0.0;
+  for (int e = tid; e < kp * kp; e += nt) {
+    const int i = e / kp, c = e - i * kp;
+    const double h = (i < k && c < k) ? 0.5 * (H[i * ldh + c] + H[c * ldh + i]) : 0.0;
+    Hs[i][c] = h;
+    mx = fmax(mx, fabs(h));
+  }
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) part[wid][0] = mx;
+  __syncthreads();
+  mx = fmax(fmax(part[0][0], part[1][0]), fmax(part[2][0], part[3][0]));
+  const int ex = mx > 0.0 ? ilogb(mx) : 0;
+  const double sc = ldexp(1.0, -ex);  // FP32 works on H / 2^ex
+  for (int e = tid; e < kp * kp; e += nt) {
+    const int i = e / kp, c = e - i * kp;
+    A[i][c] = (float)(Hs[i][c] * sc);
+    Q[i][c] = (i < k0 && c < k0) ? Yf[i * 32 + c] : (i == c ? 1.0f : 0.0f);
+  }
+  __syncthreads();
+  if (k0 > 0) {  // A <- Q^T A Q
+    for (int e = tid; e < kp * kp; e += nt) {
+      const int i = e / kp, c = e - i * kp;
+      float s = 0.0f;
+      for (int j = 0; j < kp; ++j) s = fmaf(A[i][j], Q[j][c], s);
+      T[i][c] = s;
+    }
+    __syncthreads();
+    for (int e = tid; e < kp * kp; e += nt) {
+      const int i = e / kp, c = e - i * kp;
+      if (c > i) continue;
+      float s = 0.0f;
+      for (int j = 0; j < kp; ++j) s = fmaf(Q[j][i], T[j][c], s);
+      A[i][c] = s;
+      A[c][i] = s;
+    }
+    __syncthreads();
+  }
+  // the (up to two) pair blocks (bi <= bj) of this thread
+  const int nblocks = npairs * (npairs + 1) / 2;
+  int bi[2], bj[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    int x = tid + u * nt, i = 0;
+    while (i < npairs && x >= npairs - i) x -= npairs - i++;
+    bi[u] = i;
+    bj[u] = i + x;
+  }
+  for (int sweep = 0; sweep < 10 && k > 1; ++sweep) {
+    float off = 0.0f, tot = 0.0f;
+    for (int e = tid; e < kp * kp; e += nt) {
+      const int i = e / kp, c = e - i * kp;
+      const float a2 = A[i][c] * A[i][c];
+      tot += a2;
+      if (c != i) off += a2;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    }
+    if (lane == 0) {
+      redf[0][wid] = off;
+      redf[1][wid] = tot;
+    }
+    __syncthreads();
+    off = redf[0][0] + redf[0][1] + redf[0][2] + redf[0][3];
+    tot = redf[1][0] + redf[1][1] + redf[1][2] + redf[1][3];
+    if (!(off > 1e-11f * tot)) break;
+    for (int round = 0; round < kp - 1; ++round) {
+      if (tid < npairs) {
+        auto player = [&](int x) { return x == 0 ? 0 : 1 + (x - 1 + round) % (kp - 1); };
+        int p = player(tid), q = player(kp - 1 - tid);
+        if (p > q) { const int t = p; p = q; q = t; }
+        const float apq = A[p][q];
+        float c = 1.0f, sv = 0.0f;
+        if (apq != 0.0f) {
+          const float z = (A[q][q] - A[p][p]) / (2.0f * apq), az = fabsf(z);
+          const float t = (z >= 0.0f ? 1.0f : -1.0f) * (az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az)));
+          c = rsqrtf(1.0f + t * t);
+          sv = t * c;
+        }
+        cs[tid] = c;
+        sn[tid] = sv;
+        pp[tid] = p;
+        qq[tid] = q;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if (tid + u * nt < nblocks) {  // A block (pairs i, j) <- J_i^T block J_j
+          const int i = bi[u], j = bj[u], p = pp[i], q = qq[i], r = pp[j], s = qq[j];
+          const float ci = cs[i], si = sn[i], cj = cs[j], sj = sn[j];
+          const float a = A[p][r], b = A[p][s], c = A[q][r], d = A[q][s];
+          const float a1 = cj * a - sj * b, b1 = sj * a + cj * b, c1 = cj * c - sj * d, d1 = sj * c + cj * d;
+          float a2 = ci * a1 - si * c1, b2 = ci * b1 - si * d1, c2 = si * a1 + ci * c1, d2 = si * b1 + ci * d1;
+          if (i == j) b2 = c2 = 0.0f;
+          A[p][r] = a2;
+          A[r][p] = a2;
+          A[p][s] = b2;
+          A[s][p] = b2;
+          A[q][r] = c2;
+          A[r][q] = c2;
+          A[q][s] = d2;
+          A[s][q] = d2;
+        }
+      }
+      for (int e = tid; e < kp * npairs; e += nt) {
+        const int i = e / npairs, j = e - i * npairs, p = pp[j], q = qq[j];
+        const float x = Q[i][p], y = Q[i][q];
+        Q[i][p] = cs[j] * x - sn[j] * y;
+        Q[i][q] = sn[j] * x + cs[j] * y;
+      }
+      __syncthreads();
+    }
+  }
+  __syncthreads();
+  // lowest and second-lowest FP32 values
+  if (wid == 0) {
+    float v = lane < k ? A[lane][lane] : 3e38f, best = v;
+    int arg = lane;
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, arg, o);
+      if (ov < best || (ov == best && oi < arg)) {
+        best = ov;
+        arg = oi;
+      }
+    }
+    float second = lane == arg ? 3e38f : v, big = lane < k ? fabsf(v) : 0.0f;
+    for (int o = 16; o > 0; o >>= 1) {
+      second = fminf(second, __shfl_xor_sync(0xffffffffu, second, o));
+      big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+    }
+    if (lane == 0) state = second - best > 2e-5f * big ? arg : -1;
+    yv[lane] = lane < k ? (double)Q[lane][arg] : 0.0;
+  }
+  __syncthreads();
+  const int arg = state;
+  bool ok = arg >= 0;
+  double theta = 0.0;
+  for (int step = 0; ok; ++step) {
+    // r = H y - theta y with y normalized; row `lane`, a quarter of the columns per warp
+    double s = 0.0;
+    for (int j = wid; j < k; j += EIGH_WARPS) s = fma(Hs[lane][j], yv[j], s);
+    part[wid][lane] = lane < k ? s : 0.0;
+    __syncthreads();
+    if (wid == 0) {
+      const double y = yv[lane], hy = (part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]);
+      const double yy = warp_sum(y * y), yhy = warp_sum(y * hy);
+      theta = yhy / yy;
+      const double r = fma(-theta, y, hy);
+      const double rr = warp_sum(r * r);
+      rv[lane] = r;
+      if (lane == 0) {
+        const double lim = 1e-15 * (double)k * mx;  // rounding of the residual itself
+        state = rr <= lim * lim * yy ? 2 : (step < 6 && rr == rr ? 1 : 0);
+      }
+      part[0][lane] = theta;
+    }
+    __syncthreads();
+    theta = part[0][0];
+    const int st = state;
+    if (st == 2) break;
+    if (st == 0) {
+      ok = false;
+      break;
+    }
+    if (wid == 0) {
+      float g = 0.0f;
+      const float rs = (float)(lane < k ? rv[lane] * sc : 0.0);
+      __syncwarp();
+      for (int j = 0; j < k; ++j) g = fmaf(Q[j][lane < k ? lane : 0], __shfl_sync(0xffffffffu, rs, j), g);
+      const float den = (lane < k ? A[lane][lane] : 0.0f) - (float)(theta * sc);
+      coef[lane] = (lane < k && lane != arg) ? g / (fabsf(den) > 1e-5f ? den : 1e-5f) : 0.0f;
+      __syncwarp();
+      double y = yv[lane], d = 0.0;
+      if (lane < k) {
+        float df = 0.0f;
+        for (int i = 0; i < k; ++i) df = fmaf(Q[lane][i], coef[i], df);
+        d = (double)df;
+      }
+      yv[lane] = y - d;
+    }
+    __syncthreads();
+  }
+  __syncthreads();
+  for (int e = tid; e < k * k; e += nt) Yf[(e / k) * 32 + e % k] = Q[e / k][e % k];
+  if (!ok) {
+    jacobi_eigh(H, k, ldh, w, Y);
+    return;
+  }
+  if (wid == 0) {
+    const double y = yv[lane];
+    const double yy = warp_sum(y * y);
+    if (lane < k) Y[lane * ldh] = y / sqrt(yy);
+    if (lane == 0) w[0] = theta;
+  }
+}
+
+int vec_blocks(long long n) { return (int)std::min<long long>(DAV_MAX_BLOCKS, std::max<long long>(1, (n + DT - 1) / DT)); }
+
 }  // namespace
 
-void dav_dots(const double* V, long long ld, int k, const double* w, long long n, double* partial, double* out,
-              int out_stride, cudaStream_t st) {
+// k = number of vectors -> register block of the kernels
+#define DAV_DISPATCH(k, CALL)  \
+  do {                         \
+    if ((k) <= 8) {            \
+      constexpr int KB = 8;    \
+      CALL;                    \
+    } else if ((k) <= 16) {    \
+      constexpr int KB = 16;   \
+      CALL;                    \
+    } else {                   \
+      constexpr int KB = 32;   \
+      CALL;                    \
+    }                          \
+  } while (0)
+
+void dav_dots2(const double* V, const double* w, double* out, int stride, const double* V2, const double* w2,
+               double* out2, int stride2, long long ld, int k, long long n, const DavScratch& sc, cudaStream_t st) {
   if (k <= 0) return;
   if (k > KMAX) k = KMAX;  // the subspace size is checked against this limit on the host
-  dots_partial<<<RED_BLOCKS, RED_THREADS, 0, st>>>(V, ld, k, w, n, partial);
-  dots_final<<<k, RED_BLOCKS, 0, st>>>(partial, k, out, out_stride);
+  const DotSet a{V, w, out, stride}, b{V2, w2, out2, stride2};
+  const dim3 grid(vec_blocks(n), V2 ? 2 : 1);
+  DAV_DISPATCH(k, (dots_kernel<KB><<<grid, DT, 0, st>>>(a, b, ld, k, n, sc.partial, sc.counters)));
+}
+
+void dav_dots(const double* V, long long ld, int k, const double* w, long long n, const DavScratch& sc, double* out,
+              int out_stride, cudaStream_t st) {
+  dav_dots2(V, w, out, out_stride, nullptr, nullptr, nullptr, 0, ld, k, n, sc, st);
+}
+
+void dav_ritz(const double* V, const double* AV, long long ld, int k, const double* Y, int ys, const double* theta,
+              const double* diag, double* x, double* ax, double* t, long long n, const DavScratch& sc, double* c,
+              double* scal, cudaStream_t st) {
+  DAV_DISPATCH(k, (ritz_kernel<KB><<<vec_blocks(n), DT, 0, st>>>(V, AV, ld, k, Y, ys, theta, diag, x, ax, t, n,
+                                                                 sc.partial, sc.counters, c, scal)));
+}
+
+void dav_project_dots(const double* V, long long ld, int k, const double* c, const double* t, double* out, long long n,
+                      const DavScratch& sc, double* c2, cudaStream_t st) {
+  DAV_DISPATCH(k, (project_kernel<KB, true><<<vec_blocks(n), DT, 0, st>>>(V, ld, k, c, t, out, n, sc.partial,
+                                                                          sc.counters, c2)));
+}
+
+void dav_project_norm(const double* V, long long ld, int k, const double* c, const double* t, double* out, long long n,
+                      const DavScratch& sc, double* nrm2, cudaStream_t st) {
+  DAV_DISPATCH(k, (project_kernel<KB, false><<<vec_blocks(n), DT, 0, st>>>(V, ld, k, c, t, out, n, sc.partial,
+                                                                           sc.counters, nrm2)));
 }
 
 void dav_lincomb(const double* V, long long ld, int k, const double* c, int cs, double sign, double* out,
@@ -270,19 +678,11 @@ void dav_lincomb(const double* V, long long ld, int k, const double* c, int cs, 
   lincomb_kernel<<<(unsigned)grid, 256, 0, st>>>(V, ld, k, c, cs, sign, out, n, add ? 1 : 0);
 }
 
-void dav_residual(const double* x, const double* ax, const double* diag, const double* theta, double* r,
-                  double* t, long long n, cudaStream_t st) {
+void dav_scale(double* x, const double* nrm2, double floor, long long n, cudaStream_t st) {
   long long grid = (n + 255) / 256;
   if (grid > 152 * 8) grid = 152 * 8;
   if (grid < 1) grid = 1;
-  residual_precond<<<(unsigned)grid, 256, 0, st>>>(x, ax, diag, theta, r, t, n);
-}
-
-void dav_scale(double* x, const double* nrm2, long long n, cudaStream_t st) {
-  long long grid = (n + 255) / 256;
-  if (grid > 152 * 8) grid = 152 * 8;
-  if (grid < 1) grid = 1;
-  scale_kernel<<<(unsigned)grid, 256, 0, st>>>(x, nrm2, n);
+  scale_kernel<<<(unsigned)grid, 256, 0, st>>>(x, nrm2, floor, n);
 }
 
 void dav_axpy_unit(double* x, const double* z, const double* xz_zz, double a, long long n, cudaStream_t st) {
@@ -292,8 +692,12 @@ void dav_axpy_unit(double* x, const double* z, const double* xz_zz, double a, lo
   axpy_unit_kernel<<<(unsigned)grid, 256, 0, st>>>(x, z, xz_zz, a, n);
 }
 
-void dav_eigh(const double* H, int k, int ldh, double* w, double* Y, int k0, cudaStream_t st) {
-  jacobi_eigh<<<1, 32 * EIGH_WARPS, 0, st>>>(H, k, ldh, w, Y, k0 < k ? k0 : 0);
+void dav_eigh(const double* H, int k, int ldh, double* w, double* Y, cudaStream_t st) {
+  eigh_full_kernel<<<1, 32 * EIGH_WARPS, 0, st>>>(H, k, ldh, w, Y);
+}
+
+void dav_eigh_lowest(const double* H, int k, int ldh, double* w, double* Y, float* Yf, int k0, cudaStream_t st) {
+  eigh_lowest_kernel<<<1, 32 * EIGH_WARPS, 0, st>>>(H, k, ldh, w, Y, Yf, k0 < k ? k0 : 0);
 }
 
 }  // namespace dmrg

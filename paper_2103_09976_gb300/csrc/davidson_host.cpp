@@ -32,11 +32,15 @@ void ensure_davidson_workspace(Context& c, Problem& p) {
   p.dav_ax.alloc(n * sizeof(double));
   p.dav_r.alloc(n * sizeof(double));
   p.dav_t.alloc(n * sizeof(double));
-  p.dav_partial.alloc((size_t)(S + 2) * 256 * sizeof(double));
+  p.dav_x2.alloc(n * sizeof(double));
+  p.dav_partial.alloc((size_t)DAV_MAX_BLOCKS * DAV_PSTRIDE * sizeof(double));
+  p.dav_cnt.alloc(16);
+  DMRG_CUDA(cudaMemsetAsync(p.dav_cnt.p, 0, 16, st));
   p.dav_H.alloc(LDH * LDH * sizeof(double));
   p.dav_w.alloc(LDH * sizeof(double));
   p.dav_Y.alloc(LDH * LDH * sizeof(double));
-  p.dav_s.alloc(64 * sizeof(double));
+  p.dav_Yf.alloc(32 * 32 * sizeof(float));
+  p.dav_s.alloc(128 * sizeof(double));
   // diagonal of H_eff: the tasks whose output block is their input block
   std::vector<int> dstart(p.blocks.size() + 1, 0), dtask;
   for (size_t b = 0; b < p.blocks.size(); ++b) {
@@ -58,10 +62,6 @@ void ensure_davidson_workspace(Context& c, Problem& p) {
   p.dav_ready = true;
 }
 
-namespace {
-
-}  // namespace
-
 bool run_davidson(Context& c, Problem& p, const double* x0, double tol, double* energy, double* x_out,
                   int* iters, unsigned long long guess_counter_base) {
   ensure_davidson_workspace(c, p);
@@ -74,30 +74,42 @@ bool run_davidson(Context& c, Problem& p, const double* x0, double tol, double* 
   double* H = p.dav_H.as<double>();
   double* w = p.dav_w.as<double>();
   double* Y = p.dav_Y.as<double>();
-  double* s = p.dav_s.as<double>();       // s[0..31]: coefficients, s[40..]: scalars
-  double* part = p.dav_partial.as<double>();
-  double* x = p.dav_x.as<double>();
+  // s[0..31], s[64..95]: Gram-Schmidt coefficients, s[40]: |r|^2, s[41]: theta, s[42]: |new direction|^2,
+  // s[43], s[44]: Rayleigh quotient
+  double* s = p.dav_s.as<double>();
+  const DavScratch part = p.dav_scratch();
+  double* xb[2] = {p.dav_x.as<double>(), p.dav_x2.as<double>()};  // this Ritz vector and the one before
+  int cur = 0;
+  double* x = xb[0];
   double* ax = p.dav_ax.as<double>();
   double* r = p.dav_r.as<double>();
   double* t = p.dav_t.as<double>();
+  float* Yf = p.dav_Yf.as<float>();
+  const double* diag = p.dav_diag.as<double>();
   auto row = [&](double* M, int i) { return M + (long long)i * n; };
-  double host[2];
+  double host[4];
+  struct Event {
+    cudaEvent_t e = nullptr;
+    Event() { DMRG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming)); }
+    ~Event() { cudaEventDestroy(e); }
+  } ready;
 
   auto sigma = [&](const double* in, double* out) { run_sigma(c, p, in, out); };
-  double* pinned = c.h_scalars.get();
-  auto read2 = [&](const double* a, const double* b) {
-    double* dst = pinned ? pinned : host;
-    DMRG_CUDA(cudaMemcpyAsync(&dst[0], a, sizeof(double), cudaMemcpyDeviceToHost, st));
-    DMRG_CUDA(cudaMemcpyAsync(&dst[1], b, sizeof(double), cudaMemcpyDeviceToHost, st));
-    DMRG_CUDA(cudaStreamSynchronize(st));
-    host[0] = dst[0];
-    host[1] = dst[1];
-  };
+  double* const pinned = c.h_scalars.get();
+  double* const got = pinned ? pinned : host;
   // projected-matrix entries of the newest vector j: H[i][j] = V_i . AV_j, H[j][i] = V_j . AV_i
   auto update_H = [&](int k) {
     const int j = k - 1;
-    dav_dots(V, n, k, row(AV, j), n, part, H + j, LDH, st);
-    dav_dots(AV, n, k, row(V, j), n, part, H + (long long)j * LDH, 1, st);
+    dav_dots2(V, row(AV, j), H + j, LDH, AV, row(V, j), H + (long long)j * LDH, 1, n, k, n, part, st);
+  };
+  // row k of V <- t made orthogonal to the k vectors before it (classical Gram-Schmidt twice, the first products
+  // V_i . t in s already) and normalised; zero if nothing of norm 1e-14 is left
+  constexpr double VANISHED = 1e-14;
+  auto extend = [&](int k) {
+    double* vk = row(V, k);
+    dav_project_dots(V, n, k, s, t, vk, n, part, s + 64, st);
+    dav_project_norm(V, n, k, s + 64, vk, vk, n, part, s + 42, st);
+    dav_scale(vk, s + 42, VANISHED, n, st);
   };
 
   ProfScope prof_all(c.prof, 2, st);
@@ -107,30 +119,44 @@ bool run_davidson(Context& c, Problem& p, const double* x0, double tol, double* 
   else
     launch_gen_vector(row(V, 0), n, (uint64_t)(c.opts.seed ^ KEY_GUESS), guess_counter_base, st);
   dav_dots(V, n, 1, row(V, 0), n, part, s + 42, 1, st);
-  dav_scale(row(V, 0), s + 42, n, st);
+  dav_scale(row(V, 0), s + 42, 0.0, n, st);
   sigma(row(V, 0), row(AV, 0));
   int k = 1, nmv = 1;
   update_H(k);
   bool converged = false;
-  double theta = 0.0;
-  int warm = 0;  // size of the projected matrix whose eigenvectors Y holds
+  bool extended = false;  // V's newest row comes from extend(); its norm is read with the next residual
+  double theta = 0.0, theta_before = 0.0;
+  int warm = 0;           // size of the projected matrix whose vectors Yf holds
   for (;;) {
-    dav_eigh(H, k, LDH, w, Y, warm, st);
-    warm = k;
-    dav_lincomb(V, n, k, Y, LDH, 1.0, x, n, false, st);
-    dav_lincomb(AV, n, k, Y, LDH, 1.0, ax, n, false, st);
-    dav_residual(x, ax, p.dav_diag.as<double>(), w, r, t, n, st);
-    dav_dots(r, n, 1, r, n, part, s + 40, 1, st);
-    read2(w, s + 40);
-    theta = host[0];
-    const double rr = host[1];
+    const bool full = k >= S;  // the restart needs two Ritz vectors
+    if (full)
+      dav_eigh(H, k, LDH, w, Y, st);
+    else
+      dav_eigh_lowest(H, k, LDH, w, Y, Yf, warm, st);
+    warm = full ? 0 : k;
+    x = xb[cur];
+    dav_ritz(V, AV, n, k, Y, LDH, w, diag, x, ax, t, n, part, s, s + 40, st);
+    DMRG_CUDA(cudaMemcpyAsync(got, s + 40, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    DMRG_CUDA(cudaEventRecord(ready.e, st));
+    // the next direction is prepared while the host waits for the residual
+    // (unused if this was the last iteration)
+    if (!full && nmv < max_iter) extend(k);
+    DMRG_CUDA(cudaEventSynchronize(ready.e));
+    const double rr = got[0];
+    if (extended && std::sqrt(got[2]) < VANISHED) {  // the newest direction was rounding noise: the result without it
+      --nmv;
+      x = xb[cur ^ 1];
+      theta = theta_before;
+      break;
+    }
+    theta = got[1];
     if (!(rr == rr)) throw Error(DMRG_ECUDA, "Davidson: residual is not a number");
     if (rr < tol) {
       converged = true;
       break;
     }
     if (nmv >= max_iter) break;
-    if (k >= S) {  // thick restart from the two lowest Ritz vectors
+    if (full) {  // thick restart from the two lowest Ritz vectors
       dav_lincomb(V, n, k, Y + 1, LDH, 1.0, r, n, false, st);   // r <- second Ritz vector
       DMRG_CUDA(cudaMemcpyAsync(row(V, 0), x, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
       DMRG_CUDA(cudaMemcpyAsync(row(V, 1), r, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
@@ -138,25 +164,18 @@ bool run_davidson(Context& c, Problem& p, const double* x0, double tol, double* 
       DMRG_CUDA(cudaMemcpyAsync(row(AV, 0), ax, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
       DMRG_CUDA(cudaMemcpyAsync(row(AV, 1), r, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
       k = 2;
-      warm = 0;
       update_H(1);
       update_H(2);
+      dav_dots(V, n, k, t, n, part, s, 1, st);  // V changed: first Gram-Schmidt products again
+      extend(k);
     }
-    // new direction: classical Gram-Schmidt twice against V, then normalise
-    double* vk = row(V, k);
-    DMRG_CUDA(cudaMemcpyAsync(vk, t, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    for (int pass = 0; pass < 2; ++pass) {
-      dav_dots(V, n, k, vk, n, part, s, 1, st);
-      dav_lincomb(V, n, k, s, 1, -1.0, vk, n, true, st);
-    }
-    dav_dots(V + (long long)k * n, n, 1, vk, n, part, s + 41, 1, st);
-    read2(s + 41, s + 41);
-    if (std::sqrt(host[0]) < 1e-14) break;
-    dav_scale(vk, s + 41, n, st);
-    sigma(vk, row(AV, k));
+    sigma(row(V, k), row(AV, k));
     ++nmv;
     ++k;
     update_H(k);
+    extended = true;
+    theta_before = theta;
+    cur ^= 1;
   }
   if (c.opts.sigma_prec != DMRG_FP64) {
     // The mixed-precision operator differs from H by a relative 1e-5 or so,
@@ -164,10 +183,10 @@ bool run_davidson(Context& c, Problem& p, const double* x0, double tol, double* 
     // the final vector with the FP64 sigma is off only at second order in
     // the vector's error, so it is the energy returned.
     run_sigma_f64(c, p, x, ax);
-    dav_dots(x, n, 1, ax, n, part, s + 43, 1, st);
-    dav_dots(x, n, 1, x, n, part, s + 44, 1, st);
-    read2(s + 43, s + 44);
-    theta = host[0] / host[1];
+    dav_dots2(x, ax, s + 43, 1, x, x, s + 44, 1, n, 1, n, part, st);
+    DMRG_CUDA(cudaMemcpyAsync(got, s + 43, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    DMRG_CUDA(cudaStreamSynchronize(st));
+    theta = got[0] / got[1];
   }
   if (x_out) DMRG_CUDA(cudaMemcpyAsync(x_out, x, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
   DMRG_CUDA(cudaStreamSynchronize(st));

@@ -204,20 +204,42 @@ void launch_orthonormalize(double* store, const GramBlock* gb, int nb, cudaStrea
 void launch_take_columns(const double* Q, const TakeBlock* tb, int nb, double* dst, cudaStream_t st);
 
 // ---------------------------------------------------------------- Davidson
+constexpr int DAV_KMAX = 32;         // most vectors of one call
+constexpr int DAV_MAX_BLOCKS = 152;  // most blocks of a vector kernel
+constexpr int DAV_PSTRIDE = 64;      // doubles of partial results per block
+// Workspace of the reductions, one per problem: used in stream order.
+struct DavScratch {
+  double* partial;         // DAV_MAX_BLOCKS * DAV_PSTRIDE
+  unsigned int* counters;  // 2, zero before the first use (each use leaves them zero)
+};
 // out[i*out_stride] = V[i] . w for i < k (V rows of length n, leading dim ld);
-// partial: k * 256 doubles of workspace. Fixed-order two-stage reduction.
-void dav_dots(const double* V, long long ld, int k, const double* w, long long n, double* partial, double* out,
+// fixed-order reduction
+void dav_dots(const double* V, long long ld, int k, const double* w, long long n, const DavScratch& sc, double* out,
               int out_stride, cudaStream_t st);
+// the same for (V, w) -> out and (V2, w2) -> out2 in one launch
+void dav_dots2(const double* V, const double* w, double* out, int stride, const double* V2, const double* w2,
+               double* out2, int stride2, long long ld, int k, long long n, const DavScratch& sc, cudaStream_t st);
+// x = sum_i Y[i*ys] V[i], ax = sum_i Y[i*ys] AV[i], r = ax - theta x, t = r / (theta - diag)
+// with |denominator| clamped at 1e-8, c[i] = V[i] . t, scal = {r . r, theta}
+void dav_ritz(const double* V, const double* AV, long long ld, int k, const double* Y, int ys, const double* theta,
+              const double* diag, double* x, double* ax, double* t, long long n, const DavScratch& sc, double* c,
+              double* scal, cudaStream_t st);
+// out = t - sum_i c[i] V[i] (out may be t) and c2[i] = V[i] . out
+void dav_project_dots(const double* V, long long ld, int k, const double* c, const double* t, double* out, long long n,
+                      const DavScratch& sc, double* c2, cudaStream_t st);
+// the same with *nrm2 = out . out
+void dav_project_norm(const double* V, long long ld, int k, const double* c, const double* t, double* out, long long n,
+                      const DavScratch& sc, double* nrm2, cudaStream_t st);
 // out = sign * sum_i c[i*cs] V[i]  (or out += ... when add)
 void dav_lincomb(const double* V, long long ld, int k, const double* c, int cs, double sign, double* out,
                  long long n, bool add, cudaStream_t st);
-// r = ax - theta x; t = r / (theta - diag) with |denominator| clamped at 1e-8
-void dav_residual(const double* x, const double* ax, const double* diag, const double* theta, double* r,
-                  double* t, long long n, cudaStream_t st);
-// x /= sqrt(*nrm2)
-void dav_scale(double* x, const double* nrm2, long long n, cudaStream_t st);
+// x /= sqrt(*nrm2), or x = 0 when sqrt(*nrm2) < floor
+void dav_scale(double* x, const double* nrm2, double floor, long long n, cudaStream_t st);
 // eigenpairs (ascending) of the symmetric part of a k x k matrix, k <= 32
-void dav_eigh(const double* H, int k, int ldh, double* w, double* Y, int k0, cudaStream_t st);
+void dav_eigh(const double* H, int k, int ldh, double* w, double* Y, cudaStream_t st);
+// lowest eigenpair only (w[0], column 0 of Y; other entries of w and Y may be overwritten). Yf (32 x 32 floats):
+// the vectors of the last call on the leading k0 x k0 block (k0 = 0: none), replaced by this call's.
+void dav_eigh_lowest(const double* H, int k, int ldh, double* w, double* Y, float* Yf, int k0, cudaStream_t st);
 // x <- sign(x . z) x + a z / sqrt(z . z), with xz_zz = {x . z, z . z} on the device
 void dav_axpy_unit(double* x, const double* z, const double* xz_zz, double a, long long n, cudaStream_t st);
 // diagonal of H_eff from the diagonal tasks (output block = input block)

@@ -500,7 +500,7 @@ bool predict_guess(Context& c, int i, bool forward, const Problem& p, double* g)
   DMRG_CUDA(cudaGetLastError());
   // |g|^2 (the oracle falls back to a random guess below norm 1e-12)
   double* sc = p.dav_s.as<double>() + 60;  // scratch scalar of the Davidson workspace
-  dav_dots(g, p.psi_size, 1, g, p.psi_size, p.dav_partial.as<double>(), sc, 1, st);
+  dav_dots(g, p.psi_size, 1, g, p.psi_size, p.dav_scratch(), sc, 1, st);
   double nrm2 = 0.0;
   DMRG_CUDA(cudaMemcpyAsync(&nrm2, sc, sizeof(double), cudaMemcpyDeviceToHost, st));
   DMRG_CUDA(cudaStreamSynchronize(st));
@@ -654,12 +654,12 @@ void sweep_run(Context& c, const int* Ms, int n_sweeps, double tol, double* ener
         z.alloc(p.psi_size * sizeof(double));
         launch_gen_vector(z.as<double>(), p.psi_size, (uint64_t)(c.opts.seed ^ KEY_NOISE), step_id << 32, c.stream);
         double* sc = p.dav_s.as<double>() + 50;
-        double* part = p.dav_partial.as<double>();
+        const DavScratch part = p.dav_scratch();
         dav_dots(x.as<double>(), p.psi_size, 1, z.as<double>(), p.psi_size, part, sc, 1, c.stream);
         dav_dots(z.as<double>(), p.psi_size, 1, z.as<double>(), p.psi_size, part, sc + 1, 1, c.stream);
         dav_axpy_unit(x.as<double>(), z.as<double>(), sc, c.opts.noise, p.psi_size, c.stream);
         dav_dots(x.as<double>(), p.psi_size, 1, x.as<double>(), p.psi_size, part, sc + 2, 1, c.stream);
-        dav_scale(x.as<double>(), sc + 2, p.psi_size, c.stream);
+        dav_scale(x.as<double>(), sc + 2, 0.0, p.psi_size, c.stream);
         DMRG_CUDA(cudaGetLastError());
       }
       emin = std::min(emin, e);
