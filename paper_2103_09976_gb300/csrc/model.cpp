@@ -783,6 +783,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
           r.pC8 = (short)ib.C8;
           r.p_tile = ib.tile;
           r.pblk = h.in_blk;
+          r.pad[1] = tc_per_stage(r.nterm, tn, ib.n);
           const size_t ri = (size_t)(&r - plan.recs.data());
           for (int q = 0; q < r.nterm; ++q) {
             const Base& x = base[P.order[un.t0 + q]];

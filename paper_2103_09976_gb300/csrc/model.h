@@ -278,7 +278,7 @@ struct TcUnitRec {          // 80-byte header + 16 terms = 464 bytes
   short pR8, pC8;           // psi tile geometry
   long long p_tile;         // psi tiles
   long long slot;           // the item's partial tile (tm x tn, row-major)
-  int pad[2];
+  int pad[2];               // [0]: FP16X2 exponent of the unit's tile scale; [1]: tc_per_stage
   TcTermRec t[TC_MAX_G];
 };
 
@@ -352,6 +352,21 @@ struct TcPlan {
   long long n_units = 0;
   double mma_macs = 0;                  // multiply-adds issued per slice product (padding included)
 };
+
+// Tile positions of a ring stage of the tensor-core kernel (fp16 / bf16 tiles).
+constexpr int TC_STAGE_TILES16 = 192, TC_STAGE_TILES = 128;
+// Terms whose right operators (tn columns; kw of a half's psi columns) share one ring stage.
+inline int tc_stage_terms(int nterm, int tn, int kw, int stage_tiles) {
+  const int tiles = 2 * ((tn + 15) / 16) * 2 * ((kw + 15) / 16), fit = stage_tiles / tiles;
+  return fit < 1 ? 1 : fit < nterm ? fit : nterm;
+}
+// The four cases of a record, one byte each: halves of 64 psi columns and the
+// last half of n columns, for fp16 tiles (low bytes) and bf16 tiles.
+inline int tc_per_stage(int nterm, int tn, int n) {
+  const int last = (n - 1) % 64 + 1;
+  return tc_stage_terms(nterm, tn, 64, TC_STAGE_TILES16) | tc_stage_terms(nterm, tn, last, TC_STAGE_TILES16) << 8 |
+         tc_stage_terms(nterm, tn, 64, TC_STAGE_TILES) << 16 | tc_stage_terms(nterm, tn, last, TC_STAGE_TILES) << 24;
+}
 
 struct TcShape {
   int want_items;           // items to split the work into (a multiple of the SM count)

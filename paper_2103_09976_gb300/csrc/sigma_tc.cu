@@ -40,6 +40,16 @@
 // a K-major operand (S) or an MN-major one (S^T) with no copy: transposed
 // terms only change the shared-memory descriptors.
 //
+// The kernel is bound by its serial instruction streams (the MMA-issuing warp
+// spends a third of its time on MMAs, a seventh waiting, the rest on the control
+// code around them; MMAs at rate would take 2 of the 9.1 ms at K=108, M=2000), and
+// the warps of all roles share one instruction cache. So every role's work has
+// one call site, quotients come from the records or small cases instead of
+// divisions, and a chain and its commits are issued in one elected region: 59 KB
+// of code instead of 74 (one producer) and 86 KB (three). Per sigma, before ->
+// after: 29.1 -> 24.4 ms at K=76, M=4000 (three producers, FP16X2), 11.7 -> 9.1 ms
+// for three producers at K=108, M=2000, where one producer stays at 9.2 ms.
+//
 // Every wait on an mbarrier is bounded (about one second of clock); on a
 // timeout the kernel raises a flag in *err, stops issuing work, waits (again
 // bounded) for its own copies, frees its tensor memory and returns.
@@ -61,7 +71,7 @@ constexpr int A2_SLICE = 16 * 1024;             // X half: 16 row groups x 8 K g
 constexpr int A2_OFF = 0;                       // A2 first: reads past its last slice land in stage 0
 constexpr int NMETA = 8;                        // unit records in the shared-memory ring
 constexpr int PREFETCH = 4;                     // records fetched ahead of the producer
-constexpr long long WAIT_CYCLES = 2000000000ll; // ~1 s at 2 GHz
+constexpr uint32_t WAIT_CYCLES = 2000000000u;   // ~1 s at 2 GHz (below a wrap of the 32-bit clock)
 
 // Shared-memory layout of one precision. Operator and psi tiles are stored
 // slice-interleaved: tile position k holds its NSL 8x8 slices (bf16 hi, mid,
@@ -76,7 +86,7 @@ struct Lay {
   static constexpr int NSL = F16 ? 2 : 3;
   static constexpr int TILE = 128 * NSL;
   static constexpr int STAGES = 3;
-  static constexpr int STAGE_TILES = F16 ? 192 : 128;
+  static constexpr int STAGE_TILES = F16 ? TC_STAGE_TILES16 : TC_STAGE_TILES;
   static constexpr int KG1 = F16 ? 6 : 4;
   static constexpr int PSI_TILE = 16 * KG1;
   static constexpr int NA2 = F16 ? 2 : 1;
@@ -146,6 +156,12 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+__device__ __forceinline__ uint32_t clock32() {
+  uint32_t t;
+  asm volatile("mov.u32 %0, %%clock;\n" : "=r"(t)::"memory");
+  return t;
+}
+
 // Bounded wait; returns false (and raises the abort flag) on timeout or if
 // another role already aborted. `code` names the barrier kind (wait
 // accounting and the error report). With wait accounting (PROF) the first
@@ -154,14 +170,14 @@ template <bool PROF>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                           int* err, int code) {
   if (PROF ? mbar_test(bar, parity) : mbar_try(bar, parity)) return true;
-  long long t0 = clock64();
+  const uint32_t t0 = clock32();
   for (;;) {
     if (mbar_try(bar, parity)) {
-      if (PROF) atomicAdd(&s_wait[code & 15], (unsigned long long)(clock64() - t0));
+      if (PROF) atomicAdd(&s_wait[code & 15], (unsigned long long)(clock32() - t0));
       return true;
     }
     if (*abort_flag) return false;
-    if (clock64() - t0 > WAIT_CYCLES) {
+    if (clock32() - t0 > WAIT_CYCLES) {
       *abort_flag = 1;
       atomicExch(err, code);
       return false;
@@ -217,21 +233,29 @@ __host__ __device__ __forceinline__ int kg2_of(int kw) { return 2 * ((kw + 15) >
 // of the block), the K-group stride when transposed (tn8 when the tile spans
 // all stored columns); otherwise kg2 / te. Runs measured 4% faster with one
 // producer (small blocks) and 3.5% slower with three (large blocks).
-__host__ __device__ __forceinline__ int b_stride(const TcUnitRec& r, int j, int h, bool runs) {
-  const int kg2 = kg2_of(half_cols(r, j, h)), kgx = 16 * j + 8 * h, tn8 = (r.tn + 7) >> 3;
-  if (r.flags & TC_TB) return runs && tn8 == r.bC8 ? tn8 : tn8e(r);
-  return runs && min(kg2, r.bC8 - kgx) == r.bC8 ? r.bC8 : kg2;
+__device__ __forceinline__ int b_stride(int flags, int tn, int bC8, int kgx, int kg2, bool runs) {
+  const int tn8 = (tn + 7) >> 3;
+  if (flags & TC_TB) return runs && tn8 == bC8 ? tn8 : 2 * ((tn + 15) >> 4);
+  return runs && min(kg2, bC8 - kgx) == bC8 ? bC8 : kg2;
+}
+// Terms of a unit whose right operators share one stage (halves of 64 columns,
+// and the last, narrower one): from the record (tc_per_stage), which spares every
+// role a division per half.
+template <bool F16>
+__device__ __forceinline__ int terms_per_stage(int per_stage, int kw) {
+  return (per_stage >> ((F16 ? 0 : 16) + (kw == 64 ? 0 : 8))) & 0xff;
 }
 // Terms per flush group: the most whose main K steps in one half stay within
 // max_chain (at least one); max_chain <= 0: the whole unit.
-__device__ __forceinline__ int flush_terms(const TcUnitRec& r, int max_chain) {
-  const int steps = (min(64, r.n) + 15) >> 4;
-  return max_chain > 0 ? max(1, min(r.nterm, max_chain / steps)) : r.nterm;
+__device__ __forceinline__ int flush_terms(int n, int nterm, int max_chain) {
+  const int steps = (min(64, n) + 15) >> 4;  // 1 .. 4: no division
+  const int most = steps == 4 ? max_chain >> 2 : steps == 2 ? max_chain >> 1 : steps == 1 ? max_chain : max_chain / 3;
+  return max_chain > 0 ? max(1, min(nterm, most)) : nterm;
 }
 // A unit of one term whose chunk fits the chain limit accumulates both
 // halves of chunk j in one group (one flush per chunk instead of per half).
-__device__ __forceinline__ bool whole_chunk_group(const TcUnitRec& r, int j, int max_chain) {
-  return r.nterm == 1 && (max_chain <= 0 || ((chunk_cols(r, j) + 15) >> 4) <= max_chain);
+__device__ __forceinline__ bool whole_chunk_group(int nterm, int ccols, int max_chain) {
+  return nterm == 1 && (max_chain <= 0 || ((ccols + 15) >> 4) <= max_chain);
 }
 
 // A unit's geometry, read once from its record in shared memory (the
@@ -264,68 +288,88 @@ __device__ __forceinline__ UnitGeo geo_of(const TcUnitRec& r) {
 // Copies of one stage-1 stage (psi columns of chunk j, K groups KG1*k ..):
 // the stacked left-operator rows of every term ([M group][K group], or
 // [K group][M group] when the left operator is used transposed) and the psi
-// tiles ([K group][N group] from PSI_TILE on); the list holds the operator
-// copies, then one psi copy per K group. (Moving the stage's tiles of a term
-// or of psi as one run where the stored block allows, with the run's stride
-// in shared memory, measured slower on large blocks and no faster on small
-// ones: only stage 2 does it.) f(src_tile, operand (0 operators, 1 psi),
-// dst_tile, n_tiles) moves n_tiles tile positions; lane l issues copies l,
-// l + 32, ... count_only: issue nothing, return the stage's tile positions
-// (the same on every lane).
-template <int KG1, class F>
-__device__ __forceinline__ uint32_t copies_s1(const TcUnitRec& r, const UnitGeo& g, int j, int k, int lane,
-                                              bool count_only, F&& f) {
-  constexpr int PSI_TILE = 16 * KG1;
-  const int kg0 = KG1 * k;
-  const bool tA = g.flags & TC_TA;
-  const int nkA = tA ? min(KG1, g.aR8 - kg0) : min(KG1, g.aC8 - kg0);  // K groups of A in this stage
-  const int nA = nkA > 0 ? (tA ? g.G * nkA : g.G * g.tm8) : 0;         // A copies
-  const int perA = tA ? g.tm8 : nkA;                                    // tiles per A copy
-  const int nkP = max(0, min(KG1, g.pR8 - kg0)), nn = min(16, g.pC8 - 16 * j);
-  const int ntot = nA + nkP;
-  if (count_only) return (uint32_t)(nA * perA + nkP * nn);
-  for (int c = lane; c < ntot; c += 32) {
-    if (c >= nA) {
-      const int kg = c - nA;
-      f(g.p_tile + (long long)(kg0 + kg) * g.pC8 + 16 * j, 1, PSI_TILE + kg * 16, nn);
-    } else if (!tA) {
-      const int q = c / g.tm8, rg = c - q * g.tm8;
-      f(r.t[q].a_tile + (long long)(g.r0g + rg) * g.aC8 + kg0, 0, (q * g.tm8 + rg) * KG1, perA);
-    } else {
-      const int q = c / nkA, kg = c - q * nkA;
-      f(r.t[q].a_tile + (long long)(kg0 + kg) * g.aC8 + g.r0g, 0, kg * 16 + q * g.tm8, perA);
+// tiles ([K group][N group] from PSI_TILE on). (Moving the stage's tiles of a
+// term or of psi as one run where the stored block allows, with the run's
+// stride in shared memory, measured slower on large blocks and no faster on
+// small ones: only stage 2 does it.) A lane's part of the addresses is computed
+// once per sub-unit (CopyS1), without divisions in the stage loop: lane
+// l < 16 moves row group l of the stack (its term's tiles of every K group when
+// transposed), lane 16 + g the psi tiles of K group g.
+template <int KG1>
+struct CopyS1 {
+  static_assert(KG1 <= 16, "psi lanes");
+  long long base;  // lane < 16: first operator tile of its copies; else psi tile of its K group
+  int dst;         // first tile position in the stage
+  bool mine;       // the lane moves something
+  __device__ __forceinline__ CopyS1(const TcUnitRec& r, const UnitGeo& g, int j, int lane) {
+    if (lane >= 16) {
+      base = g.p_tile + (long long)(lane - 16) * g.pC8 + 16 * j;
+      dst = 16 * KG1 + (lane - 16) * 16;
+      mine = lane - 16 < KG1;
+    } else if (g.flags & TC_TA) {  // term `lane`
+      mine = lane < g.G;
+      base = (mine ? r.t[lane].a_tile : 0) + g.r0g;
+      dst = lane * g.tm8;
+    } else {                       // row group `lane` of the stack
+      mine = lane < g.G * g.tm8;
+      const int q = mine ? lane / g.tm8 : 0;
+      base = r.t[q].a_tile + (long long)(g.r0g + lane - q * g.tm8) * g.aC8;
+      dst = lane * KG1;
     }
   }
-  return 0;
-}
+  // tile positions of stage k (the same on every lane)
+  __device__ __forceinline__ static int tiles(const UnitGeo& g, int j, int k) {
+    const int nkA = min(KG1, ((g.flags & TC_TA) ? g.aR8 : g.aC8) - KG1 * k);
+    return g.G * g.tm8 * max(0, nkA) + max(0, min(KG1, g.pR8 - KG1 * k)) * min(16, g.pC8 - 16 * j);
+  }
+  // f(src_tile, psi?, dst_tile, n_tiles) moves n_tiles tile positions
+  template <class F>
+  __device__ __forceinline__ void issue(const UnitGeo& g, int j, int k, int lane, F&& f) const {
+    const int kg0 = KG1 * k;
+    const bool tA = g.flags & TC_TA;
+    const int nkA = min(KG1, (tA ? g.aR8 : g.aC8) - kg0);
+    if (!mine) return;
+    if (lane >= 16) {
+      if (kg0 + lane - 16 < g.pR8) f(base + (long long)kg0 * g.pC8, true, dst, min(16, g.pC8 - 16 * j));
+    } else if (!tA) {
+      if (nkA > 0) f(base + kg0, false, dst, nkA);
+    } else {
+      for (int kg = 0; kg < nkA; ++kg) f(base + (long long)(kg0 + kg) * g.aC8, false, dst + kg * 16, g.tm8);
+    }
+  }
+};
 
 // Copies of one stage-2 stage: the right-operator tiles (output columns of
 // the tile, K groups of half h of chunk j) of terms q0..q1-1, each term in a
 // region of te x kg2 tile positions ([N group][K group], or [K group][N
 // group] when the right operator is used transposed; with runs one copy per
-// term where the block allows, strides as b_stride). As copies_s1.
-template <class F>
-__device__ __forceinline__ uint32_t copies_s2(const TcUnitRec& r, const UnitGeo& g, int j, int h, int q0, int q1,
-                                              bool runs, int lane, bool count_only, F&& f) {
-  const int kw = min(64, min(128, g.n - 128 * j) - 64 * h), kg2 = kg2_of(kw), kgx = 16 * j + 8 * h;
-  const bool tB = g.flags & TC_TB;
-  const int nkB = tB ? min(kg2, g.bR8 - kgx) : min(kg2, g.bC8 - kgx);  // K groups of B present
-  const bool b_run = runs && (tB ? g.tn8 == g.bC8 : nkB == g.bC8);    // one run per term
-  const int per = b_run ? nkB * g.tn8 : (tB ? g.tn8 : nkB);
-  const int span = b_run ? 1 : (tB ? nkB : g.tn8);                    // copies per term
-  const int ncopy = (q1 - q0) * span;
-  if (count_only) return (uint32_t)(ncopy * per);
-  for (int c = lane; c < ncopy; c += 32) {
-    const int qq = c / span, x = c - qq * span, reg = qq * g.te * kg2;
-    if (b_run)
-      f(r.t[q0 + qq].b_tile + (long long)(tB ? kgx : g.c0g) * g.bC8, 0, reg, per);
-    else if (!tB)
-      f(r.t[q0 + qq].b_tile + (long long)(g.c0g + x) * g.bC8 + kgx, 0, reg + x * kg2, per);
-    else
-      f(r.t[q0 + qq].b_tile + (long long)(kgx + x) * g.bC8 + g.c0g, 0, reg + x * g.te, per);
+// term where the block allows, strides as b_stride). With runs lane q moves
+// term q0 + q; otherwise lane x row group x of every term.
+struct CopyS2 {
+  int kgx, kg2, nkB, per, span;
+  bool tB, run;
+  __device__ __forceinline__ CopyS2(const UnitGeo& g, int j, int h, bool runs) {
+    kg2 = kg2_of(min(64, min(128, g.n - 128 * j) - 64 * h));
+    kgx = 16 * j + 8 * h;
+    tB = g.flags & TC_TB;
+    nkB = min(kg2, (tB ? g.bR8 : g.bC8) - kgx);            // K groups of B present
+    run = runs && (tB ? g.tn8 == g.bC8 : nkB == g.bC8);    // one run per term
+    per = run ? nkB * g.tn8 : (tB ? g.tn8 : nkB);          // tiles per copy
+    span = run ? 1 : (tB ? nkB : g.tn8);                   // copies per term
   }
-  return 0;
-}
+  template <class F>
+  __device__ __forceinline__ void issue(const TcUnitRec& r, const UnitGeo& g, int q0, int q1, int lane, F&& f) const {
+    const long long first = tB ? (long long)kgx * g.bC8 + g.c0g : (long long)g.c0g * g.bC8 + kgx;
+    const int reg = g.te * kg2;
+    if (run) {
+      if (lane < q1 - q0) f(r.t[q0 + lane].b_tile + first, false, lane * reg, per);
+    } else if (lane < span) {
+      const int dst = lane * (tB ? g.te : kg2);
+      for (int q = q0; q < q1; ++q)
+        f(r.t[q].b_tile + first + (long long)lane * g.bC8, false, (q - q0) * reg + dst, per);
+    }
+  }
+};
 
 }  // namespace
 
@@ -358,47 +402,41 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
-// One K chain of slice products into tmem_d: the correction products of all
-// NKS K steps first, then the main (hi x hi) ones. a / b: descriptors;
-// a_slice, b_slice: byte offsets of the mid slice; a_kstep, b_kstep: byte
-// offsets of one K step. All offsets are compile-time multiples after
-// unrolling, so the issuing loop is a run of MMAs on precomputed operands.
-// The whole warp evaluates the (uniform) descriptors; the elected lane issues.
-// `first`: the next MMA overwrites the accumulator (cleared after it).
+// Operand of a chain: descriptor halves (the start address in 16-byte units
+// in the low half is advanced by 32-bit additions), and the distances of the
+// next slice and of the next K step in 16-byte units.
+struct MmaOp {
+  uint32_t lo, hi, slice, kstep;
+};
+
+// One K chain of slice products into tmem_d, issued by the calling lane: the
+// correction products of all NKS K steps first, then the main (hi x hi) ones.
+// All offsets are compile-time multiples after unrolling, so the chain is a run
+// of MMAs on precomputed operands. acc = 0: the first MMA overwrites the
+// accumulator.
 template <int NPROD, int NKS>
-__device__ __forceinline__ void mma_chain_k(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t a_slice,
-                                            uint32_t b_slice, uint32_t a_kstep, uint32_t b_kstep, uint32_t idesc,
-                                            bool& first) {
-  const uint32_t alo = (uint32_t)a, ahi = (uint32_t)(a >> 32), blo = (uint32_t)b, bhi = (uint32_t)(b >> 32);
-  const uint32_t as16 = a_slice >> 4, bs16 = b_slice >> 4, ak16 = a_kstep >> 4, bk16 = b_kstep >> 4;
-  uint32_t acc = first ? 0u : 1u;
-  if (elect_one()) {
+__device__ __forceinline__ void mma_chain_k(uint32_t tmem_d, const MmaOp& a, const MmaOp& b, uint32_t idesc,
+                                            uint32_t acc) {
 #pragma unroll
-    for (int ks = 0; ks < NKS; ++ks)
+  for (int ks = 0; ks < NKS; ++ks)
 #pragma unroll
-      for (int p = 1; p < NPROD; ++p) {
-        mma_lohi(tmem_d, alo + prod_i(p) * as16 + ks * ak16, ahi, blo + prod_j(p) * bs16 + ks * bk16, bhi, idesc,
-                 acc);
-        acc = 1u;
-      }
-#pragma unroll
-    for (int ks = 0; ks < NKS; ++ks) {
-      mma_lohi(tmem_d, alo + ks * ak16, ahi, blo + ks * bk16, bhi, idesc, acc);
+    for (int p = 1; p < NPROD; ++p) {
+      mma_lohi(tmem_d, a.lo + prod_i(p) * a.slice + ks * a.kstep, a.hi, b.lo + prod_j(p) * b.slice + ks * b.kstep, b.hi,
+               idesc, acc);
       acc = 1u;
     }
-  }
-  first = false;
+#pragma unroll
+  for (int ks = 0; ks < NKS; ++ks) mma_lohi(tmem_d, a.lo + ks * a.kstep, a.hi, b.lo + ks * b.kstep, b.hi, idesc, acc);
 }
 
 template <int NPROD>
-__device__ __forceinline__ void mma_chain(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t a_slice,
-                                          uint32_t b_slice, uint32_t a_kstep, uint32_t b_kstep, int nks,
-                                          uint32_t idesc, bool& first) {
+__device__ __forceinline__ void mma_chain(uint32_t tmem_d, const MmaOp& a, const MmaOp& b, int nks, uint32_t idesc,
+                                          uint32_t acc) {
   switch (nks) {
-    case 1: mma_chain_k<NPROD, 1>(tmem_d, a, b, a_slice, b_slice, a_kstep, b_kstep, idesc, first); break;
-    case 2: mma_chain_k<NPROD, 2>(tmem_d, a, b, a_slice, b_slice, a_kstep, b_kstep, idesc, first); break;
-    case 3: mma_chain_k<NPROD, 3>(tmem_d, a, b, a_slice, b_slice, a_kstep, b_kstep, idesc, first); break;
-    default: mma_chain_k<NPROD, 4>(tmem_d, a, b, a_slice, b_slice, a_kstep, b_kstep, idesc, first); break;
+    case 1: mma_chain_k<NPROD, 1>(tmem_d, a, b, idesc, acc); break;
+    case 2: mma_chain_k<NPROD, 2>(tmem_d, a, b, idesc, acc); break;
+    case 3: mma_chain_k<NPROD, 3>(tmem_d, a, b, idesc, acc); break;
+    default: mma_chain_k<NPROD, 4>(tmem_d, a, b, idesc, acc); break;
   }
 }
 
@@ -477,44 +515,42 @@ __global__ void __launch_bounds__(NTHR, 1) sigma_tc_kernel(TcDev a) {
     bool ok = true;
     const char* const ops = (const char*)a.op;
     const char* const ps = (const char*)a.psi;
-    // one stage: wait for it to be free, announce its bytes, issue the copies
     // one stage: if it is this warp's ring slot, wait for the slot to be
-    // free, announce its bytes, issue the copies; every warp counts it
-    auto produce = [&](auto&& copies) {
+    // free, announce its bytes, issue the copies; every warp counts it. The
+    // byte count is announced before any copy can complete: lane 0 arrives
+    // with the expected bytes first, then all lanes issue copies.
+    auto produce = [&](int tiles, auto&& issue) {
       if (!ok) return;
       if (all_slots || stage == (uint32_t)pw) {
         if (!mbar_wait<PROF>(bar(B_EMPTY + stage), phase, abort_flag, a.err, 1)) { ok = false; return; }
         const uint32_t sdst = sbase + STAGE_OFF + stage * STAGE_BYTES;
         const uint32_t fb = bar(B_FULL + stage);
-        // the byte count is announced before any copy can complete: lane 0
-        // arrives with the expected bytes first, then all lanes issue copies
-        const uint32_t tiles = copies([&](long long, int, int, int) {}, true);
-        if (lane == 0) mbar_expect_tx(fb, (uint32_t)TILE * tiles);
+        if (lane == 0) mbar_expect_tx(fb, (uint32_t)TILE * (uint32_t)tiles);
         __syncwarp();
-        copies([&](long long src, int which, int dst, int n) {
-          bulk_g2s(sdst + (uint32_t)dst * TILE, (which ? ps : ops) + src * TILE, (uint32_t)TILE * (uint32_t)n, fb);
-        }, false);
+        issue([&](long long src, bool psi, int dst, int n) {
+          bulk_g2s(sdst + (uint32_t)dst * TILE, (psi ? ps : ops) + src * TILE, (uint32_t)TILE * (uint32_t)n, fb);
+        });
+        __syncwarp();
       }
       if (++stage == STAGES) { stage = 0; phase ^= 1; }
     };
     auto produce_s1 = [&](const TcUnitRec& u, int j) {
       const UnitGeo g = geo_of(u);
+      const CopyS1<KG1> cp(u, g, j, lane);
       const int nk1 = (g.pR8 + KG1 - 1) / KG1;
       for (int k = 0; k < nk1; ++k)
-        produce([&](auto&& f, bool count_only) -> uint32_t {
-          return copies_s1<KG1>(u, g, j, k, lane, count_only, f);
-        });
+        produce(CopyS1<KG1>::tiles(g, j, k), [&](auto&& f) { cp.issue(g, j, k, lane, f); });
     };
     auto produce_s2 = [&](const TcUnitRec& u, int j) {
       const UnitGeo g = geo_of(u);
-      const int ccols = min(128, g.n - 128 * j);
-      for (int h = 0; h < (ccols + 63) >> 6; ++h) {
-        const int kw = min(64, ccols - 64 * h);
-        const int P = max(1, min(g.G, STAGE_TILES / (g.te * kg2_of(kw))));
-        for (int q0 = 0; q0 < g.G; q0 += P)
-          produce([&](auto&& f, bool count_only) -> uint32_t {
-            return copies_s2(u, g, j, h, q0, min(g.G, q0 + P), all_slots, lane, count_only, f);
-          });
+      const int nh = (min(128, g.n - 128 * j) + 63) >> 6;
+      for (int h = 0; h < nh; ++h) {
+        const CopyS2 cp(g, j, h, all_slots);
+        const int P = terms_per_stage<F16>(u.pad[1], min(64, min(128, g.n - 128 * j) - 64 * h));
+        for (int q0 = 0; q0 < g.G; q0 += P) {
+          const int q1 = min(g.G, q0 + P);
+          produce((q1 - q0) * cp.span * cp.per, [&](auto&& f) { cp.issue(u, g, q0, q1, lane, f); });
+        }
       }
     };
     bool no_more = false;
@@ -543,78 +579,80 @@ __global__ void __launch_bounds__(NTHR, 1) sigma_tc_kernel(TcDev a) {
       ++pf_s;
       return true;
     };
-    long long s = 0;
-    int prev_slot = -1, prev_j = 0;  // sub-unit whose stage 2 is still to be produced
-    auto finish_prev = [&]() {
-      if (prev_slot < 0) return;
-      const TcUnitRec& pu = ring[prev_slot];
-      produce_s2(pu, prev_j);
-      if (prev_j == n_chunks(pu) - 1) {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(B_MEMPTY + prev_slot));
-      }
-      prev_slot = -1;
-    };
-    auto unit = [&](int slot) {  // the stages of one record (its slot's full barrier passed)
-      const TcUnitRec& u = ring[slot];
-      if (u.flags & TC_ZERO) {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(B_MEMPTY + slot));
+    // Sub-units (record, chunk) in order; the stage-2 stages of one follow
+    // the stage-1 stages of the next (one call site of each, so that their
+    // code is in the kernel once). Warp 0 takes the records from its prefetch
+    // and pushes the terminator after the last one, before the last sub-unit's
+    // stage-2 operands: the MMA issuer and the other producers read it before
+    // they reach those stages, and they can be more than the ring holds.
+    long long s = 0;                  // records taken
+    int cur = -1, j = 0, nch = 0;     // current record slot, chunk, chunks
+    int prev = -1, prev_j = 0;        // sub-unit whose stage 2 is still to be produced
+    bool done = false;
+    // a record without units was met with a sub-unit pending: its stage 2 comes
+    // now (a run of such records would otherwise fill the record ring, whose
+    // oldest slot that sub-unit still holds)
+    bool zero = false;
+    while (ok) {
+      if (cur >= 0 && ++j < nch) {
+        // next chunk of the same record
       } else {
-        for (int j = 0; j < n_chunks(u) && ok; ++j) {
-          produce_s1(u, j);
-          finish_prev();
-          prev_slot = slot;
-          prev_j = j;
-        }
-      }
-    };
-    if (pw == 0) {
-      for (;;) {
-        while (ok && pf_s < s + PREFETCH && prefetch_one()) {
-        }
-        if (!ok) break;
-        if (s == pf_s) break;  // nothing left
-        const int slot = (int)(s % NMETA);
-        if (!mbar_wait<PROF>(bar(B_MFULL + slot), (uint32_t)((s / NMETA) & 1), abort_flag, a.err, 10)) { ok = false; break; }
-        unit(slot);
-        ++s;
-      }
-      // terminator record, pushed before the last sub-unit's stage-2
-      // operands: the MMA issuer and the other producers read it before they
-      // reach those stages, and they can be more than the ring holds
-      if (ok) {
-        const int slot = (int)(s % NMETA);
-        const uint32_t par = (uint32_t)(((s / NMETA) & 1) ^ 1);
-        if (mbar_wait<PROF>(bar(B_MEMPTY + slot), par, abort_flag, a.err, 11)) {
-          if (lane == 0) {
-            ring[slot].flags = TC_DONE;
-            mbar_arrive(bar(B_MFULL + slot));
+        cur = -1;
+        zero = false;
+        while (ok && !done && cur < 0 && !zero) {
+          const int slot = (int)(s % NMETA);
+          const uint32_t par = (uint32_t)((s / NMETA) & 1);
+          if (pw == 0) {
+            while (ok && pf_s < s + PREFETCH && prefetch_one()) {
+            }
+            if (ok && s == pf_s) {  // nothing left: the terminator
+              if (!mbar_wait<PROF>(bar(B_MEMPTY + slot), par ^ 1u, abort_flag, a.err, 11)) { ok = false; break; }
+              if (lane == 0) {
+                ring[slot].flags = TC_DONE;
+                mbar_arrive(bar(B_MFULL + slot));
+              }
+              __syncwarp();
+              done = true;
+              break;
+            }
           }
-        } else {
-          ok = false;
+          if (!ok || !mbar_wait<PROF>(bar(B_MFULL + slot), par, abort_flag, a.err, 10)) { ok = false; break; }
+          const int fl = ring[slot].flags;
+          if (fl & TC_DONE) {
+            done = true;
+          } else if (fl & TC_ZERO) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_MEMPTY + slot));
+            if (prev >= 0) zero = true;
+          } else {
+            cur = slot;
+            j = 0;
+            nch = n_chunks(ring[slot]);
+          }
+          ++s;
         }
-        __syncwarp();
       }
-      if (ok) finish_prev();
-      __syncwarp();
+      if (!ok) break;
+      if (cur >= 0) produce_s1(ring[cur], j);
+      if (prev >= 0) {
+        produce_s2(ring[prev], prev_j);
+        if (prev != cur) {  // that was the record's last chunk
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(B_MEMPTY + prev));
+        }
+      }
+      if (cur < 0 && !zero) break;
+      prev = cur;
+      prev_j = j;
+    }
+    __syncwarp();
+    if (pw == 0) {
       // drain: wait (bounded) until the MMA side released every stage (the
       // copies of all producer warps have landed once a stage is released)
       for (int k = 0; k < STAGES; ++k) {
         mbar_wait<PROF>(bar(B_EMPTY + stage), phase, abort_flag, a.err, 0);
         if (++stage == STAGES) { stage = 0; phase ^= 1; }
       }
-    } else {
-      // records in ring order until the terminator
-      while (ok) {
-        const int slot = (int)(s % NMETA);
-        if (!mbar_wait<PROF>(bar(B_MFULL + slot), (uint32_t)((s / NMETA) & 1), abort_flag, a.err, 10)) { ok = false; break; }
-        if (ring[slot].flags & TC_DONE) break;
-        unit(slot);
-        ++s;
-      }
-      if (ok) finish_prev();
-      __syncwarp();
     }
   } else if (warp == 1) {
     // --------------------------------------------------------------- MMA
@@ -635,69 +673,81 @@ __global__ void __launch_bounds__(NTHR, 1) sigma_tc_kernel(TcDev a) {
       uint32_t h2 = 0;                     // halves consumed: A2 buffer h2 % NA2, parity (h2 / NA2) & 1
       uint32_t sb = 0, sph_empty = 3u;     // bit b: expected parity of S-empty[b]
       bool ok = true;
+      // 16-byte address of the next full stage
       auto acquire = [&]() -> uint32_t {
         if (!mbar_wait<PROF>(bar(B_FULL + stage), phase, abort_flag, a.err, 4)) { ok = false; return 0; }
         asm volatile("tcgen05.fence::after_thread_sync;\n");
-        return sbase + STAGE_OFF + stage * STAGE_BYTES;
+        return (sbase + STAGE_OFF + stage * STAGE_BYTES) >> 4;
       };
-      auto release = [&]() {
-        const long long t0 = tick();
-        if (elect_one()) commit(bar(B_EMPTY + stage));
-        tock(15, t0);
+      auto next_stage = [&]() {
         if (++stage == STAGES) { stage = 0; phase ^= 1; }
       };
+      constexpr uint32_t T16 = TILE >> 4, VER = 1u << 14;  // tile position in 16-byte units; descriptor version bit
+      // what this role needs of a unit, read once from its record
+      struct Unit {
+        int flags, G, tm8, tn, n, bC8, pR8, per_stage;
+      };
+      auto load_unit = [&](const TcUnitRec& r) {
+        const int4 w0 = *reinterpret_cast<const int4*>(&r.flags), w1 = *reinterpret_cast<const int4*>(&r.tm8);
+        static_assert(offsetof(TcUnitRec, tn) == 12 && offsetof(TcUnitRec, tm8) == 16, "record layout");
+        return Unit{w0.x, w0.y, w1.x, w0.w, r.n, r.bC8, r.pR8, r.pad[1]};
+      };
       // stage 1 of sub-unit (u, j): X = stacked left rows x psi chunk j
-      auto mma_s1 = [&](const TcUnitRec& u, int j) {
+      auto mma_s1 = [&](const Unit& u, int j) {
         const uint32_t xb = xcnt & 1;
         if (!mbar_wait<PROF>(bar(B_XEMPTY + xb), (xph_empty >> xb) & 1u, abort_flag, a.err, 3)) { ok = false; return; }
         xph_empty ^= 1u << xb;
-        asm volatile("tcgen05.fence::after_thread_sync;\n");
         const uint32_t tmem_x = tmem + xb * 128;
-        const int tA = (u.flags & TC_TA) ? 1 : 0;
-        const uint32_t id1 = idesc_of<F16>(16 * ((chunk_cols(u, j) + 15) / 16), tA, 1);
-        const uint32_t a_lbo = tA ? 16u * TILE : TILE, a_sbo = tA ? TILE : (uint32_t)KG1 * TILE;
-        const int pR8 = u.pR8, nk1 = k1_stages<KG1>(u);  // read once: the waits below clobber memory
-        bool first = true;
-        for (int k = 0; k < nk1 && ok; ++k) {
+        const bool tA = u.flags & TC_TA;
+        const uint32_t id1 = idesc_of<F16>((min(128, u.n - 128 * j) + 15) & ~15, tA, 1);
+        const uint32_t a_lbo = tA ? 16u * T16 : T16, a_sbo = tA ? T16 : (uint32_t)KG1 * T16;
+        MmaOp oa{0u, a_sbo | VER, 8u, 2 * a_lbo}, ob{0u, T16 | VER, 8u, 2 * 16u * T16};
+        uint32_t acc = 0;
+        for (int left = u.pR8; left > 0; left -= KG1) {
           const uint32_t sst = acquire();
           if (!ok) return;
           const long long t0 = tick();
-          mma_chain<NPROD>(tmem_x, sdesc(sst, a_lbo, a_sbo), sdesc(sst + PSI_TILE * TILE, 16u * TILE, TILE),
-                           128u, 128u, 2 * a_lbo, 2 * 16u * TILE, min(KG1, pR8 - KG1 * k) / 2, id1, first);
+          oa.lo = sst | (a_lbo << 16);
+          ob.lo = (sst + PSI_TILE * T16) | (16u * T16 << 16);
+          if (elect_one()) {
+            mma_chain<NPROD>(tmem_x, oa, ob, min(KG1, left) >> 1, id1, acc);
+            commit(bar(B_EMPTY + stage));
+            if (left <= KG1) commit(bar(B_XFULL + xb));
+          }
           tock(14, t0);
-          release();
-        }
-        {
-          const long long t0 = tick();
-          if (elect_one()) commit(bar(B_XFULL + xb));
-          tock(15, t0);
+          acc = 1;
+          next_stage();
         }
         ++xcnt;
       };
       // stage 2 of sub-unit (u, j): per half, per term, sigma += X_t R_t^T,
       // the tile accumulator switching buffers after every flush group
-      auto mma_s2 = [&](const TcUnitRec& u, int j) {
-        const int tB = (u.flags & TC_TB) ? 1 : 0, te = tn8e(u), G = u.nterm, F = flush_terms(u, a.max_chain);
-        const uint32_t id2 = idesc_of<F16>(16 * ((u.tn + 15) / 16), 0, tB);
-        const int nh = n_halves(u, j), tm8 = u.tm8, ccols = chunk_cols(u, j);
-        const bool whole = whole_chunk_group(u, j, a.max_chain);
+      auto mma_s2 = [&](const Unit& u, int j) {
+        const bool tB = u.flags & TC_TB;
+        const int te = 2 * ((u.tn + 15) >> 4), G = u.G;
+        const uint32_t id2 = idesc_of<F16>((u.tn + 15) & ~15, 0, tB);
+        const int ccols = min(128, u.n - 128 * j), nh = (ccols + 63) >> 6;
+        const int F = flush_terms(u.n, G, a.max_chain);
+        const bool whole = whole_chunk_group(G, ccols, a.max_chain);
         constexpr bool runs = NP == 1;
-        const int bst0 = b_stride(u, j, 0, runs), bst1 = nh > 1 ? b_stride(u, j, 1, runs) : 0;
-        bool first = true;
-        for (int h = 0; h < nh && ok; ++h) {
+        uint32_t acc = 0;
+        for (int h = 0; h < nh; ++h) {
           const uint32_t hb = h2 % NA2;
           if (!mbar_wait<PROF>(bar(B_A2FULL + hb), (h2 / NA2) & 1u, abort_flag, a.err, 5)) { ok = false; return; }
           ++h2;
-          const uint32_t a2 = sbase + A2_OFF + hb * A2_BYTES;
-          const int kw = min(64, ccols - 64 * h), kg2 = kg2_of(kw), P = max(1, min(G, STAGE_TILES / (te * kg2)));
-          const uint32_t bs = (uint32_t)(h == 0 ? bst0 : bst1) * TILE;
-          const uint32_t b_lbo = tB ? bs : TILE;
-          const uint32_t b_sbo = tB ? TILE : bs;
+          const int kw = min(64, ccols - 64 * h), kg2 = kg2_of(kw), P = terms_per_stage<F16>(u.per_stage, kw);
+          const uint32_t bs = (uint32_t)b_stride(u.flags, u.tn, u.bC8, 16 * j + 8 * h, kg2, runs) * T16;
+          const uint32_t b_lbo = tB ? bs : T16;
+          const uint32_t a2 = ((sbase + A2_OFF + hb * A2_BYTES) >> 4) | (8u << 16);
+          MmaOp oa{0u, 64u | VER, A2_SLICE >> 4, 16u}, ob{0u, (tB ? T16 : bs) | VER, 8u, 2 * b_lbo};
           int qf = 0;  // position of term q in its flush group (q % F)
-          for (int q0 = 0; q0 < G && ok; q0 += P) {
+          for (int q0 = 0; q0 < G; q0 += P) {
             const uint32_t sst = acquire();
             if (!ok) return;
-            for (int q = q0; q < min(G, q0 + P); ++q, qf = qf + 1 == F ? 0 : qf + 1) {
+            const int q1 = min(G, q0 + P);
+            oa.lo = a2 + (uint32_t)(q0 * u.tm8) * 64u;
+            ob.lo = sst | (b_lbo << 16);
+            for (int q = q0; q < q1; ++q) {
               const bool gstart = whole ? h == 0 : qf == 0;
               const bool gend = whole ? h == nh - 1 : (qf == F - 1 || q == G - 1);
               if (gstart) {  // a flush group starts: its tile accumulator must be free
@@ -707,55 +757,72 @@ __global__ void __launch_bounds__(NTHR, 1) sigma_tc_kernel(TcDev a) {
                 }
                 sph_empty ^= 1u << sb;
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
-                first = true;
+                acc = 0;
               }
               const long long t0 = tick();
-              mma_chain<NPROD>(tmem + 256 + sb * 128, sdesc(a2 + (uint32_t)(q * tm8) * 1024u, 128u, 1024u),
-                               sdesc(sst + (uint32_t)((q - q0) * te * kg2) * TILE, b_lbo, b_sbo), A2_SLICE, 128u,
-                               2 * 128u, 2 * b_lbo, kg2 / 2, id2, first);
-              tock(14, t0);
-              if (gend) {  // the group ends: hand the accumulator to the epilogue
-                const long long t1 = tick();
-                if (elect_one()) commit(bar(B_SFULL + sb));
-                tock(15, t1);
-                sb ^= 1;
+              if (elect_one()) {
+                mma_chain<NPROD>(tmem + 256 + sb * 128, oa, ob, kg2 >> 1, id2, acc);
+                if (gend) commit(bar(B_SFULL + sb));  // the group ends: hand the accumulator to the epilogue
+                if (q == q1 - 1) {
+                  commit(bar(B_EMPTY + stage));
+                  if (q1 == G) commit(bar(B_A2EMPTY + hb));
+                }
               }
+              tock(14, t0);
+              acc = 1;
+              if (gend) sb ^= 1;
+              qf = qf + 1 == F ? 0 : qf + 1;
+              oa.lo += (uint32_t)u.tm8 * 64u;
+              ob.lo += (uint32_t)(te * kg2) * T16;
             }
-            release();
+            next_stage();
           }
-          const long long t1 = tick();
-          if (elect_one()) commit(bar(B_A2EMPTY + hb));
-          tock(15, t1);
         }
       };
+      // sub-units in the producers' order: stage 1 of one, then stage 2 of the
+      // one before it (one call site of each)
       long long s = 0;
-      int prev_slot = -1, prev_j = 0;
-      auto finish_prev = [&]() {
-        if (prev_slot < 0 || !ok) return;
-        const TcUnitRec& pu = ring[prev_slot];
-        mma_s2(pu, prev_j);
-        if (prev_j == n_chunks(pu) - 1 && leader) mbar_arrive(bar(B_MEMPTY + prev_slot));
-        prev_slot = -1;
-      };
+      int cur = -1, j = 0, nch = 0, prev = -1, prev_j = 0;
+      Unit uc{}, up{};
+      bool done = false, zero = false;
       while (ok) {
-        const int slot = (int)(s % NMETA);
-        if (!mbar_wait<PROF>(bar(B_MFULL + slot), (uint32_t)((s / NMETA) & 1), abort_flag, a.err, 12)) { ok = false; break; }
-        const TcUnitRec& u = ring[slot];
-        const int fl = u.flags;
-        if (fl & TC_DONE) break;
-        if (fl & TC_ZERO) {
-          if (leader) mbar_arrive(bar(B_MEMPTY + slot));
+        if (cur >= 0 && ++j < nch) {
+          // next chunk of the same record
         } else {
-          for (int j = 0; j < n_chunks(u) && ok; ++j) {
-            mma_s1(u, j);
-            finish_prev();
-            prev_slot = slot;
-            prev_j = j;
+          cur = -1;
+          zero = false;
+          while (!done && cur < 0 && !zero) {
+            const int slot = (int)(s % NMETA);
+            if (!mbar_wait<PROF>(bar(B_MFULL + slot), (uint32_t)((s / NMETA) & 1), abort_flag, a.err, 12)) {
+              ok = false;
+              break;
+            }
+            const int fl = ring[slot].flags;
+            if (fl & TC_DONE) {
+              done = true;
+            } else if (fl & TC_ZERO) {
+              if (leader) mbar_arrive(bar(B_MEMPTY + slot));
+              if (prev >= 0) zero = true;
+            } else {
+              cur = slot;
+              j = 0;
+              uc = load_unit(ring[slot]);
+              nch = (uc.n + 127) >> 7;
+            }
+            ++s;
           }
         }
-        ++s;
+        if (!ok) break;
+        if (cur >= 0) mma_s1(uc, j);
+        if (prev >= 0 && ok) {
+          mma_s2(up, prev_j);
+          if (prev != cur && leader) mbar_arrive(bar(B_MEMPTY + prev));
+        }
+        if (cur < 0 && !zero) break;
+        prev = cur;
+        prev_j = j;
+        up = uc;
       }
-      finish_prev();
     }
     __syncwarp();
   } else if (warp < 2 + NEPI) {
@@ -877,7 +944,7 @@ __global__ void __launch_bounds__(NTHR, 1) sigma_tc_kernel(TcDev a) {
           xph_full ^= 1u << xb;
           asm volatile("tcgen05.fence::after_thread_sync;\n");
           const int nh = n_halves(u, j);
-          const bool whole = whole_chunk_group(u, j, a.max_chain);
+          const bool whole = whole_chunk_group(u.nterm, chunk_cols(u, j), a.max_chain);
           const bool wrows = quarter * 32 < u.nterm * u.tm8 * 8;  // warp-uniform: stacked rows here
           for (int h = 0; h < nh && ok; ++h) {
             const uint32_t hb = h2 % NA2;
@@ -913,7 +980,7 @@ __global__ void __launch_bounds__(NTHR, 1) sigma_tc_kernel(TcDev a) {
             // (with two tile accumulators the MMA would then wait for them)
             // or ends its item. One call site keeps the (unrolled) flush code
             // once in the kernel.
-            const int F = flush_terms(u, a.max_chain);
+            const int F = flush_terms(u.n, u.nterm, a.max_chain);
             const int ng = whole ? (h == nh - 1 ? 1 : 0) : (u.nterm + F - 1) / F;
             const bool item_end = (fl & TC_ITEM_LAST) && j == n_chunks(u) - 1 && h == nh - 1;
             const bool defer = ng <= 2 && !item_end;
