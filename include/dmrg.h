@@ -63,8 +63,8 @@ typedef enum {
  * element lies in [2^14, 2^15)), the 3 products with i + j <= 1, FP32
  * accumulation bounded as for BF16X3; the scales are exact and undone in
  * the coefficients and the flushes. Classes whose blocks are all at most 32
- * wide run on the CUDA cores in FP32 from the same split in every mixed
- * mode. */
+ * wide run with warp-level matrix instructions from the same split in every
+ * mixed mode, with FP32 accumulation of all products above 2^-24 relative. */
 typedef enum { DMRG_FP64 = 0, DMRG_BF16X2 = 1, DMRG_BF16X3 = 2, DMRG_FP16X2 = 3 } dmrg_prec;
 
 typedef struct {
@@ -410,7 +410,7 @@ void dmrg_server_destroy(dmrg_server* s);
  * that kernel; see dmrg_profile_waits); 0 stops.
  * dmrg_profile_read synchronizes the stream and returns, for kernel id
  * `kernel` (0 = sigma product kernels, 1 = sigma reduction, 2 = Davidson
- * vector kernels, 3 = blocking / transformation kernels, 4 = the CUDA-core
+ * vector kernels, 3 = blocking / transformation kernels, 4 = the
  * kernels of the mixed-precision sigma's small classes, also counted in 0),
  * the summed duration in ms and the number of launches. DMRG_EINVAL for
  * unknown ids.

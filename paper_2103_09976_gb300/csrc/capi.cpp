@@ -329,7 +329,7 @@ static void run_sigma_tc(Context& c, Problem& p, const double* d_psi, double* d_
     }
     t.wait_prof = c.d_wait_prof.as<unsigned long long>();
   }
-  DMRG_CUDA(cudaMemsetAsync(p.d_counter.p, 0, sizeof(unsigned int), c.stream));
+  DMRG_CUDA(cudaMemsetAsync(p.d_counter.p, 0, 3 * sizeof(unsigned int), c.stream));
   {
     ProfScope ps_(c.prof, 0, c.stream);
     SmallDev sd;
@@ -344,6 +344,7 @@ static void run_sigma_tc(Context& c, Problem& p, const double* d_psi, double* d_
     sd.n_items = (int)p.tc.small_schedule.size();
     sd.n_mid = p.tc.n_small_mid;
     sd.scratch = p.d_tc_scratch.as<double>();
+    sd.counter = p.d_counter.as<unsigned int>() + 1;
     {
       ProfScope ps4_(c.prof, 4, c.stream);  // the small classes alone (also inside kind 0)
       launch_sigma_small(sd, c.n_sm, c.stream);

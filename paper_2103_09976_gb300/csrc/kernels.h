@@ -85,7 +85,7 @@ struct TcDev {
   unsigned long long* wait_prof;  // optional [17]: wait cycles per barrier kind, total cycles
 };
 
-// Small classes of the mixed-precision sigma on the CUDA cores (see TC_SMALL_MAX).
+// Small classes of the mixed-precision sigma (see TC_SMALL_MAX).
 struct SmallDev {
   const void* op;             // operator split (the tensor-core kernel's tiles)
   const void* psi;            // psi split
@@ -98,6 +98,7 @@ struct SmallDev {
   int n_items;
   int n_mid;                  // kind-2 items (all blocks <= TC_SMALL_MID) at the head of the schedule
   double* scratch;            // partial tiles (item slots)
+  unsigned int* counter;      // [2]: next item of each size class; zero at launch
 };
 void launch_sigma_small(const SmallDev& a, int n_sm, cudaStream_t st);
 

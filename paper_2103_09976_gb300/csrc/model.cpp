@@ -559,7 +559,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
   };
   const double unit_overhead = shape.unit_cost;  // fixed cost of a unit in the item split
   double total = 0;
-  long long n_small[2] = {0, 0};  // CUDA-core terms: all blocks <= TC_SMALL_MID, the rest
+  long long n_small[2] = {0, 0};  // small-class terms: all blocks <= TC_SMALL_MID, the rest
   for (size_t b = 0; b < nblk; ++b) {
     const PsiBlock& ob = blocks[b];
     if (std::max(ob.mL, ob.mR) <= TC_SMALL_MAX)
@@ -595,15 +595,13 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
     long long n_terms = 0;
     double macs = 0;
   };
-  // Terms per CUDA-core item: enough items to fill the resident CTAs several
-  // times over (3 per SM of the <= 16 class, 2 of the rest), at least 8 terms
-  // per warp of a CTA (8 or 4 warps) against the cost of an item's final sum
-  // and its partial tile. Against 512 terms always, per kernel of one sigma:
-  // <= 32 class 222 -> 45 us at K=16, M=150 (22 items before), 857 -> 520 us at
-  // K=54, M=1000; <= 16 class 136 -> 67 us at K=24, M=250.
+  // Terms per small-class item: enough items to fill the resident CTAs (of 4
+  // warps: 6-7 per SM of the <= 16 class, 3-4 of the rest) twice over, at least
+  // 8 terms per warp against the cost of an item's start, its final sum and its
+  // partial tile. (Always 512 terms left 22 items for 152 SMs at K=16, M=150.)
   int small_item[2];
-  small_item[0] = (int)std::min<long long>(512, std::max<long long>(64, n_small[0] / (shape.n_sm * 12)));
-  small_item[1] = (int)std::min<long long>(512, std::max<long long>(32, n_small[1] / (shape.n_sm * 8)));
+  small_item[0] = (int)std::min<long long>(512, std::max<long long>(32, n_small[0] / (shape.n_sm * 14)));
+  small_item[1] = (int)std::min<long long>(512, std::max<long long>(16, n_small[1] / (shape.n_sm * 8)));
   std::vector<Part> parts(nparts);
   in_parallel([&](int j) {
     Part& P = parts[j];
@@ -633,7 +631,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
           }
           TcItem it{(int)b, r0, tm, c0, tn, (int)P.units.size(), 0, 0, P.scratch};
           double acc = 0;
-          std::vector<SmallTerm> sm[2];  // CUDA-core terms: all blocks <= TC_SMALL_MID, the rest
+          std::vector<SmallTerm> sm[2];  // small-class terms: all blocks <= TC_SMALL_MID, the rest
           std::vector<int> smb[2];       // their split-block indices (left, right)
           int k = obase;
           const int kend = obase + (t1 - t0);
@@ -643,7 +641,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
             int e = k;
             while (e < kend && base[P.order[e]].in_blk == h.in_blk && (base[P.order[e]].flags & 3) == (h.flags & 3)) ++e;
             const TcPsiBlock& ib = plan.psi[h.in_blk];
-            // CUDA-core class: the whole output block (one tile) and the psi block are small
+            // small class: the whole output block (one tile) and the psi block are small
             const int wmax = std::max(std::max(ob.mL, ob.mR), std::max(ib.m, ib.n));
             if (wmax <= TC_SMALL_MAX) {
               const int cls = wmax <= TC_SMALL_MID ? 0 : 1;
@@ -683,7 +681,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
             P.icost.push_back(acc);
             P.scratch += (long long)tm * tn;
           }
-          for (int cls = 0; cls < 2; ++cls) {  // CUDA-core items: kind 2 (<= TC_SMALL_MID), kind 1
+          for (int cls = 0; cls < 2; ++cls) {  // small-class items: kind 2 (<= TC_SMALL_MID), kind 1
             const size_t base0 = P.small.size();
             P.small.insert(P.small.end(), sm[cls].begin(), sm[cls].end());
             P.small_blk.insert(P.small_blk.end(), smb[cls].begin(), smb[cls].end());

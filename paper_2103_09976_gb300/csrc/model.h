@@ -285,7 +285,7 @@ struct TcUnitRec {          // 80-byte header + 16 terms = 464 bytes
 // Output tile and its record range; same layout as Item (r_begin/r_end in
 // the place of the task range) so the reduction can read it. kind 0: unit
 // records of the tensor-core kernel; kind 1 / 2: small terms (SmallTerm) of the
-// CUDA-core kernel.
+// small-class kernels.
 struct TcItem {
   int out, r0, nrows, c0, ncols, r_begin, r_end, kind;
   long long slot;
@@ -293,9 +293,8 @@ struct TcItem {
 
 // Classes whose blocks (output tile and psi block) are all at most
 // TC_SMALL_MAX wide fill a tcgen05 instruction (128 x 16 x 16 at least) by a
-// few percent; they run on the CUDA cores instead, in FP32 products of the
-// operators (hi + mid + lo of their split, K <= 32 per product) with FP64
-// sums over terms.
+// few percent; they run with warp-level 16 x 8 x 16 instructions instead, on
+// the same split, with FP32 products (K <= 32) and wider sums over terms.
 constexpr int TC_SMALL_MAX = 32;
 // Small items whose blocks are all at most TC_SMALL_MID wide (kind 2) run
 // with a smaller footprint than the rest of the small classes (kind 1).
@@ -371,7 +370,7 @@ inline int tc_per_stage(int nterm, int tn, int n) {
 struct TcShape {
   int want_items;           // items to split the work into (a multiple of the SM count)
   double unit_cost = 128.0 * 128 * 64;  // fixed cost of a unit in the item split, in multiply-adds
-  int n_sm = 152;           // SMs that share the CUDA-core items
+  int n_sm = 152;           // SMs that share the small-class items
 };
 void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const OpSet& R,
                    const WorkList& wl, TcPlan& plan, const TcShape& shape);

@@ -1,24 +1,39 @@
-// Products of small classes on the CUDA cores (part of the mixed-precision
-// sigma, Sec. II.D-E: the same (term, sector) products as the tensor-core
-// kernel, for the classes whose output tile and psi block are all at most
-// TC_SMALL_MAX wide).
+// Products of small classes with warp-level matrix instructions (part of the
+// mixed-precision sigma, Sec. II.D-E: the same (term, sector) products as the
+// tensor-core kernel, for the classes whose output tile and psi block are all at
+// most TC_SMALL_MAX wide).
 //
 // A tcgen05 instruction is at least 128 x 16 x 16, so a product of 8x8 or
 // 16x16 blocks would use it by a few percent, and such products are most of
 // the (term, block) pairs of a middle bond while carrying about 1% of the
 // flops. Here one warp computes one term at a time,
 //     sigma[tile] += c * (L psi_b) R^T,
-// from the operators and psi in FP32 (products of at most 32 along K,
-// accumulated in FP32: a few 2^-24 relative), summing the terms of an item
-// in FP64 (in FP32 over groups of 8 terms of a warp first). The warps of a CTA take every NW-th term of the item and their
-// sums are added in warp order, so the result does not depend on scheduling.
+// with mma.sync (16 x 8 x 16), whose granularity fits. The split store's 8x8
+// tiles are its fragments: lane l of a warp needs bytes 4l .. 4l+3 of a tile's
+// slice, so operands go from global memory to registers with 128-byte coalesced
+// loads and no shared memory; a transposed use transposes the fragments
+// (movmatrix). psi's fragments stay in registers while the block is the same.
+// The accumulators of X = L psi have the layout of the second product's left
+// fragments, so X only has to be split again.
 //
-// A term of 16 x 16 blocks is ~16k flops against three block loads, so the
-// kernel keeps many terms in flight (two size classes: all blocks <= 16 with
-// 8 warps per CTA and several CTAs per SM, the rest with 4 warps), reads
-// the operands from their bf16 split (no FP64 -> FP32 conversion, which
-// runs on the narrow FP64 pipe), issues all loads of a block before storing
-// any, and computes register-blocked products from shared memory.
+// Arithmetic: FP32 accumulation of slice products. The fp16 split (hi + lo)
+// takes all four products in the first product, and X as three fp16 slices (at
+// least 30 bits; scaled by 2^-20 so that it stays in range) in the second; the
+// bf16 split (hi + mid + lo) takes the six products above 2^-24 in both, X as
+// three bf16 slices. That is the accuracy of FP32 multiply-adds on the summed
+// slices, which this kernel used before (measured below). Terms of a warp are
+// summed in FP32 over groups of 8, groups in float-float (48 bits), warps in
+// FP64 in warp order, so the result does not depend on scheduling.
+//
+// Bound by instruction issue (<= 16: 65% of issue slots) and load latency (<= 32:
+// 12-16 warps per SM of 128-159 registers); a term of 16 x 16 blocks reads 2-3 KB
+// for 18-24 matrix instructions. So a warp takes 16 rows (a term of more rows is
+// shared by two), CTAs are 4 warps, items come from a counter, the next term's
+// record is loaded a term ahead and its L and R before psi and the first product.
+// Both kernels per sigma, against FP32 multiply-adds from shared memory: 1.63 ->
+// 0.82 ms at K=108, M=2000 (FP16X2), 0.74 -> 0.38 ms at K=54, M=1000 (BF16X2), 63
+// -> 41 us at K=24, M=250; error of sigma against 64 bits 1.3e-7 -> 1.2e-7 there.
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "kernels.h"
@@ -27,291 +42,335 @@ namespace dmrg {
 
 namespace {
 
-template <int D>
+// D: size class; NT 8-wide tiles per side, NW warps per CTA, MINB CTAs per SM
+template <int D, bool F16>
 struct SmallCfg;
-template <>
-struct SmallCfg<16> {
-  static constexpr int NW = 8, MINB = 3;
+template <bool F16>
+struct SmallCfg<16, F16> {
+  static constexpr int NT = 2, NW = 4, MINB = F16 ? 7 : 6;
 };
-template <>
-struct SmallCfg<32> {
-  static constexpr int NW = 4, MINB = 2;
+template <bool F16>
+struct SmallCfg<32, F16> {
+  static constexpr int NT = 4, NW = 4, MINB = F16 ? 4 : 3;
 };
+static_assert(TC_SMALL_MAX == 32 && TC_SMALL_MID == 16, "size classes");
 
-template <int D>
-struct Tile;
+// d += a b, 16 x 8 x 16: lane (g = lane / 4, c = lane % 4) holds d[g][2c], d[g][2c+1], d[g+8][..]
+template <bool F16>
+__device__ __forceinline__ void mma16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  if (F16)
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+  else
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
 
-template <int D>
-constexpr int small_smem();
+// transpose of an 8x8 fragment
+__device__ __forceinline__ uint32_t trans8(uint32_t x) {
+  uint32_t r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(r) : "r"(x));
+  return r;
+}
 
-// Load a stored block from its split tiles (8 x 8 tiles, row-major by tile,
-// slices hi / mid / lo at bytes 0 / 128 / 256 of each 384-byte tile
-// position) into a padded FP32 tile: T[r * LD + c] = stored(r, c), or
-// T[c * LD + r] when `trans`. Each value is hi + mid + lo in FP32 (the
-// slices hold 24 significant bits, so this is the FP64 value rounded to
-// FP32 within an ulp); the bf16 -> FP32 widening is a shift on the integer
-// pipe. Lane q takes tile row q (of 8 per tile) and reads its three 16-byte
-// slice rows, all loads of the block first; tile padding holds zeros.
-template <int D, int LD, bool F16>
-__device__ __forceinline__ void load_tiles(float* T, const unsigned char* __restrict__ op, long long tile, int R8,
-                                           int C8, bool trans, int lane) {
-  constexpr int TILE = F16 ? 256 : 384;  // bytes per tile position
-  // tile rows per lane, taken PASS at a time (registers of the <= 32 class)
-  constexpr int PER = (D / 8) * (D / 8) * 8 / 32, PASS = PER < 2 ? PER : 2;
-  const int nrow = R8 * C8 * 8;
-#pragma unroll 1
-  for (int k0 = 0; k0 < PER && 32 * k0 < nrow; k0 += PASS) {
-    uint4 h[PASS], m[PASS], l[PASS];
+// The NSL slices of the tile at byte offset `off` as fragments (zero when !valid).
+template <int NSL>
+__device__ __forceinline__ void load_tile(uint32_t (&f)[NSL], const unsigned char* __restrict__ base, int off,
+                                          bool valid) {
+  const uint32_t* p = reinterpret_cast<const uint32_t*>(base + off);
 #pragma unroll
-    for (int k = 0; k < PASS; ++k) {
-      const int q = lane + 32 * (k0 + k);
-      if (q < nrow) {
-        const uint4* p = reinterpret_cast<const uint4*>(op + (tile + (q >> 3)) * TILE + (q & 7) * 16);
-        h[k] = __ldg(p);
-        m[k] = __ldg(p + 8);
-        if (!F16) l[k] = __ldg(p + 16);
-      }
-    }
+  for (int s = 0; s < NSL; ++s) f[s] = valid ? __ldg(p + 32 * s) : 0u;
+}
+
+// (x0, x1) as three slices, x = s[0] + s[1] + s[2]
+template <bool F16>
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t (&s)[3]) {
 #pragma unroll
-    for (int k = 0; k < PASS; ++k) {
-      const int q = lane + 32 * (k0 + k);
-      if (q < nrow) {
-        const int t = q >> 3, tr = t / C8, tc = t - tr * C8, r = 8 * tr + (q & 7), c0 = 8 * tc;
-        const uint32_t hw[4] = {h[k].x, h[k].y, h[k].z, h[k].w}, mw[4] = {m[k].x, m[k].y, m[k].z, m[k].w};
-        uint32_t lw[4] = {0u, 0u, 0u, 0u};
-        if (!F16) {
-          lw[0] = l[k].x;
-          lw[1] = l[k].y;
-          lw[2] = l[k].z;
-          lw[3] = l[k].w;
-        }
-        float v[8];
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          if (!F16) {
-            v[2 * w] = (__uint_as_float(hw[w] << 16) + __uint_as_float(mw[w] << 16)) + __uint_as_float(lw[w] << 16);
-            v[2 * w + 1] = (__uint_as_float(hw[w] & 0xFFFF0000u) + __uint_as_float(mw[w] & 0xFFFF0000u)) +
-                           __uint_as_float(lw[w] & 0xFFFF0000u);
-          } else {  // fp16 hi + lo (scaled values; the coefficients undo the scales)
-            const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&hw[w]));
-            const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&mw[w]));
-            v[2 * w] = a.x + b.x;
-            v[2 * w + 1] = a.y + b.y;
-          }
-        }
-        if (!trans) {
-          *reinterpret_cast<float4*>(T + r * LD + c0) = make_float4(v[0], v[1], v[2], v[3]);
-          *reinterpret_cast<float4*>(T + r * LD + c0 + 4) = make_float4(v[4], v[5], v[6], v[7]);
-        } else {
-#pragma unroll
-          for (int c = 0; c < 8; ++c) T[(c0 + c) * LD + r] = v[c];
-        }
-      }
+  for (int k = 0; k < 3; ++k) {
+    if (F16) {
+      const __half2 h = __floats2half2_rn(x0, x1);
+      s[k] = *reinterpret_cast<const uint32_t*>(&h);
+      const float2 v = __half22float2(h);
+      x0 -= v.x;
+      x1 -= v.y;
+    } else {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+      s[k] = *reinterpret_cast<const uint32_t*>(&h);
+      x0 -= __uint_as_float(s[k] << 16);
+      x1 -= __uint_as_float(s[k] & 0xFFFF0000u);
     }
   }
 }
 
-// Register-blocked products of one term whose operands are in shared
-// memory: lane (rp, cg) = (lane / 4, lane % 4) owns rows rp + 8i (i < D/8)
-// and columns D/4 * cg .. + D/4 - 1 of X = L psi and of the tile, so one
-// step along K reads D/8 values of a column of L (or X) and D/4 consecutive
-// values of a row of psi (or R^T) as 16-byte loads, for D*D/32 FMAs. Rows
-// and columns past the blocks are computed from stale shared memory and
-// never read: the K loops stay inside the blocks. LD (a multiple of 4 for
-// the 16-byte loads) spreads the D/8 column reads of L over distinct banks.
+// Slice pairs (A slice, B slice) of the two products, smallest first.
+template <bool F16>
+struct Pairs;
 template <>
-struct Tile<16> {
-  static constexpr int LD = 20, RI = 2, CJ = 4;
+struct Pairs<true> {  // first: 2 x 2 slices; second: X has 3
+  static constexpr int N1 = 4, N2 = 5;
+  __device__ static constexpr int a1(int p) { return p == 0 || p == 2 ? 1 : 0; }
+  __device__ static constexpr int b1(int p) { return p <= 1 ? 1 : 0; }
+  __device__ static constexpr int a2(int p) { return p == 0 ? 2 : p <= 2 ? 1 : 0; }
+  __device__ static constexpr int b2(int p) { return p == 1 || p == 3 ? 1 : 0; }
 };
 template <>
-struct Tile<32> {
-  static constexpr int LD = 36, RI = 4, CJ = 8;
+struct Pairs<false> {  // hl, mm, lh, hm, mh, hh
+  static constexpr int N1 = 6, N2 = 6;
+  __device__ static constexpr int a1(int p) { return p == 1 || p == 4 ? 1 : p == 2 ? 2 : 0; }
+  __device__ static constexpr int b1(int p) { return p == 0 ? 2 : p == 1 || p == 3 ? 1 : 0; }
+  __device__ static constexpr int a2(int p) { return a1(p); }
+  __device__ static constexpr int b2(int p) { return b1(p); }
 };
 
-template <int D>
-__device__ __forceinline__ void term_product(float (&y)[Tile<D>::RI][Tile<D>::CJ], const float* sPsi,
-                                             const float* sL, const float* sRt, float* sX, int m, int n, bool idL,
-                                             bool idR, int lane) {
-  constexpr int LD = Tile<D>::LD, RI = Tile<D>::RI, CJ = Tile<D>::CJ;
-  const int rp = lane >> 2, c0 = CJ * (lane & 3);
-  if (!idL) {  // X = L psi (tm x n)
-    float x[RI][CJ];
-#pragma unroll
-    for (int i = 0; i < RI; ++i)
-#pragma unroll
-      for (int j = 0; j < CJ; ++j) x[i][j] = 0.0f;
-    for (int kk = 0; kk < m; ++kk) {
-      float b[CJ];
-#pragma unroll
-      for (int j = 0; j < CJ; j += 4) *reinterpret_cast<float4*>(b + j) = *reinterpret_cast<const float4*>(sPsi + kk * LD + c0 + j);
-#pragma unroll
-      for (int i = 0; i < RI; ++i) {
-        const float a = sL[(rp + 8 * i) * LD + kk];
-#pragma unroll
-        for (int j = 0; j < CJ; ++j) x[i][j] = fmaf(a, b[j], x[i][j]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < RI; ++i)
-#pragma unroll
-      for (int j = 0; j < CJ; j += 4)
-        *reinterpret_cast<float4*>(sX + (rp + 8 * i) * LD + c0 + j) = make_float4(x[i][j], x[i][j + 1], x[i][j + 2], x[i][j + 3]);
-    __syncwarp();
-  }
-  const float* X = idL ? sPsi : sX;
-  if (idR) {  // tile = X
-#pragma unroll
-    for (int i = 0; i < RI; ++i)
-#pragma unroll
-      for (int j = 0; j < CJ; j += 4) *reinterpret_cast<float4*>(&y[i][j]) = *reinterpret_cast<const float4*>(X + (rp + 8 * i) * LD + c0 + j);
-    return;
-  }
-#pragma unroll
-  for (int i = 0; i < RI; ++i)
-#pragma unroll
-    for (int j = 0; j < CJ; ++j) y[i][j] = 0.0f;
-  for (int kk = 0; kk < n; ++kk) {  // tile = X R^T
-    float b[CJ];
-#pragma unroll
-    for (int j = 0; j < CJ; j += 4) *reinterpret_cast<float4*>(b + j) = *reinterpret_cast<const float4*>(sRt + kk * LD + c0 + j);
-#pragma unroll
-    for (int i = 0; i < RI; ++i) {
-      const float a = X[(rp + 8 * i) * LD + kk];
-#pragma unroll
-      for (int j = 0; j < CJ; ++j) y[i][j] = fmaf(a, b[j], y[i][j]);
-    }
-  }
-}
+// 8-byte slot of a running sum: a float-float pair while terms are added, an
+// FP64 number when the warps' sums are added
+union Slot {
+  float2 ff;
+  double d;
+};
 
 template <int D, bool F16>
-__global__ void __launch_bounds__(32 * SmallCfg<D>::NW, SmallCfg<D>::MINB) sigma_small_kernel(SmallDev a) {
-  constexpr int NW = SmallCfg<D>::NW, LD = Tile<D>::LD, BLK = D * LD, RI = Tile<D>::RI, CJ = Tile<D>::CJ;
-  // terms summed in FP32 (scaled products) before each FP64 addition
-  constexpr int GROUP = 8;
-  extern __shared__ __align__(16) float smem[];
+__global__ void __launch_bounds__(32 * SmallCfg<D, F16>::NW, SmallCfg<D, F16>::MINB) sigma_small_kernel(SmallDev a) {
+  constexpr int NT = SmallCfg<D, F16>::NT, NW = SmallCfg<D, F16>::NW, NSL = F16 ? 2 : 3, TILE = 128 * NSL;
+  constexpr int GROUP = 8;           // terms summed in FP32 before each float-float addition
+  using P = Pairs<F16>;
+  // running sums, [warp][element of the lane][lane]
+  __shared__ Slot acc[NW][NT * 4][32];
+  __shared__ int next;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rp = lane >> 2, c0 = CJ * (lane & 3);
-  float* sPsi = smem + warp * 4 * BLK;
-  float* sL = sPsi + BLK;
-  float* sRt = sL + BLK;
-  float* sX = sRt + BLK;
-  for (int qi = blockIdx.x; qi < a.n_items; qi += gridDim.x) {
-    const TcItem it = a.items[a.schedule[qi]];
-    const int tm = it.nrows, tn = it.ncols;
-    double acc[RI][CJ];
-    float grp[RI][CJ];
-#pragma unroll
-    for (int i = 0; i < RI; ++i)
-#pragma unroll
-      for (int j = 0; j < CJ; ++j) {
-        acc[i][j] = 0.0;
-        grp[i][j] = 0.0f;
-      }
-    int cur = -1, ng = 0;
-    for (int t = it.r_begin + warp; t < it.r_end; t += NW) {
-      const SmallTerm tk = a.terms[t];
-      const TcPsiBlock pb = a.pblk[tk.in_blk];
-      const int m = pb.m, n = pb.n;
-      const bool idL = tk.a_tile < 0, idR = tk.b_tile < 0;
-      // the operands of this term; psi only when the block changes (the
-      // terms of a class share it). L is tm x m (stored m x tm when used
-      // transposed); R is kept transposed in shared memory (n x tn), from
-      // its stored tn x n (or n x tn when used transposed).
-      const unsigned char* op = reinterpret_cast<const unsigned char*>(a.op);
-      if (tk.in_blk != cur)
-        load_tiles<D, LD, F16>(sPsi, reinterpret_cast<const unsigned char*>(a.psi), pb.tile, pb.R8, pb.C8, false, lane);
-      if (!idL) {
-        const bool tA = tk.flags & 1;
-        load_tiles<D, LD, F16>(sL, op, tk.a_tile, tA ? (m + 7) / 8 : (tm + 7) / 8, tA ? (tm + 7) / 8 : (m + 7) / 8, tA, lane);
-      }
-      if (!idR) {
-        const bool tB = tk.flags & 2;
-        load_tiles<D, LD, F16>(sRt, op, tk.b_tile, tB ? (n + 7) / 8 : (tn + 7) / 8, tB ? (tn + 7) / 8 : (n + 7) / 8, !tB, lane);
-      }
-      cur = tk.in_blk;
-      __syncwarp();
-      float y[RI][CJ];
-      term_product<D>(y, sPsi, sL, sRt, sX, m, n, idL, idR, lane);
-      if (GROUP == 1) {
-#pragma unroll
-        for (int i = 0; i < RI; ++i)
-#pragma unroll
-          for (int j = 0; j < CJ; ++j) acc[i][j] += tk.scale * (double)y[i][j];
-      } else {
-        const float sc = (float)tk.scale;
-#pragma unroll
-        for (int i = 0; i < RI; ++i)
-#pragma unroll
-          for (int j = 0; j < CJ; ++j) grp[i][j] = fmaf(sc, y[i][j], grp[i][j]);
-        if (++ng == GROUP) {
-#pragma unroll
-          for (int i = 0; i < RI; ++i)
-#pragma unroll
-            for (int j = 0; j < CJ; ++j) {
-              acc[i][j] += (double)grp[i][j];
-              grp[i][j] = 0.0f;
-            }
-          ng = 0;
-        }
-      }
-      __syncwarp();
-    }
-#pragma unroll
-    for (int i = 0; i < RI; ++i)
-#pragma unroll
-      for (int j = 0; j < CJ; ++j) acc[i][j] += (double)grp[i][j];
-    // add the warps' sums in warp order
+  const unsigned char* const op = reinterpret_cast<const unsigned char*>(a.op) + 4 * lane;
+  const unsigned char* const psi = reinterpret_cast<const unsigned char*>(a.psi) + 4 * lane;
+  for (;;) {
+    if (threadIdx.x == 0) next = (int)atomicAdd(a.counter, 1u);
     __syncthreads();
-    double* sum = reinterpret_cast<double*>(smem);
+    const int qi = next;
+    __syncthreads();
+    if (qi >= a.n_items) return;
+    const TcItem it = a.items[a.schedule[qi]];
+    const int tm = it.nrows, tn = it.ncols, tm8 = (tm + 7) >> 3, tn8 = (tn + 7) >> 3;
+    // a warp computes 16 rows of a term: tiles of more rows take two warps per term
+    const int n_rows = tm > 16 ? 2 : 1, step = NW / n_rows, i = warp % n_rows, r8 = 2 * i;
+    float grp[NT][4];
 #pragma unroll
-    for (int i = 0; i < RI; ++i)
+    for (int j = 0; j < NT; ++j)
 #pragma unroll
-      for (int j = 0; j < CJ; ++j) {
-        const int r = rp + 8 * i, c = c0 + j;
-        if (r < tm && c < tn) sum[warp * D * D + r * tn + c] = acc[i][j];
+      for (int e = 0; e < 4; ++e) {
+        grp[j][e] = 0.0f;
+        acc[warp][j * 4 + e][lane].ff = make_float2(0.0f, 0.0f);
       }
+    auto flush_group = [&]() {  // acc += grp (two-sum), grp = 0
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          Slot& s = acc[warp][j * 4 + e][lane];
+          const float2 v = s.ff;
+          const float x = grp[j][e], sum = v.x + x, z = sum - v.x;
+          const float lo = v.y + ((v.x - (sum - z)) + (x - z));
+          const float hi = sum + lo;
+          s.ff = make_float2(hi, lo - (hi - sum));
+          grp[j][e] = 0.0f;
+        }
+    };
+    uint32_t fp[NT][NT][NSL];  // psi^T fragments: [K tile][N tile]
+    int cur = -1, ng = 0, m8 = 0, n8 = 0;
+    const int t0 = it.r_begin + warp / n_rows;
+    SmallTerm nx{};
+    if (t0 < it.r_end) nx = a.terms[t0];
+    for (int t = t0; t < it.r_end; t += step) {
+      const SmallTerm tk = nx;
+      if (t + step < it.r_end) nx = a.terms[t + step];  // in flight during this term
+      const bool idL = tk.a_tile < 0, idR = tk.b_tile < 0, tA = tk.flags & 1, tB = tk.flags & 2;
+      const unsigned char* pp = nullptr;
+      int pc8 = 0;
+      if (tk.in_blk != cur || idL) {
+        const TcPsiBlock pb = a.pblk[tk.in_blk];
+        m8 = (pb.m + 7) >> 3;
+        n8 = (pb.n + 7) >> 3;
+        pp = psi + pb.tile * TILE;
+        pc8 = pb.C8;
+      }
+      // fragments of R for K step ks: [N tile][K tile of the step]
+      const unsigned char* const pr = op + tk.b_tile * TILE;
+      const int rj = (tB ? 1 : n8) * TILE, rk = (tB ? tn8 : 1) * TILE;
+      uint32_t fr[NT][2][NSL];
+      auto load_r = [&](int ks) {
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            load_tile<NSL>(fr[j][h], pr, j * rj + (2 * ks + h) * rk, !idR && j < tn8 && 2 * ks + h < n8);
+      };
+      const unsigned char* const pl = op + tk.a_tile * TILE;
+      const int lr = (tA ? 1 : m8) * TILE, lk = (tA ? tm8 : 1) * TILE;
+      uint32_t fa[NSL][4];
+      auto load_l = [&](int ks) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int r = r8 + (q & 1), k = 2 * ks + (q >> 1);
+          uint32_t v[NSL];
+          load_tile<NSL>(v, pl, r * lr + k * lk, !idL && r < tm8 && k < m8);
+#pragma unroll
+          for (int s = 0; s < NSL; ++s) fa[s][q] = v[s];
+        }
+      };
+      load_l(0);
+      load_r(0);  // in flight during the first product
+      if (tk.in_blk != cur) {
+#pragma unroll
+        for (int k = 0; k < NT; ++k)
+#pragma unroll
+          for (int j = 0; j < NT; ++j) load_tile<NSL>(fp[k][j], pp, (k * pc8 + j) * TILE, k < m8 && j < n8);
+#pragma unroll
+        for (int k = 0; k < NT; ++k)
+#pragma unroll
+          for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int s = 0; s < NSL; ++s) fp[k][j][s] = trans8(fp[k][j][s]);
+        cur = tk.in_blk;
+      }
+      const float sc = (float)tk.scale;
+      // fp16: |X| <= 32 * 2^30 of the scaled operands (2^15 with an identity)
+      const float f = F16 && !idL ? 0x1p-20f : 1.0f, finv = F16 && !idL ? 0x1p20f : 1.0f;
+      float x[NT][4];
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[j][e] = 0.0f;
+      if (!idL) {  // X = L psi
+#pragma unroll
+        for (int ks = 0; ks < NT / 2; ++ks) {
+          if (ks > 0 && 2 * ks >= m8) break;
+          if (ks > 0) load_l(ks);
+          if (tA) {
+#pragma unroll
+            for (int s = 0; s < NSL; ++s)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) fa[s][q] = trans8(fa[s][q]);
+          }
+#pragma unroll
+          for (int p = 0; p < P::N1; ++p)
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+              if (j < n8) mma16<F16>(x[j], fa[P::a1(p)], fp[2 * ks][j][P::b1(p)], fp[2 * ks + 1][j][P::b1(p)]);
+        }
+      } else {  // X = psi (the tile's rows and columns)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            uint32_t v[NSL];
+            load_tile<NSL>(v, pp, ((r8 + h) * pc8 + j) * TILE, r8 + h < m8 && j < n8);
+#pragma unroll
+            for (int s = NSL - 1; s >= 0; --s) {
+              if (F16) {
+                const float2 w = __half22float2(*reinterpret_cast<const __half2*>(&v[s]));
+                x[j][2 * h] += w.x;
+                x[j][2 * h + 1] += w.y;
+              } else {
+                x[j][2 * h] += __uint_as_float(v[s] << 16);
+                x[j][2 * h + 1] += __uint_as_float(v[s] & 0xFFFF0000u);
+              }
+            }
+          }
+      }
+      if (idR) {
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) grp[j][e] = fmaf(sc, x[j][e], grp[j][e]);
+      } else {  // Y = X R^T
+        float y[NT][4];
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) y[j][e] = 0.0f;
+#pragma unroll
+        for (int ks = 0; ks < NT / 2; ++ks) {
+          if (ks > 0 && 2 * ks >= n8) break;
+          if (ks > 0) load_r(ks);
+          if (tB) {
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+              for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int s = 0; s < NSL; ++s) fr[j][h][s] = trans8(fr[j][h][s]);
+          }
+          uint32_t fx[3][4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            uint32_t s3[3];
+            split_pair<F16>(x[2 * ks + (q >> 1)][2 * (q & 1)] * f, x[2 * ks + (q >> 1)][2 * (q & 1) + 1] * f, s3);
+#pragma unroll
+            for (int s = 0; s < 3; ++s) fx[s][q] = s3[s];
+          }
+#pragma unroll
+          for (int p = 0; p < P::N2; ++p)
+#pragma unroll
+            for (int j = 0; j < NT; ++j)
+              if (j < tn8) mma16<F16>(y[j], fx[P::a2(p)], fr[j][0][P::b2(p)], fr[j][1][P::b2(p)]);
+        }
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) grp[j][e] = fmaf(sc, y[j][e] * finv, grp[j][e]);
+      }
+      if (++ng == GROUP) {
+        flush_group();
+        ng = 0;
+      }
+    }
+    flush_group();
+#pragma unroll
+    for (int e = 0; e < NT * 4; ++e) {
+      Slot& s = acc[warp][e][lane];
+      const float2 v = s.ff;
+      s.d = (double)v.x + (double)v.y;
+    }
+    // add the warps' sums in warp order
     __syncthreads();
     double* out = a.scratch + it.slot;
     const double ps = F16 ? ldexp(1.0, psi_exponent(*a.psi_exp) - 14) : 1.0;  // undo psi's split scale
     for (int e = threadIdx.x; e < tm * tn; e += blockDim.x) {
-      double v = sum[e];
-      for (int w = 1; w < NW; ++w) v += sum[w * D * D + e];
+      const int r = e / tn, c = e - r * tn;
+      const int idx = (c >> 3) * 4 + ((r >> 3) & 1) * 2 + (c & 1), ln = (r & 7) * 4 + ((c & 7) >> 1);
+      double v = acc[r >> 4][idx][ln].d;
+      for (int w = (r >> 4) + n_rows; w < NW; w += n_rows) v += acc[w][idx][ln].d;
       out[e] = F16 ? v * ps : v;
     }
-    __syncthreads();
+    // the next item's barriers come before acc is written again
   }
 }
 
-template <int D>
-constexpr int small_smem() {
-  return SmallCfg<D>::NW * 4 * D * Tile<D>::LD * (int)sizeof(float);
-}
-static_assert(SmallCfg<16>::NW * 16 * 16 * (int)sizeof(double) <= small_smem<16>(), "final sums fit");
-static_assert(SmallCfg<32>::NW * 32 * 32 * (int)sizeof(double) <= small_smem<32>(), "final sums fit");
-static_assert(TC_SMALL_MAX == 32 && TC_SMALL_MID == 16, "size classes");
-
-template <int D>
-void launch_class(const SmallDev& a, int n_items, const int* schedule, int n_sm, cudaStream_t st) {
+template <int D, bool F16>
+void launch_class(const SmallDev& a, int n_items, const int* schedule, unsigned int* counter, int n_sm, cudaStream_t st) {
   if (n_items <= 0) return;
-  const void* fn = a.f16 ? (const void*)sigma_small_kernel<D, true> : (const void*)sigma_small_kernel<D, false>;
-  set_max_dynamic_smem(fn, small_smem<D>());
   SmallDev b = a;
   b.schedule = schedule;
   b.n_items = n_items;
-  int grid = SmallCfg<D>::MINB * n_sm;
+  b.counter = counter;
+  int grid = SmallCfg<D, F16>::MINB * n_sm;
   if (grid > n_items) grid = n_items;
-  if (a.f16)
-    sigma_small_kernel<D, true><<<grid, 32 * SmallCfg<D>::NW, small_smem<D>(), st>>>(b);
-  else
-    sigma_small_kernel<D, false><<<grid, 32 * SmallCfg<D>::NW, small_smem<D>(), st>>>(b);
+  sigma_small_kernel<D, F16><<<grid, 32 * SmallCfg<D, F16>::NW, 0, st>>>(b);
+}
+
+template <bool F16>
+void launch_both(const SmallDev& a, int n_sm, cudaStream_t st) {
+  // the schedule lists the <= 16 class first
+  launch_class<16, F16>(a, a.n_mid, a.schedule, a.counter, n_sm, st);
+  launch_class<32, F16>(a, a.n_items - a.n_mid, a.schedule + a.n_mid, a.counter + 1, n_sm, st);
 }
 
 }  // namespace
 
 void launch_sigma_small(const SmallDev& a, int n_sm, cudaStream_t st) {
-  // the schedule lists the <= 16 class first
-  launch_class<16>(a, a.n_mid, a.schedule, n_sm, st);
-  launch_class<32>(a, a.n_items - a.n_mid, a.schedule + a.n_mid, n_sm, st);
+  if (a.f16)
+    launch_both<true>(a, n_sm, st);
+  else
+    launch_both<false>(a, n_sm, st);
 }
 
 }  // namespace dmrg
