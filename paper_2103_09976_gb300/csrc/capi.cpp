@@ -132,7 +132,8 @@ static_assert(sizeof(TcItem) == sizeof(Item), "reduction reads TcItem as Item");
 // operator store is unchanged by it).
 static void prepare_tc_plan(Context& c, Problem& p) {
   cudaStream_t st = c.stream;
-  build_tc_plan(p.blocks, p.L, p.R, p.wl, p.tc, TcShape{c.n_sm * p.tc_items_per_sm, p.tc_unit_cost, c.n_sm});
+  build_tc_plan(p.blocks, p.L, p.R, p.wl, p.tc, 
+                TcShape{c.n_sm * p.tc_items_per_sm, p.tc_unit_cost, c.n_sm, TC_MEDIUM_MAX});
   p.tc_producers[0] = tc_default_producers(p.tc, false);
   p.tc_producers[1] = tc_default_producers(p.tc, true);
   p.d_tc_recs.upload(p.tc.recs, st);
@@ -329,7 +330,7 @@ static void run_sigma_tc(Context& c, Problem& p, const double* d_psi, double* d_
     }
     t.wait_prof = c.d_wait_prof.as<unsigned long long>();
   }
-  DMRG_CUDA(cudaMemsetAsync(p.d_counter.p, 0, 3 * sizeof(unsigned int), c.stream));
+  DMRG_CUDA(cudaMemsetAsync(p.d_counter.p, 0, 4 * sizeof(unsigned int), c.stream));
   {
     ProfScope ps_(c.prof, 0, c.stream);
     SmallDev sd;
@@ -343,7 +344,10 @@ static void run_sigma_tc(Context& c, Problem& p, const double* d_psi, double* d_
     sd.schedule = p.d_tc_small_sched.as<int>();
     sd.n_items = (int)p.tc.small_schedule.size();
     sd.n_mid = p.tc.n_small_mid;
+    sd.n_medium = p.tc.n_medium;
+    sd.nprod = t.nprod;
     sd.scratch = p.d_tc_scratch.as<double>();
+    sd.err = p.d_err.as<int>();
     sd.counter = p.d_counter.as<unsigned int>() + 1;
     {
       ProfScope ps4_(c.prof, 4, c.stream);  // the small classes alone (also inside kind 0)

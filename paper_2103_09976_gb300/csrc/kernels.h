@@ -93,12 +93,15 @@ struct SmallDev {
   int f16;                    // 1: the split is FP16X2's (2 fp16 slices, scaled operands)
   const TcPsiBlock* pblk;     // psi blocks: split tiles and dimensions
   const SmallTerm* terms;
-  const TcItem* items;        // kind-1/2 items index terms
-  const int* schedule;        // kind-2 items, then kind-1 items, each most expensive first
+  const TcItem* items;        // items of kinds 1, 2 and 3 index terms
+  const int* schedule;        // kind-2, kind-1, kind-3 items, each most expensive first
   int n_items;
   int n_mid;                  // kind-2 items (all blocks <= TC_SMALL_MID) at the head of the schedule
+  int n_medium;               // kind-3 items (all blocks <= TC_MEDIUM_MAX) at its tail
+  int nprod;                  // slice products of the medium class: 6 (three bf16 slices) or 3 (two slices)
   double* scratch;            // partial tiles (item slots)
-  unsigned int* counter;      // [2]: next item of each size class; zero at launch
+  int* err;                   // nonzero after a bounded wait of the medium class gave up
+  unsigned int* counter;      // [3]: next item of each size class; zero at launch
 };
 void launch_sigma_small(const SmallDev& a, int n_sm, cudaStream_t st);
 

@@ -559,20 +559,36 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
   };
   const double unit_overhead = shape.unit_cost;  // fixed cost of a unit in the item split
   double total = 0;
-  long long n_small[2] = {0, 0};  // small-class terms: all blocks <= TC_SMALL_MID, the rest
+  // size class of the terms of (output block, psi block): -1 tensor cores, 0 all blocks <= TC_SMALL_MID,
+  // 1 <= TC_SMALL_MAX, 2 <= TC_MEDIUM_MAX
+  int small_max = shape.small_max;
+  auto small_class = [&](const PsiBlock& ob, int in_blk) {
+    const PsiBlock& ib = blocks[in_blk];
+    const int wmax = std::max(std::max(ob.mL, ob.mR), std::max(ib.mL, ib.mR));
+    return wmax > small_max ? -1 : wmax <= TC_SMALL_MID ? 0 : wmax <= TC_SMALL_MAX ? 1 : 2;
+  };
+  long long n_small[3] = {0, 0, 0};  // terms per small class
   for (size_t b = 0; b < nblk; ++b) {
     const PsiBlock& ob = blocks[b];
-    if (std::max(ob.mL, ob.mR) <= TC_SMALL_MAX)
-      for (int t = wl.out_start[b]; t < wl.out_start[b + 1]; ++t) {
-        const PsiBlock& ib = blocks[base[t].in_blk];
-        const int wmax = std::max(std::max(ob.mL, ob.mR), std::max(ib.mL, ib.mR));
-        if (wmax <= TC_SMALL_MAX) ++n_small[wmax <= TC_SMALL_MID ? 0 : 1];
-      }
+    for (int t = wl.out_start[b]; t < wl.out_start[b + 1]; ++t) {
+      const int cls = small_class(ob, base[t].in_blk);
+      if (cls >= 0) ++n_small[cls];
+    }
+  }
+  // the <= 64 class needs enough terms to fill the GPU by itself; fewer join the
+  // tensor cores' items, which run anyway (at K=16, M=150 a kernel of their own
+  // takes 35 us and their partial tiles 18 us of the reduction, and the
+  // tensor-core kernel is 17 us faster without them)
+  constexpr int MEDIUM_TERMS_PER_SM = 64;
+  if (n_small[2] < (long long)MEDIUM_TERMS_PER_SM * shape.n_sm) small_max = std::min(small_max, TC_SMALL_MAX);
+  for (size_t b = 0; b < nblk; ++b) {
+    const PsiBlock& ob = blocks[b];
     for (int r0 = 0; r0 < ob.mL; r0 += 128)
       for (int c0 = 0; c0 < ob.mR; c0 += 128) {
         const int tm = std::min(128, ob.mL - r0), tn = std::min(128, ob.mR - c0);
         const int G = std::max(1, 16 / ceil8(tm));
         for (int t = wl.out_start[b]; t < wl.out_start[b + 1]; ++t) {
+          if (small_class(ob, base[t].in_blk) >= 0) continue;  // not part of the tensor-core items
           const TcPsiBlock& ib = plan.psi[base[t].in_blk];
           total += unit_macs(1, tn, ib.m, ib.n) / G + unit_overhead / G;
         }
@@ -584,7 +600,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
     int t0, t1;
   };
   struct Part {
-    std::vector<TcItem> items;           // kind 0: r_begin/r_end index units; kind 1/2: small terms
+    std::vector<TcItem> items;           // kind 0: r_begin/r_end index units; other kinds: small terms
     std::vector<Group> groups;
     std::vector<std::pair<int, Unit>> units;  // (output block, unit)
     std::vector<SmallTerm> small;
@@ -599,9 +615,12 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
   // warps: 6-7 per SM of the <= 16 class, 3-4 of the rest) twice over, at least
   // 8 terms per warp against the cost of an item's start, its final sum and its
   // partial tile. (Always 512 terms left 22 items for 152 SMs at K=16, M=150.)
-  int small_item[2];
+  // The <= 64 class (12 warps, one CTA per SM) holds one psi block per item in
+  // shared memory: 6 items per SM.
+  int small_item[3];
   small_item[0] = (int)std::min<long long>(512, std::max<long long>(32, n_small[0] / (shape.n_sm * 14)));
   small_item[1] = (int)std::min<long long>(512, std::max<long long>(16, n_small[1] / (shape.n_sm * 8)));
+  small_item[2] = (int)std::min<long long>(512, std::max<long long>(1, n_small[2] / (shape.n_sm * 6)));
   std::vector<Part> parts(nparts);
   in_parallel([&](int j) {
     Part& P = parts[j];
@@ -631,8 +650,8 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
           }
           TcItem it{(int)b, r0, tm, c0, tn, (int)P.units.size(), 0, 0, P.scratch};
           double acc = 0;
-          std::vector<SmallTerm> sm[2];  // small-class terms: all blocks <= TC_SMALL_MID, the rest
-          std::vector<int> smb[2];       // their split-block indices (left, right)
+          std::vector<SmallTerm> sm[3];  // terms of the small classes
+          std::vector<int> smb[3];       // their split-block indices (left, right)
           int k = obase;
           const int kend = obase + (t1 - t0);
           while (k < kend) {
@@ -642,9 +661,8 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
             while (e < kend && base[P.order[e]].in_blk == h.in_blk && (base[P.order[e]].flags & 3) == (h.flags & 3)) ++e;
             const TcPsiBlock& ib = plan.psi[h.in_blk];
             // small class: the whole output block (one tile) and the psi block are small
-            const int wmax = std::max(std::max(ob.mL, ob.mR), std::max(ib.m, ib.n));
-            if (wmax <= TC_SMALL_MAX) {
-              const int cls = wmax <= TC_SMALL_MID ? 0 : 1;
+            const int cls = small_class(ob, h.in_blk);
+            if (cls >= 0) {
               for (int q = k; q < e; ++q) {
                 const Base& x = base[P.order[q]];
                 const Task& tk = wl.tasks[x.task];
@@ -681,18 +699,23 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
             P.icost.push_back(acc);
             P.scratch += (long long)tm * tn;
           }
-          for (int cls = 0; cls < 2; ++cls) {  // small-class items: kind 2 (<= TC_SMALL_MID), kind 1
+          constexpr int KIND[3] = {2, 1, 3};
+          for (int cls = 0; cls < 3; ++cls) {
             const size_t base0 = P.small.size();
             P.small.insert(P.small.end(), sm[cls].begin(), sm[cls].end());
             P.small_blk.insert(P.small_blk.end(), smb[cls].begin(), smb[cls].end());
-            for (size_t s0 = base0; s0 < P.small.size(); s0 += small_item[cls]) {
-              const size_t s1 = std::min(P.small.size(), s0 + small_item[cls]);
+            for (size_t s0 = base0, s1 = base0; s0 < P.small.size(); s0 = s1) {
+              s1 = std::min(P.small.size(), s0 + small_item[cls]);
+              if (cls == 2)  // one psi block per item
+                for (s1 = s0 + 1; s1 < P.small.size() && s1 - s0 < (size_t)small_item[cls] &&
+                                  P.small[s1].in_blk == P.small[s0].in_blk;)
+                  ++s1;
               double c = 0;
               for (size_t q = s0; q < s1; ++q) {
                 const PsiBlock& ib = blocks[P.small[q].in_blk];
                 c += 2.0 * ((double)tm * ib.mL * ib.mR + (double)tm * ib.mR * tn);
               }
-              P.items.push_back({(int)b, r0, tm, c0, tn, (int)s0, (int)s1, cls == 0 ? 2 : 1, P.scratch});
+              P.items.push_back({(int)b, r0, tm, c0, tn, (int)s0, (int)s1, KIND[cls], P.scratch});
               P.icost.push_back(c);
               P.scratch += (long long)tm * tn;
             }
@@ -806,17 +829,16 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
   });
   plan.max_tile = largest_tile(plan.groups);
   for (const Part& P : parts) plan.n_units += (long long)P.units.size();
-  std::vector<int> small1;
-  for (size_t i = 0; i < plan.items.size(); ++i) {
-    const int kd = plan.items[i].kind;
-    (kd == 0 ? plan.schedule : kd == 2 ? plan.small_schedule : small1).push_back((int)i);
-  }
   auto by_cost = [&](int a, int b) { return icost[a] > icost[b]; };
-  std::stable_sort(plan.schedule.begin(), plan.schedule.end(), by_cost);
-  std::stable_sort(plan.small_schedule.begin(), plan.small_schedule.end(), by_cost);
-  std::stable_sort(small1.begin(), small1.end(), by_cost);
-  plan.n_small_mid = (int)plan.small_schedule.size();
-  plan.small_schedule.insert(plan.small_schedule.end(), small1.begin(), small1.end());
+  for (int kd : {0, 2, 1, 3}) {
+    std::vector<int>& sched = kd == 0 ? plan.schedule : plan.small_schedule;
+    const size_t first = sched.size();
+    for (size_t i = 0; i < plan.items.size(); ++i)
+      if (plan.items[i].kind == kd) sched.push_back((int)i);
+    std::stable_sort(sched.begin() + first, sched.end(), by_cost);
+    if (kd == 2) plan.n_small_mid = (int)(sched.size() - first);
+    if (kd == 3) plan.n_medium = (int)(sched.size() - first);
+  }
 }
 
 }  // namespace dmrg

@@ -284,8 +284,8 @@ struct TcUnitRec {          // 80-byte header + 16 terms = 464 bytes
 
 // Output tile and its record range; same layout as Item (r_begin/r_end in
 // the place of the task range) so the reduction can read it. kind 0: unit
-// records of the tensor-core kernel; kind 1 / 2: small terms (SmallTerm) of the
-// small-class kernels.
+// records of the tensor-core kernel; kinds 1, 2 and 3: small terms (SmallTerm) of
+// the small-class kernels.
 struct TcItem {
   int out, r0, nrows, c0, ncols, r_begin, r_end, kind;
   long long slot;
@@ -299,6 +299,15 @@ constexpr int TC_SMALL_MAX = 32;
 // Small items whose blocks are all at most TC_SMALL_MID wide (kind 2) run
 // with a smaller footprint than the rest of the small classes (kind 1).
 constexpr int TC_SMALL_MID = 16;
+// Classes whose blocks are all at most TC_MEDIUM_MAX wide (kind 3, one psi block
+// per item) also run with warp-level instructions: a tcgen05 unit costs the
+// tensor-core kernel about 7400 cycles of control and latency whatever its size
+// (1.7 products on average), the warp-level kernel 1400 per product of 33 - 64
+// wide blocks. Per sigma (tensor-core + small kernels): 9.2 + 0.8 -> 5.9 + 2.7 ms at
+// K=108, M=2000 (FP16X2), 6.3 + 0.6 -> 4.5 + 1.8 ms at K=76, M=2000 (BF16X3), 0.70 +
+// 0.38 -> 0.78 ms at K=54, M=1000 (BF16X2). With the line at 48 instead: 7.3 + 1.7,
+// 5.3 + 1.2, 0.23 + 0.64 ms.
+constexpr int TC_MEDIUM_MAX = 64;
 struct SmallTerm {          // 32 bytes
   long long a_tile, b_tile; // first split tile of the left / right stored block, -1 = identity
   int in_blk;               // psi block
@@ -345,8 +354,9 @@ struct TcPlan {
   // identity blocks of the left and right sectors); -1 for unused slots
   std::vector<int> term_blk;
   std::vector<int> small_blk;           // per small term (2k, 2k+1): split-block indices as in term_blk
-  std::vector<int> small_schedule;      // kind-2 items, then kind-1 items, each most expensive first
+  std::vector<int> small_schedule;      // kind-2, kind-1, kind-3 items, each most expensive first
   int n_small_mid = 0;                  // kind-2 items (the head of small_schedule)
+  int n_medium = 0;                     // kind-3 items (its tail)
   long long n_terms = 0;                // term products (tasks x tiles), counted once
   long long n_units = 0;
   double mma_macs = 0;                  // multiply-adds issued per slice product (padding included)
@@ -371,6 +381,7 @@ struct TcShape {
   int want_items;           // items to split the work into (a multiple of the SM count)
   double unit_cost = 128.0 * 128 * 64;  // fixed cost of a unit in the item split, in multiply-adds
   int n_sm = 152;           // SMs that share the small-class items
+  int small_max = TC_SMALL_MAX;  // widest blocks of the small classes (TC_SMALL_MAX or TC_MEDIUM_MAX)
 };
 void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const OpSet& R,
                    const WorkList& wl, TcPlan& plan, const TcShape& shape);

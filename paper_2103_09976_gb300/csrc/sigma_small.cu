@@ -36,6 +36,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "kernels.h"
 
 namespace dmrg {
@@ -357,20 +359,368 @@ void launch_class(const SmallDev& a, int n_items, const int* schedule, unsigned 
   sigma_small_kernel<D, F16><<<grid, 32 * SmallCfg<D, F16>::NW, 0, st>>>(b);
 }
 
+// ------------------------------------------------------------ medium class
+// Blocks of 33 - 64 (TC_MEDIUM_MAX): a term's tile rows are shared by up to four
+// warps (16 rows each) of a CTA of 12 (a multiple of 1, 2, 3 and 4). The blocks
+// of a term are contiguous tile runs, so one bulk copy each brings L and R into
+// a ring slot of the group of warps that works on the term, while the group is
+// busy with the term before; psi (one block per item) stays in shared memory.
+// ldmatrix turns the tiles into fragments, transposing where the operator is
+// used transposed. Arithmetic as the tensor-core kernel's: two slices and three
+// products (fp16, or the first two bf16 slices), or three slices and six
+// products, X split again into as many slices, FP32 sums over a warp's terms of
+// an item, float-float over warps, FP64 over items.
+//
+// Bound by shared-memory reads and the matrix instructions (0.5 per cycle and SM:
+// 1500 cycles for a 64 x 64 product in three products, whose fragments are 140
+// KB of reads), in practice by the instruction latencies of 3 warps per scheduler:
+// the matrix pipe is busy 40% of the time at K=54, M=1000 (0.40 ms per sigma).
+// Fragments loaded from global memory by every warp took 0.75 ms there, a barrier
+// of the group per term and FP64 sums over the warps 0.48 ms.
+constexpr int MED_NT = TC_MEDIUM_MAX / 8, MED_KS = MED_NT / 2, MED_NW = 12;
+constexpr int MED_DEPTH = 4;                       // most ring slots per group
+constexpr uint32_t MED_WAIT = 2000000000u;         // cycles (~1 s) before a wait gives up
+
 template <bool F16>
-void launch_both(const SmallDev& a, int n_sm, cudaStream_t st) {
-  // the schedule lists the <= 16 class first
+struct MedSmem {  // dynamic shared memory
+  static constexpr int TILE = F16 ? 256 : 384;
+  static constexpr int PSI = MED_NT * MED_NT * TILE;  // psi tiles
+  // fragment reads past a block's last tile: at most one tile row or column (odd tile counts), 8 tiles; what they
+  // read is not used or zeroed
+  static constexpr int SLACK = 8 * TILE;
+  static constexpr int RING = (225 * 1024 - PSI - SLACK) / 128 * 128;
+  static constexpr int BYTES = PSI + RING + SLACK;
+  static_assert(RING >= 4 * 2 * PSI, "two slots for two groups of the largest blocks");
+  static_assert(RING >= 12 * 16 * TC_MEDIUM_MAX * 4, "the sums of 12 warps of 16 rows fit the ring");
+};
+
+// four 8x8 fragments; lane l gives the address of row l % 8 of tile l / 8
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+  if constexpr (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+
+template <bool F16, int NPROD>
+__global__ void __launch_bounds__(32 * MED_NW, 1) sigma_medium_kernel(SmallDev a) {
+  constexpr int NT = MED_NT, KS = MED_KS, NU = NPROD == 6 ? 3 : 2, TILE = MedSmem<F16>::TILE;
+  // slice pairs, smallest first
+  auto pa = [](int p) constexpr { return NPROD == 6 ? Pairs<false>::a1(p) : p == 0 ? 1 : 0; };
+  auto pb_ = [](int p) constexpr { return NPROD == 6 ? Pairs<false>::b1(p) : p == 1 ? 1 : 0; };
+  extern __shared__ __align__(128) unsigned char smem[];
+  constexpr int NB = MED_NW * MED_DEPTH;   // (group, slot) pairs
+  __shared__ __align__(8) uint64_t bars[2 * NB + 1];  // slot loaded; slot read (4 arrivals); psi loaded
+  __shared__ uint32_t phase[NB];           // uses of each slot so far, mod 2
+  __shared__ int next;
+  __shared__ volatile int abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t s_psi = (uint32_t)__cvta_generic_to_shared(smem), s_ring = s_psi + MedSmem<F16>::PSI;
+  const uint32_t s_bars = (uint32_t)__cvta_generic_to_shared(bars);
+  float* const part = reinterpret_cast<float*>(smem + MedSmem<F16>::PSI);  // after the terms: the groups' sums
+  const unsigned char* const op = reinterpret_cast<const unsigned char*>(a.op);
+  auto bar = [&](int b) { return s_bars + 8u * (uint32_t)b; };
+  auto expect = [&](int b, uint32_t bytes) {
+    asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(bar(b)), "r"(bytes)
+                 : "memory");
+  };
+  auto bulk = [&](uint32_t dst, const unsigned char* src, int bytes, int b) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar(b))
+                 : "memory");
+  };
+  // bounded; a warp that gives up, or finds that another has, keeps to the barriers below but computes nothing more
+  auto wait = [&](int b, uint32_t parity, bool drain = false) -> bool {
+    uint32_t t0 = 0, ok = 0;
+    for (int n = 0;; ++n) {
+      asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                   : "=r"(ok) : "r"(bar(b)), "r"(parity) : "memory");
+      if (ok) return true;
+      if (abort_flag && !drain) return false;
+      uint32_t t;
+      asm volatile("mov.u32 %0, %%clock;\n" : "=r"(t)::"memory");
+      if (n == 0) t0 = t;
+      if (t - t0 > MED_WAIT) {
+        abort_flag = 1;
+        atomicExch(a.err, 32);
+        return false;
+      }
+    }
+  };
+  if (threadIdx.x <= 2 * NB) {
+    const uint32_t count = threadIdx.x >= NB && threadIdx.x < 2 * NB ? 4 : 1;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar(threadIdx.x)), "r"(count));
+    if (threadIdx.x < NB) phase[threadIdx.x] = 0;
+  }
+  if (threadIdx.x == 0) abort_flag = 0;
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  constexpr int PSI_BAR = 2 * NB;
+  uint32_t psi_phase = 0;
+  for (;;) {
+    if (threadIdx.x == 0) next = (int)atomicAdd(a.counter, 1u);
+    __syncthreads();  // also: the previous item's tile has been read
+    const int qi = next;
+    if (qi >= a.n_items) return;
+    const TcItem it = a.items[a.schedule[qi]];
+    const int tm = it.nrows, tn = it.ncols, tm8 = (tm + 7) >> 3, tn8 = (tn + 7) >> 3;
+    const TcPsiBlock pb = a.pblk[a.terms[it.r_begin].in_blk];
+    const int m8 = (pb.m + 7) >> 3, n8 = (pb.n + 7) >> 3;
+    // groups of n_rows warps, each with `depth` ring slots of one term
+    const int n_rows = (tm + 15) >> 4;
+    const int l_bytes = tm8 * m8 * TILE, r_bytes = tn8 * n8 * TILE;
+    const int slots = MedSmem<F16>::RING / (l_bytes + r_bytes);
+    const int groups = min(MED_NW / n_rows, slots >> 1), depth = min(MED_DEPTH, slots / groups);
+    const int gi = warp / n_rows, i = warp - gi * n_rows, r8 = 2 * i;
+    const bool active = gi < groups, leader = active && i == 0 && lane == 0;
+    const int n_terms = active ? max(0, (it.r_end - it.r_begin - gi + groups - 1) / groups) : 0;
+    if (threadIdx.x == 0) {
+      expect(PSI_BAR, pb.R8 * pb.C8 * TILE);
+      bulk(s_psi, reinterpret_cast<const unsigned char*>(a.psi) + pb.tile * TILE, pb.R8 * pb.C8 * TILE, PSI_BAR);
+    }
+    auto fetch = [&](int k) {  // the group's k-th term into slot k % depth (leader)
+      const SmallTerm* t = a.terms + it.r_begin + gi + k * groups;
+      const int sl = gi * depth + k % depth, b = gi * MED_DEPTH + k % depth;
+      const long long at = t->a_tile, bt = t->b_tile;
+      const uint32_t dst = s_ring + (uint32_t)sl * (uint32_t)(l_bytes + r_bytes);
+      expect(b, (at >= 0 ? l_bytes : 0) + (bt >= 0 ? r_bytes : 0));
+      if (at >= 0) bulk(dst, op + at * TILE, l_bytes, b);
+      if (bt >= 0) bulk(dst + l_bytes, op + bt * TILE, r_bytes, b);
+    };
+    if (leader)
+      for (int k = 0; k < min(depth, n_terms); ++k) fetch(k);
+    bool ok = wait(PSI_BAR, psi_phase);
+    psi_phase ^= 1u;
+    float grp[NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) grp[j][e] = 0.0f;
+    // fragment addresses: lane l names row l % 8 of the tile l / 8 of four
+    const int q = lane >> 3;
+    const uint32_t row = (lane & 7) * 16;
+    const uint32_t psi_lane = s_psi + ((q & 1) * pb.C8 + (q >> 1)) * TILE + row;  // (K tile, N tile)
+    int bslot = 0, before = 0;       // barrier slot of the current term and of the one before
+    uint32_t turn = 0, turn_before = 0;  // rounds of the ring completed then
+    int fetched = min(depth, n_terms);
+    // term k - 1 + depth into the slot of term k - 1 (barrier slot `sl`, after `rounds` rounds), once the group has read
+    // it: in the middle of term k, when the group's other warps are past it
+    auto refill = [&](int k, int sl, uint32_t rounds) {
+      if (leader && k > 0 && k - 1 + depth < n_terms && wait(NB + gi * MED_DEPTH + sl, (phase[gi * MED_DEPTH + sl] + rounds) & 1u)) {
+        fetch(k - 1 + depth);
+        fetched = k + depth;
+      }
+      __syncwarp();
+    };
+    // one term from the ring slot `bslot`; the uses of its operators (transposed or not) as types: the four forms
+    // are separate straight-line code, and an item's terms come in runs of one form
+    auto compute = [&](const SmallTerm& tk, int k, auto TA, auto TB) {
+      constexpr bool tA = decltype(TA)::value, tB = decltype(TB)::value;
+      const bool idL = tk.a_tile < 0, idR = tk.b_tile < 0;
+      const float sc = (float)tk.scale;
+      const uint32_t sl = s_ring + (uint32_t)(gi * depth + bslot) * (uint32_t)(l_bytes + r_bytes), sr = sl + l_bytes;
+      float x[NT][4];
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[j][e] = 0.0f;
+      if (!idL) {  // X = L psi
+        const int lr = (tA ? 1 : m8) * TILE, lk = (tA ? tm8 : 1) * TILE;
+        uint32_t al = sl + min(r8 + (q & 1), tm8 - 1) * lr + (q >> 1) * lk + row;
+        uint32_t ap = psi_lane;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+          if (2 * ks >= m8) break;
+          uint32_t f[NU][4];
+#pragma unroll
+          for (int s = 0; s < NU; ++s) {
+            ldsm4<tA>(f[s], al + 128 * s);
+            if (2 * ks + 1 >= m8) f[s][2] = f[s][3] = 0u;  // past the block
+          }
+#pragma unroll
+          for (int j = 0; j < NT; j += 2) {  // pairs of N tiles; one past the block is cleared below
+            if (j >= n8) break;
+            uint32_t v[NU][4];
+#pragma unroll
+            for (int s = 0; s < NU; ++s) ldsm4<true>(v[s], ap + j * TILE + 128 * s);
+#pragma unroll
+            for (int p = 0; p < NPROD; ++p) {
+              mma16<F16>(x[j], f[pa(p)], v[pb_(p)][0], v[pb_(p)][1]);
+              mma16<F16>(x[j + 1], f[pa(p)], v[pb_(p)][2], v[pb_(p)][3]);
+            }
+          }
+          al += 2 * lk;
+          ap += 2 * pb.C8 * TILE;
+        }
+#pragma unroll
+        for (int j = 1; j < NT; j += 2)
+          if (j == n8) x[j][0] = x[j][1] = x[j][2] = x[j][3] = 0.0f;
+      } else {  // X = psi (the tile's rows and columns)
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (r8 + h < m8 && j < n8) {
+              const unsigned char* t = smem + ((r8 + h) * pb.C8 + j) * TILE + 4 * lane;
+#pragma unroll
+              for (int s = TILE / 128 - 1; s >= 0; --s) {
+                const uint32_t v = *reinterpret_cast<const uint32_t*>(t + 128 * s);
+                if (F16) {
+                  const float2 w = __half22float2(*reinterpret_cast<const __half2*>(&v));
+                  x[j][2 * h] += w.x;
+                  x[j][2 * h + 1] += w.y;
+                } else {
+                  x[j][2 * h] += __uint_as_float(v << 16);
+                  x[j][2 * h + 1] += __uint_as_float(v & 0xFFFF0000u);
+                }
+              }
+            }
+      }
+      refill(k, before, turn_before);
+      if (idR) {
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) grp[j][e] = fmaf(sc, x[j][e], grp[j][e]);
+      } else {
+        // Y = X R^T; fp16: |X| <= 64 * 2^30 of the scaled operands (2^15 with an identity)
+        const float f = F16 && !idL ? 0x1p-21f : 1.0f, finv = F16 && !idL ? 0x1p21f : 1.0f;
+        const int rj = (tB ? 1 : n8) * TILE, rk = (tB ? tn8 : 1) * TILE;
+        float y[NT][4];
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) y[j][e] = 0.0f;
+        uint32_t ar = sr + (q >> 1) * rj + (q & 1) * rk + row;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+          if (2 * ks >= n8) break;
+          uint32_t fx[3][4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            uint32_t s3[3];
+            split_pair<F16>(x[2 * ks + (u >> 1)][2 * (u & 1)] * f, x[2 * ks + (u >> 1)][2 * (u & 1) + 1] * f, s3);
+#pragma unroll
+            for (int s = 0; s < NU; ++s) fx[s][u] = s3[s];
+          }
+#pragma unroll
+          for (int j = 0; j < NT; j += 2) {  // one N tile past the block is computed and never stored
+            if (j >= tn8) break;
+            uint32_t v[NU][4];
+#pragma unroll
+            for (int s = 0; s < NU; ++s) {
+              ldsm4<tB>(v[s], ar + j * rj + 128 * s);
+              if (2 * ks + 1 >= n8) v[s][1] = v[s][3] = 0u;  // past the block
+            }
+#pragma unroll
+            for (int p = 0; p < NPROD; ++p) {
+              mma16<F16>(y[j], fx[pa(p)], v[pb_(p)][0], v[pb_(p)][1]);
+              mma16<F16>(y[j + 1], fx[pa(p)], v[pb_(p)][2], v[pb_(p)][3]);
+            }
+          }
+          ar += 2 * rk;
+        }
+#pragma unroll
+        for (int j = 0; j < NT; ++j)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) grp[j][e] = fmaf(sc, y[j][e] * finv, grp[j][e]);
+      }
+    };
+    SmallTerm nx{};
+    if (n_terms > 0) nx = a.terms[it.r_begin + gi];
+    for (int k = 0; k < n_terms; ++k) {
+      const SmallTerm tk = nx;
+      if (k + 1 < n_terms) nx = a.terms[it.r_begin + gi + (k + 1) * groups];  // in flight during this term
+      const int b = gi * MED_DEPTH + bslot;
+      ok = ok && wait(b, (phase[b] + turn) & 1u);
+      if (!ok) {  // the copy may still be in flight: its leader waits for it (again bounded)
+        if (leader && k < fetched) wait(b, (phase[b] + turn) & 1u, true);
+      } else if (tk.flags & 1) {
+        if (tk.flags & 2) compute(tk, k, std::true_type{}, std::true_type{});
+        else compute(tk, k, std::true_type{}, std::false_type{});
+      } else {
+        if (tk.flags & 2) compute(tk, k, std::false_type{}, std::true_type{});
+        else compute(tk, k, std::false_type{}, std::false_type{});
+      }
+      __syncwarp();
+      if (lane == 0)  // this warp has read the slot (4 arrivals per slot, whatever the number of warps)
+        asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(bar(NB + b)),
+                     "r"(i == 0 ? 5 - n_rows : 1)
+                     : "memory");
+      before = bslot;
+      turn_before = turn;
+      if (++bslot == depth) {
+        bslot = 0;
+        ++turn;
+      }
+    }
+    __syncthreads();  // every slot has been read: the ring becomes the groups' sums
+    if (abort_flag) return;
+    if (leader)
+      for (int d = 0; d < depth; ++d) phase[gi * MED_DEPTH + d] = (phase[gi * MED_DEPTH + d] + (n_terms - d + depth - 1) / depth) & 1u;
+    const int g = lane >> 2, c = lane & 3, n = tm * tn;
+    if (active) {
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int r = 16 * i + g + 8 * (e >> 1), col = 8 * j + 2 * c + (e & 1);
+          if (r < tm && col < tn) part[gi * n + r * tn + col] = grp[j][e];
+        }
+    }
+    __syncthreads();
+    // the groups' sums in order, float-float (an FP64 addition per group would cost as much as several terms)
+    double* out = a.scratch + it.slot;
+    const double ps = F16 ? ldexp(1.0, psi_exponent(*a.psi_exp) - 14) : 1.0;  // undo psi's split scale
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+      float hi = part[e], lo = 0.0f;
+      for (int s = 1; s < groups; ++s) {
+        const float v = part[s * n + e], t = hi + v, z = t - hi;
+        lo += (hi - (t - z)) + (v - z);
+        hi = t;
+      }
+      const double v = (double)hi + (double)lo;
+      out[e] = F16 ? v * ps : v;
+    }
+    // bulk copies overwrite what was written and read here through the generic proxy
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+  }
+}
+
+template <bool F16, int NPROD>
+void launch_medium(const SmallDev& a, int n_items, const int* schedule, unsigned int* counter, int n_sm, cudaStream_t st) {
+  if (n_items <= 0) return;
+  set_max_dynamic_smem((const void*)sigma_medium_kernel<F16, NPROD>, MedSmem<F16>::BYTES);
+  SmallDev b = a;
+  b.schedule = schedule;
+  b.n_items = n_items;
+  b.counter = counter;
+  sigma_medium_kernel<F16, NPROD>
+      <<<n_sm < n_items ? n_sm : n_items, 32 * MED_NW, MedSmem<F16>::BYTES, st>>>(b);
+}
+
+template <bool F16>
+void launch_classes(const SmallDev& a, int n_sm, cudaStream_t st) {
+  // the schedule lists the <= 16 class, the <= 32 class, the <= 64 class
+  const int n32 = a.n_items - a.n_mid - a.n_medium;
   launch_class<16, F16>(a, a.n_mid, a.schedule, a.counter, n_sm, st);
-  launch_class<32, F16>(a, a.n_items - a.n_mid, a.schedule + a.n_mid, a.counter + 1, n_sm, st);
+  launch_class<32, F16>(a, n32, a.schedule + a.n_mid, a.counter + 1, n_sm, st);
+  const int* const med = a.schedule + a.n_mid + n32;
+  if (F16 || a.nprod == 3)
+    launch_medium<F16, 3>(a, a.n_medium, med, a.counter + 2, n_sm, st);
+  else
+    launch_medium<F16, F16 ? 3 : 6>(a, a.n_medium, med, a.counter + 2, n_sm, st);
 }
 
 }  // namespace
 
 void launch_sigma_small(const SmallDev& a, int n_sm, cudaStream_t st) {
   if (a.f16)
-    launch_both<true>(a, n_sm, st);
+    launch_classes<true>(a, n_sm, st);
   else
-    launch_both<false>(a, n_sm, st);
+    launch_classes<false>(a, n_sm, st);
 }
 
 }  // namespace dmrg

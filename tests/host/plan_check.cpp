@@ -5,7 +5,8 @@
 // prints a JSON summary (task count, algorithmic flops, violations) that
 // the Python test compares with the oracle's independent count.
 //
-//   plan_check <sectors file> <nL modes> <n modes> <N> <2Sz> <nc|cn>
+//   plan_check <sectors file> <nL modes> <n modes> <N> <2Sz> <nc|cn> [medium]
+//   medium: the plan with the <= TC_MEDIUM_MAX class, as the library builds it
 //   sectors file: "nl nr" then nl + nr lines "N 2Sz dim"
 #include <algorithm>
 #include <cstdio>
@@ -53,7 +54,9 @@ int main(int argc, char** argv) {
   build_tasks(blocks, oL, oR, terms, wl);
   build_items(blocks, wl, TileShape{32, 256, 2e6, 16384.0}, 152 * 8);
   TcPlan plan;
-  build_tc_plan(blocks, oL, oR, wl, plan, TcShape{152 * 4});
+  TcShape shape{152 * 4};
+  if (argc > 7 && std::string(argv[7]) == "medium") shape.small_max = TC_MEDIUM_MAX;
+  build_tc_plan(blocks, oL, oR, wl, plan, shape);
 
   // (0) FP64 work list: groups tile every output block into 32 x 256 tiles;
   //     the items of a group split the block's task range in order; slots
@@ -165,6 +168,20 @@ int main(int argc, char** argv) {
   for (size_t i = 0; i < plan.items.size(); ++i) {
     const TcItem& it = plan.items[i];
     if (it.r_end <= it.r_begin) fail("item without records or terms");
+    if (it.kind == 3) {
+      // one psi block; some block wider than TC_SMALL_MAX, none than TC_MEDIUM_MAX
+      if (shape.small_max != TC_MEDIUM_MAX) fail("medium item in a plan without them");
+      if (it.r_begin != next_small) fail("medium term ranges");
+      next_small = it.r_end;
+      if (it.r0 != 0 || it.c0 != 0) fail("medium item tile");
+      for (int k = it.r_begin; k < it.r_end && k < (int)plan.small.size(); ++k) {
+        const PsiBlock& ib = blocks[plan.small[k].in_blk];
+        const int w = std::max(std::max(it.nrows, it.ncols), std::max(ib.mL, ib.mR));
+        if (w > TC_MEDIUM_MAX || w <= TC_SMALL_MAX) fail("size class of a medium term");
+        if (plan.small[k].in_blk != plan.small[it.r_begin].in_blk) fail("two psi blocks in a medium item");
+      }
+      continue;
+    }
     if (it.kind == 1 || it.kind == 2) {
       // kind 2: every block at most TC_SMALL_MID wide; kind 1: at most
       // TC_SMALL_MAX, and some block of every term wider than TC_SMALL_MID
@@ -278,8 +295,9 @@ int main(int argc, char** argv) {
   std::vector<int> sch = plan.schedule;
   for (int i : plan.schedule)
     if (plan.items[i].kind != 0) fail("tensor-core schedule holds a small item");
-  for (size_t k = 0; k < plan.small_schedule.size(); ++k)  // kind 2 first, then kind 1
-    if (plan.items[plan.small_schedule[k]].kind != ((int)k < plan.n_small_mid ? 2 : 1))
+  for (size_t k = 0; k < plan.small_schedule.size(); ++k)  // kind 2 first, then kind 1, then kind 3
+    if (plan.items[plan.small_schedule[k]].kind !=
+        ((int)k < plan.n_small_mid ? 2 : k + plan.n_medium < plan.small_schedule.size() ? 1 : 3))
       fail("small schedule: kinds or their order");
   sch.insert(sch.end(), plan.small_schedule.begin(), plan.small_schedule.end());
   std::sort(sch.begin(), sch.end());
@@ -439,11 +457,11 @@ int main(int argc, char** argv) {
   }
   std::printf("{\"psi_size\": %lld, \"blocks\": %zu, \"terms\": %zu, \"tasks\": %zu, \"flops\": %.17g, "
               "\"plan_tasks\": %lld, \"units\": %lld, \"items\": %zu, \"mma_s1\": %lld, \"mma_s2\": %lld, "
-              "\"stages\": %lld, \"op_elements\": %lld, \"f64_request_bytes\": %.17g, "
+              "\"stages\": %lld, \"medium_items\": %d, \"op_elements\": %lld, \"f64_request_bytes\": %.17g, "
               "\"tc_copy_bytes_bf16\": %lld, \"tc_copy_bytes_fp16\": %lld, \"small_read_bytes_bf16\": %lld, "
               "\"small_read_bytes_fp16\": %lld, \"layout\": [",
               size, blocks.size(), terms.size(), wl.tasks.size(), wl.flops, plan.n_terms, plan.n_units,
-              plan.items.size(), mma_s1, mma_s2, stages, (long long)(oL.elements + oR.elements), f64_req,
+              plan.items.size(), mma_s1, mma_s2, stages, plan.n_medium, (long long)(oL.elements + oR.elements), f64_req,
               copy_tiles[0] * 384, copy_tiles[1] * 256, small_tiles * 384, small_tiles * 256);
   for (size_t b = 0; b < blocks.size(); ++b) {
     const PsiBlock& pb = blocks[b];
