@@ -105,6 +105,7 @@ struct SmallDev {
 };
 void launch_sigma_small(const SmallDev& a, int n_sm, cudaStream_t st);
 
+constexpr int PSI_SPLIT_CTAS = 16;  // CTAs that share a psi block in the splits of psi
 void launch_split_ops(const double* store, const SplitJob* jobs, long long njobs, void* out, cudaStream_t st);
 void launch_split_psi(const double* psi, const PsiBlock* blocks, const TcPsiBlock* pb, int nblk, void* out,
                       cudaStream_t st);

@@ -104,7 +104,7 @@ __global__ void split_psi16_kernel(const double* __restrict__ psi, const PsiBloc
     const TcPsiBlock p = pb[b];
     const long long off = blocks[b].off;
     const long long n = (long long)p.R8 * p.C8 * 64;
-    for (long long e = threadIdx.x; e < n; e += blockDim.x) {
+    for (long long e = blockIdx.y * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.y * blockDim.x) {
       const long long t = e >> 6;
       const int w = (int)(e & 63);
       const int i = (int)(t / p.C8) * 8 + (w >> 3), c = (int)(t % p.C8) * 8 + (w & 7);
@@ -190,7 +190,7 @@ void launch_split_psi16(const double* psi, long long n, const PsiBlock* blocks, 
   if (nblk <= 0) return;
   DMRG_CUDA(cudaMemsetAsync(e_psi, 0x80, sizeof(int), st));  // below any exponent: an all-zero psi keeps it
   psi_exp_kernel<<<256, 256, 0, st>>>(psi, n, e_psi);
-  split_psi16_kernel<<<nblk, 256, 0, st>>>(psi, blocks, pb, nblk, e_psi, (__half*)out);
+  split_psi16_kernel<<<dim3(nblk, PSI_SPLIT_CTAS), 256, 0, st>>>(psi, blocks, pb, nblk, e_psi, (__half*)out);
 }
 
 void launch_fix_recs16(const TcUnitRec* in, long long n, const int* term_blk, const int* exps, TcUnitRec* out,
