@@ -99,9 +99,8 @@ typedef struct {
                                   unbounded setting for all three. */
   int tc_producers;            /* tensor-core sigma: warps that fill the kernel's 3-stage operand ring.
                                   1 = one warp fills every stage in order; 3 = warp w fills stage w,
-                                  three stages prepared at once (faster when units hold many K
-                                  stages, i.e. large blocks); 0 = default: 3 when the plan's units
-                                  average 5 or more stages, else 1, until dmrg_autotune picks one.
+                                  three stages prepared at once; 0 = default: 3, until dmrg_autotune
+                                  picks one.
                                   Results are bitwise the same for 1 and 3. */
 } dmrg_opts;
 
@@ -262,8 +261,8 @@ dmrg_status dmrg_sigma_noalloc(dmrg_ctx* ctx, int site, const double* psi, doubl
  * chosen setting; they can differ in the last bits from another setting
  * because items sum their terms in another grouping. A tuned FP64 work list
  * may need more scratch than dmrg_sigma_noalloc holds. Defaults without
- * tuning: FP64 8 items per SM and cost 16384; tensor cores 4 items per SM
- * and unit cost 2^20.
+ * tuning: FP64 8 items per SM and cost 16384; tensor cores 2 to 16 items
+ * per SM by the number of units, and unit cost 2^20.
  */
 dmrg_status dmrg_autotune(dmrg_ctx* ctx, int site, int* items_per_sm, double* per_task_cost, double* best_ms);
 

@@ -132,10 +132,8 @@ static_assert(sizeof(TcItem) == sizeof(Item), "reduction reads TcItem as Item");
 // operator store is unchanged by it).
 static void prepare_tc_plan(Context& c, Problem& p) {
   cudaStream_t st = c.stream;
-  build_tc_plan(p.blocks, p.L, p.R, p.wl, p.tc, 
+  build_tc_plan(p.blocks, p.L, p.R, p.wl, p.tc,
                 TcShape{c.n_sm * p.tc_items_per_sm, p.tc_unit_cost, c.n_sm, TC_MEDIUM_MAX});
-  p.tc_producers[0] = tc_default_producers(p.tc, false);
-  p.tc_producers[1] = tc_default_producers(p.tc, true);
   p.d_tc_recs.upload(p.tc.recs, st);
   p.d_tc_items.upload(p.tc.items, st);
   p.d_tc_small.upload(p.tc.small, st);
@@ -825,7 +823,9 @@ dmrg_status dmrg_get_sigma_info(dmrg_ctx* ctx, int site, dmrg_sigma_info* info) 
     info->op_elements = p.L.elements + p.R.elements;
     info->op_bytes_read = p.wl.bytes_ops;
     info->psi_size = p.psi_size;
-    info->tc_items_per_sm = p.tc_items_per_sm;
+    info->tc_items_per_sm = p.tc_items_per_sm > 0 ? p.tc_items_per_sm
+                            : p.tc_plan_ready      ? std::max(1, p.tc.want_items / ctx->c.n_sm)
+                                                   : 16;
     info->tc_producers = ctx->c.opts.tc_producers > 0 ? ctx->c.opts.tc_producers
                                                        : p.tc_producers[ctx->c.opts.sigma_prec == DMRG_FP16X2 ? 1 : 0];
     info->tc_unit_cost = p.tc_unit_cost;

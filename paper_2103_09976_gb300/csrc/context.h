@@ -164,12 +164,14 @@ struct Problem {
   // FP64 work-list tuning (dmrg_autotune): items per SM and per-task cost term
   int items_per_sm = 8;
   double per_task_cost = 16384.0;
-  // tensor-core plan tuning (dmrg_autotune at a mixed precision): items per SM
-  int tc_items_per_sm = 4;
+  // tensor-core plan tuning (dmrg_autotune at a mixed precision): items per SM, 0 = by the plan's units
+  int tc_items_per_sm = 0;
   double tc_unit_cost = 128.0 * 128 * 64;  // fixed cost of a unit of stacked terms in the item split
-  // producer warps of the tensor-core kernel per tile geometry (bf16, fp16):
-  // the plan's default (tc_default_producers) or the autotuner's choice
-  int tc_producers[2] = {1, 1};
+  // producer warps of the tensor-core kernel per tile geometry (bf16, fp16): the default or the autotuner's
+  // choice. With the kernel's code in one instruction cache three fill the ring faster at every size measured (K=108,
+  // M=2000 FP16X2: 4.6 ms against 5.3 with one; K=76, M=2000 BF16X3: 3.9 against 4.1; K=76, M=4000: 18.7 against 24.0;
+  // sweeps at K=16, M=150: equal)
+  int tc_producers[2] = {3, 3};
   // sub-Hamiltonian parts: (n_ranks, rank) -> work list of that rank's terms
   std::map<std::pair<int, int>, std::unique_ptr<DevWork>> parts;
 };

@@ -110,10 +110,6 @@ void launch_split_ops(const double* store, const SplitJob* jobs, long long njobs
 void launch_split_psi(const double* psi, const PsiBlock* blocks, const TcPsiBlock* pb, int nblk, void* out,
                       cudaStream_t st);
 void launch_sigma_tc(const TcDev& a, int n_sm, cudaStream_t st);
-// Default producer setting of the tensor-core kernel for a plan (TcDev::producers):
-// 3 when its units average 5 or more ring stages of the kernel's geometry
-// (bf16 or fp16 tiles), else 1.
-int tc_default_producers(const TcPlan& plan, bool f16);
 
 // FP16X2 split (split_f16.cu). Operator blocks and psi are scaled by powers
 // of two before the split: block b by 2^(14 - exps[b]), psi by

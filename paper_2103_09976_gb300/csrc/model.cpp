@@ -558,7 +558,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
     return s1 + G * s2;
   };
   const double unit_overhead = shape.unit_cost;  // fixed cost of a unit in the item split
-  double total = 0;
+  double total = 0, n_units = 0;
   // size class of the terms of (output block, psi block): -1 tensor cores, 0 all blocks <= TC_SMALL_MID,
   // 1 <= TC_SMALL_MAX, 2 <= TC_MEDIUM_MAX
   int small_max = shape.small_max;
@@ -591,10 +591,20 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
           if (small_class(ob, base[t].in_blk) >= 0) continue;  // not part of the tensor-core items
           const TcPsiBlock& ib = plan.psi[base[t].in_blk];
           total += unit_macs(1, tn, ib.m, ib.n) / G + unit_overhead / G;
+          n_units += 1.0 / G;
         }
       }
   }
-  const double target = total / std::max(1, shape.want_items);
+  // Items: an even finish wants many per SM, but each costs a partial tile
+  // written and reduced and a start. 16 per SM where they hold 40 units or more,
+  // at least 2. Kernel per sigma with 4 / 8 / 16 / 32 per SM (three producers):
+  // 23.8 / 19.8 / 18.7 / 18.6 ms at K=76, M=4000, 5.6 / 4.7 / 4.6 / 4.6 ms at K=108,
+  // M=2000 (reduction 0.03 / 0.05 / 0.10 / 0.19 ms); solves at K=16, M=150: 313 us per
+  // product with 4, 298 with 2, 301 with 1.
+  plan.want_items = shape.want_items > 0
+                        ? shape.want_items
+                        : (int)std::min(16.0 * shape.n_sm, std::max(2.0 * shape.n_sm, n_units / 40));
+  const double target = total / plan.want_items;
 
   struct Unit {  // one unit: positions [t0, t1) of its part's sorted task order
     int t0, t1;

@@ -357,6 +357,7 @@ struct TcPlan {
   std::vector<int> small_schedule;      // kind-2, kind-1, kind-3 items, each most expensive first
   int n_small_mid = 0;                  // kind-2 items (the head of small_schedule)
   int n_medium = 0;                     // kind-3 items (its tail)
+  int want_items = 0;                   // kind-0 items the split aimed at
   long long n_terms = 0;                // term products (tasks x tiles), counted once
   long long n_units = 0;
   double mma_macs = 0;                  // multiply-adds issued per slice product (padding included)
@@ -378,7 +379,7 @@ inline int tc_per_stage(int nterm, int tn, int n) {
 }
 
 struct TcShape {
-  int want_items;           // items to split the work into (a multiple of the SM count)
+  int want_items;           // items to split the work into (a multiple of the SM count), 0: by the number of units
   double unit_cost = 128.0 * 128 * 64;  // fixed cost of a unit in the item split, in multiply-adds
   int n_sm = 152;           // SMs that share the small-class items
   int small_max = TC_SMALL_MAX;  // widest blocks of the small classes (TC_SMALL_MAX or TC_MEDIUM_MAX)

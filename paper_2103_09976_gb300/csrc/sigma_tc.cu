@@ -217,15 +217,11 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 }
 
 // ------------------------------------------------------ unit geometry
-// (host and device: the host counts ring stages with the same formulas)
-__host__ __device__ __forceinline__ int n_chunks(const TcUnitRec& r) { return (r.n + 127) >> 7; }
-__host__ __device__ __forceinline__ int chunk_cols(const TcUnitRec& r, int j) { return min(128, r.n - 128 * j); }
-__host__ __device__ __forceinline__ int n_halves(const TcUnitRec& r, int j) { return (chunk_cols(r, j) + 63) >> 6; }
-__host__ __device__ __forceinline__ int half_cols(const TcUnitRec& r, int j, int h) { return min(64, chunk_cols(r, j) - 64 * h); }
-template <int KG1>
-__host__ __device__ __forceinline__ int k1_stages(const TcUnitRec& r) { return (r.pR8 + KG1 - 1) / KG1; }
-__host__ __device__ __forceinline__ int tn8e(const TcUnitRec& r) { return 2 * ((r.tn + 15) >> 4); }  // N groups read by the MMA
-__host__ __device__ __forceinline__ int kg2_of(int kw) { return 2 * ((kw + 15) >> 4); }               // K groups of a half
+__device__ __forceinline__ int n_chunks(const TcUnitRec& r) { return (r.n + 127) >> 7; }
+__device__ __forceinline__ int chunk_cols(const TcUnitRec& r, int j) { return min(128, r.n - 128 * j); }
+__device__ __forceinline__ int n_halves(const TcUnitRec& r, int j) { return (chunk_cols(r, j) + 63) >> 6; }
+__device__ __forceinline__ int half_cols(const TcUnitRec& r, int j, int h) { return min(64, chunk_cols(r, j) - 64 * h); }
+__device__ __forceinline__ int kg2_of(int kw) { return 2 * ((kw + 15) >> 4); }               // K groups of a half
 // Shared-memory stride (tile positions) of the right operator of a stage-2
 // stage. With runs (one producer warp), copies_s2 moves a term's tiles as
 // one run where the stored block allows, keeping the block's stride: the
@@ -1120,33 +1116,6 @@ void launch_sigma_tc(const TcDev& a, int n_sm, cudaStream_t st) {
     launch_tc<6, false>(a, grid, st);
   else
     launch_tc<3, false>(a, grid, st);
-}
-
-// Ring stages per unit, counted as the producers fill them. Large blocks
-// give units of many K stages, each a long list of copies: the kernel is then
-// bound by preparing and issuing stages, and three producer warps fill the
-// ring faster; with few stages per unit one producer keeps the stages in
-// the order the MMA issuer takes them, which is faster there.
-template <bool F16>
-static int default_producers(const TcPlan& plan) {
-  using L = Lay<F16>;
-  long long units = 0, stages = 0;
-  for (const TcUnitRec& r : plan.recs) {
-    if (r.flags & TC_ZERO) continue;
-    ++units;
-    for (int j = 0; j < n_chunks(r); ++j) {
-      stages += k1_stages<L::KG1>(r);
-      for (int h = 0; h < n_halves(r, j); ++h) {
-        const int P = max(1, min(r.nterm, L::STAGE_TILES / (tn8e(r) * kg2_of(half_cols(r, j, h)))));
-        stages += (r.nterm + P - 1) / P;
-      }
-    }
-  }
-  return units > 0 && stages >= 5 * units ? NPW : 1;
-}
-
-int tc_default_producers(const TcPlan& plan, bool f16) {
-  return f16 ? default_producers<true>(plan) : default_producers<false>(plan);
 }
 
 }  // namespace dmrg
