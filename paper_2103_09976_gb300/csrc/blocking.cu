@@ -6,6 +6,8 @@
 // dedicated work list (see sweep.cpp).
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "kernels.h"
 
 namespace dmrg {
@@ -319,6 +321,7 @@ __global__ void svd_setup_kernel(const double* __restrict__ psi, const SvdBlock*
                                  double* __restrict__ work, int left) {
   for (int b = blockIdx.y; b < nb; b += gridDim.y) {
     const SvdBlock s = sb[b];
+    if (s.cluster) continue;
     const long long na = (long long)s.d * s.m;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < na; e += (long long)gridDim.x * blockDim.x) {
       const int c = (int)(e / s.m), i = (int)(e % s.m);
@@ -343,6 +346,7 @@ __global__ void svd_norm_kernel(const SvdBlock* __restrict__ sb, int nb, const d
   __shared__ double red[32];
   for (int b = blockIdx.x; b < nb; b += gridDim.x) {
     const SvdBlock s = sb[b];
+    if (s.cluster) continue;
     const long long na = (long long)s.d * s.m;
     double v = 0.0;
     for (long long e = threadIdx.x; e < na; e += blockDim.x) v = fma(work[s.a_off + e], work[s.a_off + e], v);
@@ -365,47 +369,93 @@ __global__ void svd_norm_kernel(const SvdBlock* __restrict__ sb, int nb, const d
 // mutual cosines are rounding noise and would never settle. Sweeps stop when
 // no pair of any block is above its tolerance (at most 30).
 //
-// Bound by the latency of a round (one pair per warp, then a grid barrier),
-// and on this GPU mostly by the FP64 pipe within it: a warp instruction takes
-// about 67 cycles of its SM sub-partition, so the two divisions and three square
-// roots of the rotation, a few dozen instructions each, cost more than the
-// vectors. Hence: the rotation's tangent is computed in FP32 (an angle off
-// by 1e-7 leaves 1e-7 of the product, which later sweeps remove) and only its
-// cosine, which keeps the rotation orthogonal, in FP64 by Newton steps; the
-// squared column norms are carried along (al - t ga, be + t ga; exact to
-// second order in the angle) and recomputed at the start of every sweep; both
-// vectors and their columns of V are loaded once, before the angle is known;
-// every warp keeps its pair's block description for all rounds; and one CTA per
-// SM takes part in the barrier, consecutive pairs on different SMs. Decimations
-// of two sweeps, against three full dot products per pair, a plain FP64
-// rotation and 608 CTAs: 474 -> 112 ms at K=16, M=150 (30 steps), 1771 -> 449 ms
-// at K=24, M=300 (46 steps).
+// On this GPU a round is bound by the FP64 pipe: a warp instruction takes about
+// 67 cycles of its SM sub-partition, whatever the number of warps, so a pair
+// costs what its FP64 instructions cost, one after the other. Hence:
+//  - angle, scaling and the clear cases of the test in FP32, on exponent-shifted
+//    bits (a conversion instruction would go through the same pipe): an angle off
+//    by 1e-7 leaves 1e-7 of the product, which later sweeps remove;
+//  - the rotation is fixed by tau = tan(angle / 2), any FP32 number, and its
+//    sine 2 tau / (1 + tau^2), found in FP64 by Newton's step from an FP32
+//    reciprocal; applied as three shears (x -= tau y, y += s x, x -= tau y), three
+//    instructions per element pair where a rotation by sine and cosine takes four;
+//  - the squared column norms are carried along (al - t ga, be + t ga; exact to
+//    first order in the angle's error) and recomputed at the start of every sweep.
 constexpr int SVD_THREADS = 256;
 constexpr int SVD_REG = 8;         // vectors up to 32 * SVD_REG long stay in registers
 
-// Tangent of the rotation that makes two columns of squared norms al, be and
-// product ga orthogonal (|t| <= 1), to FP32 accuracy.
-__device__ __forceinline__ double jacobi_tangent(double al, double be, double ga) {
-  const double hi = fmax(al, be);
-  const int e = (__double2hiint(hi) >> 20) & 0x7ff;
-  if (e < 64 || e > 1980) {  // 2^-e out of range: plain FP64
-    const double zeta = (be - al) / (2.0 * ga);
-    return (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-  }
-  const double sc = __hiloint2double((2046 - e) << 20, 0);  // brings hi into [1, 2)
-  const float d = (float)((be - al) * sc), g = (float)(ga * sc);
-  const float z = d / (2.0f * g);
-  const float az = fabsf(z);
-  const float t = az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az));
-  return z >= 0.0f ? (double)t : -(double)t;
+// v * 2^-(e - 1023) in FP32 (truncated), e a biased exponent not below that
+// of v by construction; 0 where that is below FP32's range
+__device__ __forceinline__ float scaled_float(double v, int e) {
+  const int h = __double2hiint(v), l = __double2loint(v);
+  const int ef = ((h >> 20) & 0x7ff) - e + 127;
+  const int bits = (h & 0x80000000) | (ef << 23) | ((h & 0xfffff) << 3) | ((unsigned)l >> 29);
+  return ef <= 0 ? 0.0f : __int_as_float(bits);
 }
 
-// 1 / sqrt(u), u in [1, 2], by Newton's iteration from an FP32 start
-__device__ __forceinline__ double newton_rsqrt(double u) {
-  double r = (double)rsqrtf((float)u);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) r = fma(0.5 * r, fma(-u * r, r, 1.0), r);
-  return r;
+// exact (a normal number or zero)
+__device__ __forceinline__ double wide(float v) {
+  const int b = __float_as_int(v), e = (b >> 23) & 0xff;
+  return e == 0 ? 0.0 : __hiloint2double((b & 0x80000000) | ((e + 896) << 20) | ((b & 0x7fffff) >> 3), b << 29);
+}
+
+struct SvdRotation {
+  double tau, s, t;  // tan(angle / 2), sine, tangent (FP32 accuracy, for the norms)
+};
+
+// What the angle needs of the norms alone: ready before the product is
+struct SvdNorms {
+  bool large;    // both squared norms above floor2 (numbers, or NaN)
+  int e;         // biased exponent of the larger
+  float d, lim;  // (be - al) and tol |a_p| |a_q|, over 2^(e - 1023)
+};
+
+__device__ __forceinline__ SvdNorms svd_norms(double al, double be, double floor2, double tol2) {
+  const long long ia = __double_as_longlong(al), ib = __double_as_longlong(be), fl = __double_as_longlong(floor2);
+  SvdNorms n;
+  n.large = ia > fl && ib > fl;
+  n.e = (int)((ia > ib ? ia : ib) >> 52);
+  n.d = scaled_float(be - al, n.e);
+  const float ab = scaled_float(al, n.e) * scaled_float(be, n.e);
+  n.lim = sqrtf((float)tol2) * (ab * rsqrtf(ab));  // ab >= 1e-30 where it is used
+  return n;
+}
+
+// Rotation that makes two columns of squared norms al, be and product ga
+// orthogonal; false when the pair is within its tolerance. Uniform over a warp.
+__device__ __forceinline__ bool svd_angle(const SvdNorms& n, double al, double be, double ga, double tol2,
+                                          SvdRotation& rot) {
+  if (!n.large || (__double_as_longlong(ga) << 1) == 0) return false;
+  const int eg = (__double2hiint(ga) >> 20) & 0x7ff;
+  float t;
+  if (n.e >= 64 && n.e <= 1980 && eg <= n.e + 1) {
+    const float g = scaled_float(ga, n.e), ag = fabsf(g);
+    if (ag < 0.999f * n.lim) return false;
+    if (!(ag > 1.001f * n.lim) && !(ga * ga >= tol2 * (al * be))) return false;
+    const float z = __fdividef(n.d, 2.0f * g);
+    const float az = fabsf(z), q = fmaf(z, z, 1.0f);
+    t = az > 1e8f ? __fdividef(0.5f, az) : __fdividef(1.0f, fmaf(q, rsqrtf(q), az));
+    t = z >= 0.0f ? t : -t;
+  } else {  // outside FP32's reach, or not finite: plain FP64
+    if (!(ga * ga >= tol2 * (al * be))) return false;
+    const double zeta = (be - al) / (2.0 * ga);
+    t = (float)((zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta)));
+  }
+  const float u = fmaf(t, t, 1.0f);
+  const float tau = __fdividef(t, fmaf(u, rsqrtf(u), 1.0f));
+  rot.t = wide(t);
+  rot.tau = wide(tau);
+  // s = 2 tau / w, w = 1 + tau^2: 1 / w = r (1 + e1 + e1^2 + ...), e1 ~ 1e-7
+  const double r = wide(__fdividef(1.0f, fmaf(tau, tau, 1.0f)));
+  const double e1 = fma(-r, fma(rot.tau, rot.tau, 1.0), 1.0), s0 = wide(2.0f * tau) * r;
+  rot.s = fma(s0, fma(e1, e1, e1), s0);
+  return true;
+}
+
+__device__ __forceinline__ void svd_rotate(const SvdRotation& rot, double& x, double& y) {
+  x = fma(-rot.tau, y, x);
+  y = fma(rot.s, x, y);
+  x = fma(-rot.tau, y, x);
 }
 
 // Round `r` of block s, pair i: true when the pair was above its tolerance.
@@ -468,50 +518,295 @@ __device__ bool svd_pair(const SvdBlock& s, int i, int r, bool fresh, double* __
       }
     }
   }
-  ga = warp_sum(ga);
   if (fresh) {
     al = warp_sum(al);
     be = warp_sum(be);
   }
   const double tol2 = fmax(1e-30, 4.930380657631324e-32 * (double)s.m);
-  const bool rotate = ga != 0.0 && al > floor2 && be > floor2 && ga * ga >= tol2 * (al * be);
-  double t = 0.0;
+  const SvdNorms norms = svd_norms(al, be, floor2, tol2);
+  ga = warp_sum(ga);
+  SvdRotation rot;
+  rot.t = 0.0;
+  const bool rotate = svd_angle(norms, al, be, ga, tol2, rot);
   if (rotate) {
-    t = jacobi_tangent(al, be, ga);
-    const double c = newton_rsqrt(fma(t, t, 1.0)), sn = c * t;
     if (in_regs) {
 #pragma unroll
       for (int k = 0; k < SVD_REG; ++k) {
         const int e = lane + 32 * k;
         if (32 * k < s.m && e < s.m) {
-          ap[e] = fma(c, x[k], -sn * y[k]);
-          aq[e] = fma(sn, x[k], c * y[k]);
+          svd_rotate(rot, x[k], y[k]);
+          ap[e] = x[k];
+          aq[e] = y[k];
         }
         if (32 * k < s.d && e < s.d) {
-          vp[e] = fma(c, vx[k], -sn * vy[k]);
-          vq[e] = fma(sn, vx[k], c * vy[k]);
+          svd_rotate(rot, vx[k], vy[k]);
+          vp[e] = vx[k];
+          vq[e] = vy[k];
         }
       }
     } else {
       for (int e = lane; e < s.m; e += 32) {
-        const double u = ap[e], v = aq[e];
-        ap[e] = fma(c, u, -sn * v);
-        aq[e] = fma(sn, u, c * v);
+        double u = ap[e], v = aq[e];
+        svd_rotate(rot, u, v);
+        ap[e] = u;
+        aq[e] = v;
       }
       for (int e = lane; e < s.d; e += 32) {
-        const double u = vp[e], v = vq[e];
-        vp[e] = fma(c, u, -sn * v);
-        vq[e] = fma(sn, u, c * v);
+        double u = vp[e], v = vq[e];
+        svd_rotate(rot, u, v);
+        vp[e] = u;
+        vq[e] = v;
       }
     }
   }
   if (lane == 0 && (rotate || fresh)) {
-    nrm[s.q_off + p] = fma(-t, ga, al);
-    nrm[s.q_off + q] = fma(t, ga, be);
+    nrm[s.q_off + p] = fma(-rot.t, ga, al);
+    nrm[s.q_off + q] = fma(rot.t, ga, be);
   }
   return rotate;
 }
 
+// Wait for a phase of an mbarrier, at most about a second; false: it did not come.
+__device__ __forceinline__ bool svd_wait(unsigned bar, unsigned parity) {
+  for (int k = 0; k < (1 << 20); ++k) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 1000;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+__device__ __forceinline__ unsigned cluster_addr(const void* p, int rank) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  unsigned r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+
+// v to a shared-memory address of the cluster, its 8 bytes counted by the mbarrier beside it
+__device__ __forceinline__ void svd_send(unsigned addr, double v, unsigned bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(addr),
+               "l"(__double_as_longlong(v)), "r"(bar)
+               : "memory");
+}
+
+// Both columns of a warp's buffer are awaited: 2 ld doubles
+__device__ __forceinline__ void svd_arm(unsigned bar, int ld) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(2 * ld * 8) : "memory");
+}
+
+// Blocks that fit: one cluster each. Warp w of CTA k holds the pair
+// k * ppc + w, its two columns (A, V and squared norm) in the CTA's shared
+// memory, and after a round sends them where the next round's pairs want
+// them, in its own CTA or a neighbour's, into the other of two buffers: a pair
+// waits for its two columns and for nothing else. Clusters of 16 CTAs (the most
+// there is), so that up to 64 pairs have an SM sub-partition each: 2.1 ms a
+// decimation against 2.6 with 8 (K=16, M=150, an earlier form). Bound by the latency of
+// a round, a chain of some 25 FP64 instructions, the FP32 angle and the way of
+// the columns. C: 32-element chunks of the longer of A's and V's
+// columns; what lies past the shorter's end is skipped by branches that
+// the compiler is kept from turning into selects (all the instructions
+// would go through the FP64 pipe: 4200 of a round's 9000 cycles).
+// One 96 x 96 block takes 1.9 us a round, 4.9 on the grid-wide kernel (columns
+// through L2, a grid barrier a round, every block waiting for the largest);
+// 26 blocks of up to 96 2.8 ms against 6.7, up to 200 16.6 against 30.4, 80 of
+// up to 250 93 against 109. Decimations of two sweeps: 113 -> 35 ms at K=16,
+// M=150 (30 steps), 447 -> 222 at K=24, M=300 (46 steps).
+template <int C>
+__device__ __forceinline__ void svd_cluster_block(const SvdBlock& s, const double* __restrict__ psi,
+                                                  double* __restrict__ work, int left, double* cols, double* part,
+                                                  unsigned int* above, unsigned long long* full) {
+  namespace cgp = cooperative_groups;
+  cgp::cluster_group cluster = cgp::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int ppc = (s.npairs + SVD_CLUSTER - 1) / SVD_CLUSTER;
+  const int pair = rank * ppc + wid;
+  const bool active = wid < ppc && pair < s.npairs;
+  const int m = s.m, d = s.d, dp = d + (d & 1), ld = m + d + 1;
+  const int px = pair, py = dp - 1 - pair;  // positions of the pair; the next round finds position x at x - 1, 1 at dp - 1
+  double *cx = cols + wid * 4 * ld, *cy = cx + ld;  // buffer 1: 2 ld doubles on
+  const unsigned my_full = (unsigned)__cvta_generic_to_shared(full + 2 * wid);  // buffer 1: 8 bytes on
+  unsigned tx = 0, ty = 0, tx_full = 0, ty_full = 0;  // where the columns go, and the mbarriers there (of buffer 0)
+  if (active) {
+    auto home = [&](int x, unsigned& col, unsigned& bar) {
+      const int pr = x < s.npairs ? x : dp - 1 - x, w = pr % ppc, k = pr / ppc;
+      col = cluster_addr(cols + (w * 4 + (x < s.npairs ? 0 : 1)) * ld, k);
+      bar = cluster_addr(full + 2 * w, k);
+    };
+    home(px == 0 ? 0 : px == 1 ? dp - 1 : px - 1, tx, tx_full);
+    home(py == 1 ? dp - 1 : py - 1, ty, ty_full);
+    if (lane == 0)
+      for (int b = 0; b < 2; ++b) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(my_full + 8 * b) : "memory");
+        svd_arm(my_full + 8 * b, ld);
+      }
+    double nn = 0.0;
+    for (int h = 0; h < 2; ++h) {
+      double* c = h ? cy : cx;
+      const int col = h ? py : px;  // a column past d: zero
+      for (int e = lane; e < m; e += 32) {
+        const double v = col >= d ? 0.0
+                         : left   ? psi[s.psi_off + (long long)col * m + e]
+                                  : psi[s.psi_off + (long long)e * d + col];
+        c[e] = v;
+        nn = fma(v, v, nn);
+      }
+      for (int e = lane; e < d; e += 32) c[m + e] = e == col ? 1.0 : 0.0;
+    }
+    nn = warp_sum(nn);
+    if (lane == 0) part[wid] = nn;
+  }
+  if (threadIdx.x < 3) above[threadIdx.x] = 0u;
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  cluster.sync();
+  double floor2 = 0.0;  // 1e-30 |A|_F^2
+  for (int pr = lane; pr < s.npairs; pr += 32) floor2 += *cluster.map_shared_rank(part + pr % ppc, pr / ppc);
+  floor2 = 1e-30 * warp_sum(floor2);
+  const double tol2 = fmax(1e-30, 4.930380657631324e-32 * (double)m);
+  unsigned int* flags = cluster.map_shared_rank(above, 0);
+  // Columns of round g (counted over all sweeps) lie in buffer g & 1. A neighbour
+  // writes a buffer again only after it has the columns sent from it, so
+  // the two buffers need no other guard.
+  unsigned g = 0;
+  bool lost = false;  // a wait ran out: no more waits, the caller sees an error
+  auto arrived = [&]() {
+    if (g == 0) return;
+    const unsigned bar = my_full + 8 * (g & 1);
+    if (!lost) lost = !svd_wait(bar, ((g - 1) >> 1) & 1);
+    if (lane == 0) svd_arm(bar, ld);  // for round g + 2
+  };
+  for (int sweep = 0; sweep < 30; ++sweep) {
+    bool any = false;
+    for (int r = 0; r < s.rounds; ++r, ++g) {
+      if (!active) continue;
+      arrived();
+      const int from = (g & 1) * 2 * ld, to = 2 * ld - from;
+      const double *bx = cx + from, *by = cy + from;
+      double x[C], y[C], vx[C], vy[C];
+      double al = bx[ld - 1], be = by[ld - 1], ga = 0.0;
+#pragma unroll
+      for (int k = 0; k < C; ++k) {
+        const int e = lane + 32 * k;
+        x[k] = y[k] = vx[k] = vy[k] = 0.0;
+        if (e < m) {
+          x[k] = bx[e];
+          y[k] = by[e];
+        }
+        if (e < d) {
+          vx[k] = bx[m + e];
+          vy[k] = by[m + e];
+        }
+      }
+      if (r == 0) {
+        al = be = 0.0;
+#pragma unroll
+        for (int k = 0; k < C; ++k)
+          if (32 * k < m) {
+            asm volatile("" ::: "memory");
+            al = fma(x[k], x[k], al);
+            be = fma(y[k], y[k], be);
+          }
+        al = warp_sum(al);
+        be = warp_sum(be);
+      }
+      const SvdNorms norms = svd_norms(al, be, floor2, tol2);
+#pragma unroll
+      for (int k = 0; k < C; ++k)
+        if (32 * k < m) {
+          asm volatile("" ::: "memory");
+          ga = fma(x[k], y[k], ga);
+        }
+      ga = warp_sum(ga);
+      SvdRotation rot;
+      if (svd_angle(norms, al, be, ga, tol2, rot)) {  // never with a column past d: its norm is 0
+        any = true;
+#pragma unroll
+        for (int k = 0; k < C; ++k) {
+          if (32 * k < m) {
+            asm volatile("" ::: "memory");
+            svd_rotate(rot, x[k], y[k]);
+          }
+          if (32 * k < d) {
+            asm volatile("" ::: "memory");
+            svd_rotate(rot, vx[k], vy[k]);
+          }
+        }
+        al = fma(-rot.t, ga, al);
+        be = fma(rot.t, ga, be);
+      }
+      const unsigned ox = tx + 8 * to, oy = ty + 8 * to, fx = tx_full + 8 * (~g & 1), fy = ty_full + 8 * (~g & 1);
+#pragma unroll
+      for (int k = 0; k < C; ++k) {
+        const int e = lane + 32 * k;
+        if (e < m) {
+          svd_send(ox + 8 * e, x[k], fx);
+          svd_send(oy + 8 * e, y[k], fy);
+        }
+        if (e < d) {
+          svd_send(ox + 8 * (m + e), vx[k], fx);
+          svd_send(oy + 8 * (m + e), vy[k], fy);
+        }
+      }
+      if (lane == 0) {
+        svd_send(ox + 8 * (ld - 1), al, fx);
+        svd_send(oy + 8 * (ld - 1), be, fy);
+      }
+    }
+    lost = __any_sync(0xffffffffu, lost);
+    // above[sweep % 3] of CTA 0, as in the grid-wide kernel; bit 1: give up
+    if (lane == 0 && (any || lost)) atomicOr(flags + sweep % 3, lost ? 2u : 1u);
+    cluster.sync();
+    const unsigned int more = *(volatile unsigned int*)(flags + sweep % 3);
+    if (rank == 0 && threadIdx.x == 0) above[(sweep + 2) % 3] = 0u;
+    if (more & 2u) lost = true;
+    if (more != 1u) break;
+  }
+  if (active) arrived();
+  if (lost) {
+    atomicOr(reinterpret_cast<unsigned int*>(work) + SVD_LOST, 1u);
+    __nanosleep(100000);  // columns that nobody awaits any more may still be on their way
+  }
+  cluster.sync();  // no CTA leaves while its flags or columns are in use
+  if (active)      // a whole number of cycles: every column is back at its first position
+    for (int h = 0; h < 2; ++h) {
+      const double* c = (h ? cy : cx) + (g & 1) * 2 * ld;
+      const int col = h ? py : px;
+      if (col >= d) continue;
+      for (int e = lane; e < m; e += 32) work[s.a_off + (long long)col * m + e] = c[e];
+      for (int e = lane; e < d; e += 32) work[s.v_off + (long long)col * d + e] = c[m + e];
+    }
+}
+
+__global__ void __launch_bounds__(32 * SVD_CLUSTER_WARPS, 1)
+svd_cluster_kernel(const SvdBlock* __restrict__ sb, const double* __restrict__ psi, double* __restrict__ work, int left) {
+  extern __shared__ double svd_cols[];
+  __shared__ double part[SVD_CLUSTER_WARPS];
+  __shared__ unsigned int above[3];
+  __shared__ unsigned long long full[2 * SVD_CLUSTER_WARPS];  // mbarriers: the columns of a warp's buffers
+  const SvdBlock s = sb[sb[blockIdx.x / SVD_CLUSTER].order];
+  auto run = [&](auto c) { svd_cluster_block<decltype(c)::value>(s, psi, work, left, svd_cols, part, above, full); };
+  const int chunks = ((s.m > s.d ? s.m : s.d) + 31) / 32;
+  if (chunks <= 1)
+    run(std::integral_constant<int, 1>());
+  else if (chunks <= 2)
+    run(std::integral_constant<int, 2>());
+  else if (chunks <= 3)
+    run(std::integral_constant<int, 3>());
+  else if (chunks <= 4)
+    run(std::integral_constant<int, 4>());
+  else
+    run(std::integral_constant<int, SVD_REG>());
+}
+
+// The other blocks: columns in global memory, one pair per warp over the whole
+// grid, one CTA per SM in the barrier and consecutive pairs on different SMs.
 __global__ void __launch_bounds__(SVD_THREADS, 1)
 svd_jacobi_kernel(const SvdBlock* __restrict__ sb, int nb, int total_pairs, int max_rounds, double* __restrict__ work,
                   double* __restrict__ nrm, const double* __restrict__ fro, unsigned int* __restrict__ above) {
@@ -614,18 +909,41 @@ void launch_take_columns(const double* Q, const TakeBlock* tb, int nb, double* d
 
 namespace dmrg {
 
-void launch_svd_blocks(const double* psi, const SvdBlock* sb, int nb, int total_pairs, int max_rounds, int max_d_hint,
-                       double* Q, double* w, double* work, bool left, int n_sm, cudaStream_t st) {
+bool svd_cluster_fits(int d, int m) {
+  const int npairs = (d + 1) / 2, ppc = (npairs + SVD_CLUSTER - 1) / SVD_CLUSTER;
+  return d >= 1 && d <= 32 * SVD_REG && m <= 32 * SVD_REG && ppc <= SVD_CLUSTER_WARPS &&
+         (size_t)ppc * 4 * (m + d + 1) * sizeof(double) <= SVD_CLUSTER_SMEM;
+}
+
+void launch_svd_blocks(const double* psi, const SvdBlock* sb, const SvdShape& shape, double* Q, double* w, double* work,
+                       bool left, int n_sm, cudaStream_t st) {
+  int nb = shape.nb, total_pairs = shape.grid_pairs, max_rounds = shape.grid_rounds;
   if (nb <= 0) return;
-  if ((size_t)max_d_hint * sizeof(double) > 48 * 1024)
-    set_max_dynamic_smem((const void*)svd_finish_kernel, (int)((size_t)max_d_hint * sizeof(double)));
-  {
-    dim3 grid(32, nb < 65535 ? nb : 65535);
-    svd_setup_kernel<<<grid, 256, 0, st>>>(psi, sb, nb, work, left ? 1 : 0);
+  const size_t sig_bytes = (size_t)shape.max_d * sizeof(double);
+  if (sig_bytes > 48 * 1024) set_max_dynamic_smem((const void*)svd_finish_kernel, (int)sig_bytes);
+  if (cudaMemsetAsync(work, 0, 64, st) != cudaSuccess) return;  // the flags of both kernels; the caller's cudaGetLastError reports it
+  if (shape.n_cluster > 0) {
+    set_max_dynamic_smem((const void*)svd_cluster_kernel, (int)SVD_CLUSTER_SMEM);
+    if (cudaFuncSetAttribute((const void*)svd_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+        cudaSuccess)
+      return;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)shape.n_cluster * SVD_CLUSTER);
+    cfg.blockDim = dim3(32u * shape.cluster_warps);
+    cfg.dynamicSmemBytes = shape.cluster_smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = SVD_CLUSTER;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, svd_cluster_kernel, sb, psi, work, left ? 1 : 0) != cudaSuccess) return;
   }
   if (total_pairs > 0 && max_rounds > 0) {
+    dim3 grid(32, nb < 65535 ? nb : 65535);
+    svd_setup_kernel<<<grid, 256, 0, st>>>(psi, sb, nb, work, left ? 1 : 0);
     unsigned int* above = reinterpret_cast<unsigned int*>(work);  // first words of work
-    cudaMemsetAsync(above, 0, 4 * sizeof(unsigned int), st);
     svd_norm_kernel<<<nb < 65535 ? nb : 65535, 256, 0, st>>>(sb, nb, work, w);
     const double* fro = w;
     double* nrm = Q;  // Q is written by the finish kernel: until then the squared column norms, d per block
@@ -634,7 +952,7 @@ void launch_svd_blocks(const double* psi, const SvdBlock* sb, int nb, int total_
     const cudaError_t e = cudaLaunchCooperativeKernel((void*)svd_jacobi_kernel, dim3(n_sm), dim3(SVD_THREADS), args, 0, st);
     if (e != cudaSuccess) return;  // the caller's cudaGetLastError reports it
   }
-  svd_finish_kernel<<<nb < 65535 ? nb : 65535, 256, (size_t)max_d_hint * sizeof(double), st>>>(sb, nb, work, Q, w);
+  svd_finish_kernel<<<nb < 65535 ? nb : 65535, 256, sig_bytes, st>>>(sb, nb, work, Q, w);
 }
 
 }  // namespace dmrg

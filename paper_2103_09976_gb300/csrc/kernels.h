@@ -197,10 +197,23 @@ void launch_opcomb(const double* src, const long long* xoff, const double* coef,
 // v_off. max_d_hint >= every d (shared memory of the final sort).
 struct SvdBlock {
   long long psi_off, q_off, w_off, a_off, v_off;
-  int d, m, pair0, npairs, rounds, pad;
+  int d, m, pair0, npairs, rounds;
+  int cluster;  // 1: one cluster of CTAs takes the block (svd_cluster_fits), 0: the grid-wide kernel
+  int order;    // of entry i: the i-th block of the cluster kernel, largest first
+  int pad;
 };
-void launch_svd_blocks(const double* psi, const SvdBlock* sb, int nb, int total_pairs, int max_rounds, int max_d_hint,
-                       double* Q, double* w, double* work, bool left, int n_sm, cudaStream_t st);
+constexpr int SVD_CLUSTER = 16;                   // CTAs of a cluster
+constexpr int SVD_CLUSTER_WARPS = 16;             // most warps, one pair each, of a CTA
+constexpr size_t SVD_CLUSTER_SMEM = 220 * 1024;   // most shared memory of a CTA
+constexpr int SVD_LOST = 8;  // 32-bit word of the work area: not zero when a wait of the cluster kernel ran out
+bool svd_cluster_fits(int d, int m);
+struct SvdShape {
+  int nb = 0, max_d = 1;
+  int grid_pairs = 0, grid_rounds = 0;                    // of the grid-wide kernel's blocks
+  int n_cluster = 0, cluster_warps = 1, cluster_smem = 0;  // blocks, warps and shared memory of a CTA
+};
+void launch_svd_blocks(const double* psi, const SvdBlock* sb, const SvdShape& shape, double* Q, double* w, double* work,
+                       bool left, int n_sm, cudaStream_t st);
 void launch_orthonormalize(double* store, const GramBlock* gb, int nb, cudaStream_t st);
 void launch_take_columns(const double* Q, const TakeBlock* tb, int nb, double* dst, cudaStream_t st);
 

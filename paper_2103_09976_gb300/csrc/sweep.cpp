@@ -386,20 +386,33 @@ void decimate(Context& c, Problem& p, const Enlarged& E, const double* psi, int 
   std::vector<GramBlock> gb(nb);   // Q / w offsets and the two dimensions of every block
   std::vector<SvdBlock> sb(nb);
   long long goff = 0, woff = 0, aoff = 64;
-  int pairs = 0, max_rounds = 0, max_d = 1;
+  SvdShape shape;
+  shape.nb = nb;
+  std::vector<int> cl;  // blocks of the cluster kernel
   for (int b = 0; b < nb; ++b) {
     const PsiBlock& pb = p.blocks[b];
     const int d = forward ? pb.mL : pb.mR, m = forward ? pb.mR : pb.mL;
     gb[b] = {pb.off, goff, woff, d, m};
     const int dp = d + (d & 1);
-    sb[b] = {pb.off, goff, woff, aoff, aoff + (long long)d * m, d, m, pairs, dp / 2, dp - 1, 0};
-    pairs += dp / 2;
-    max_rounds = std::max(max_rounds, dp - 1);
-    max_d = std::max(max_d, d);
+    const bool fits = svd_cluster_fits(d, m);
+    sb[b] = {pb.off, goff, woff, aoff, aoff + (long long)d * m, d, m, shape.grid_pairs, dp / 2, dp - 1, fits ? 1 : 0, 0, 0};
+    if (fits) {
+      const int ppc = (dp / 2 + SVD_CLUSTER - 1) / SVD_CLUSTER;
+      shape.cluster_warps = std::max(shape.cluster_warps, ppc);
+      shape.cluster_smem = std::max(shape.cluster_smem, (int)(ppc * 4 * (m + d + 1) * sizeof(double)));
+      cl.push_back(b);
+    } else {
+      shape.grid_pairs += dp / 2;
+      shape.grid_rounds = std::max(shape.grid_rounds, dp - 1);
+    }
+    shape.max_d = std::max(shape.max_d, d);
     aoff += (long long)d * m + (long long)d * d;
     goff += (long long)d * d;
     woff += d;
   }
+  std::stable_sort(cl.begin(), cl.end(), [&](int a, int b) { return sb[a].d > sb[b].d; });
+  for (size_t i = 0; i < cl.size(); ++i) sb[i].order = cl[i];
+  shape.n_cluster = (int)cl.size();
   DevBuf dsb, Q, W, work;
   dsb.upload(sb, st);
   Q.alloc(std::max<long long>(1, goff) * sizeof(double));
@@ -407,13 +420,16 @@ void decimate(Context& c, Problem& p, const Enlarged& E, const double* psi, int 
   work.alloc((size_t)aoff * sizeof(double));
   {
     ProfScope ps(c.prof, 3, st);
-    launch_svd_blocks(psi, dsb.as<SvdBlock>(), nb, pairs, max_rounds, max_d, Q.as<double>(), W.as<double>(),
-                      work.as<double>(), forward, c.n_sm, st);
+    launch_svd_blocks(psi, dsb.as<SvdBlock>(), shape, Q.as<double>(), W.as<double>(), work.as<double>(), forward,
+                      c.n_sm, st);
   }
   DMRG_CUDA(cudaGetLastError());
   std::vector<double> w(woff);
+  unsigned int flags[16] = {};
   DMRG_CUDA(cudaMemcpyAsync(w.data(), W.p, woff * sizeof(double), cudaMemcpyDeviceToHost, st));
+  DMRG_CUDA(cudaMemcpyAsync(flags, work.p, sizeof(flags), cudaMemcpyDeviceToHost, st));
   DMRG_CUDA(cudaStreamSynchronize(st));
+  if (flags[SVD_LOST]) throw Error(DMRG_ECUDA, "decimation: a wait of the SVD kernel ran out");
   std::vector<std::vector<double>> sv(nb);  // singular values per block, descending
   std::vector<QN> qLs(nb);
   for (int b = 0; b < nb; ++b) {
