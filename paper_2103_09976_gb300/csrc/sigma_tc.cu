@@ -42,13 +42,14 @@
 //
 // The kernel is bound by its serial instruction streams (the MMA-issuing warp
 // spends a third of its time on MMAs, a seventh waiting, the rest on the control
-// code around them; MMAs at rate would take 2 of the 9.1 ms at K=108, M=2000), and
+// code around them), and
 // the warps of all roles share one instruction cache. So every role's work has
 // one call site, quotients come from the records or small cases instead of
 // divisions, and a chain and its commits are issued in one elected region: 59 KB
-// of code instead of 74 (one producer) and 86 KB (three). Per sigma, before ->
-// after: 29.1 -> 24.4 ms at K=76, M=4000 (three producers, FP16X2), 11.7 -> 9.1 ms
-// for three producers at K=108, M=2000, where one producer stays at 9.2 ms.
+// of code instead of 74 (one producer) and 86 KB (three): 29.1 -> 24.4 ms a launch
+// at K=76, M=4000 (FP16X2, three producers). With 16 items per SM 18.9 ms there
+// (24.2 with one producer), and 4.6 ms at K=108, M=2000 (5.3), where blocks
+// of 33-64 columns go to their own class.
 //
 // Every wait on an mbarrier is bounded (about one second of clock); on a
 // timeout the kernel raises a flag in *err, stops issuing work, waits (again
@@ -657,8 +658,8 @@ __global__ void __launch_bounds__(NTHR, 1) sigma_tc_kernel(TcDev a) {
     // commits, lane 0 the plain arrivals.
     {
       const bool leader = lane == 0;
-      // with profiling on, slots 14 / 15 of the wait accounting receive the
-      // cycles this warp spends issuing MMAs / committing them
+      // with profiling on, slot 14 of the wait accounting receives the cycles
+      // this warp spends issuing MMAs and their commits
       constexpr bool prof = PROF;
       auto tick = [&]() -> long long { return prof ? clock64() : 0ll; };
       auto tock = [&](int slot, long long t0) {
