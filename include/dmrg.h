@@ -64,7 +64,8 @@ typedef enum {
  * accumulation bounded as for BF16X3; the scales are exact and undone in
  * the coefficients and the flushes. Classes whose blocks are all at most 32
  * wide run with warp-level matrix instructions from the same split in every
- * mixed mode, with FP32 accumulation of all products above 2^-24 relative. */
+ * mixed mode (BF16X2 included, all three slices), with the slice products down
+ * to 2^-24 and FP32 sums: the error of FP32 arithmetic on the split operands. */
 typedef enum { DMRG_FP64 = 0, DMRG_BF16X2 = 1, DMRG_BF16X3 = 2, DMRG_FP16X2 = 3 } dmrg_prec;
 
 typedef struct {

@@ -16,14 +16,15 @@
 // The accumulators of X = L psi have the layout of the second product's left
 // fragments, so X only has to be split again.
 //
-// Arithmetic: FP32 accumulation of slice products. The fp16 split (hi + lo)
-// takes all four products in the first product, and X as three fp16 slices (at
-// least 30 bits; scaled by 2^-20 so that it stays in range) in the second; the
-// bf16 split (hi + mid + lo) takes the six products above 2^-24 in both, X as
-// three bf16 slices. That is the accuracy of FP32 multiply-adds on the summed
-// slices, which this kernel used before (measured below). Terms of a warp are
-// summed in FP32 over groups of 8, groups in float-float (48 bits), warps in
-// FP64 in warp order, so the result does not depend on scheduling.
+// Arithmetic: FP32 accumulation of slice products, the error of FP32 multiply-adds
+// on the summed slices or less (mma_step). The fp16 split (hi + lo) takes all four
+// products in the first product and, with X as three fp16 slices, five in the second
+// (lo x the third slice, below 2^-33, is left out); every row of X is scaled so that
+// its largest element fills the range of fp16 (row_scale). The bf16 split (hi + mid +
+// lo) takes the six products above 2^-24 in both, X as three bf16 slices; what is left
+// out is below 2^-25. Terms of a warp are summed in FP32 over groups of 8, groups in
+// float-float (48 bits), warps in FP64 in warp order, so the result does not depend on
+// scheduling.
 //
 // Bound by instruction issue (<= 16: 65% of issue slots) and load latency (<= 32:
 // 12-16 warps per SM of 128-159 registers); a term of 16 x 16 blocks reads 2-3 KB
@@ -31,8 +32,8 @@
 // shared by two), CTAs are 4 warps, items come from a counter, the next term's
 // record is loaded a term ahead and its L and R before psi and the first product.
 // Both kernels per sigma, against FP32 multiply-adds from shared memory: 1.63 ->
-// 0.82 ms at K=108, M=2000 (FP16X2), 0.74 -> 0.38 ms at K=54, M=1000 (BF16X2), 63
-// -> 41 us at K=24, M=250; error of sigma against 64 bits 1.3e-7 -> 1.2e-7 there.
+// 0.96 ms at K=108, M=2000 (FP16X2), 0.74 -> 0.40 ms at K=54, M=1000 (BF16X2), 63
+// -> 46 us at K=24, M=250.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -106,7 +107,7 @@ __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t (&s)[3])
   }
 }
 
-// Slice pairs (A slice, B slice) of the two products, smallest first.
+// Slice pairs (A slice, B slice) of the two products, smallest first (the last pair is hi x hi).
 template <bool F16>
 struct Pairs;
 template <>
@@ -126,6 +127,57 @@ struct Pairs<false> {  // hl, mm, lh, hm, mh, hh
   __device__ static constexpr int b2(int p) { return b1(p); }
 };
 
+// x[j] += a b[j] for the N tiles j < nj of one K step (x[j] = a b[j] when `first`);
+// b(j, h, s): slice s of K tile h. The matrix instruction adds with truncation
+// (measured: operands aligned to the largest exponent with two extra bits, the
+// result cut to 24), so a sum left to it shrinks by up to a unit in the last place
+// an instruction, always in one direction. Hence hi x hi of every K step goes to a
+// fresh accumulator z, the other products to c, and FP32 additions, which round to
+// nearest, join them. REST: c starts with hi x hi on top of -z, which gives what was
+// cut off (to a quarter unit); the <= 16 class needs it, where FP32 multiply-adds
+// round a few times only. Relative error of sigma against 64 bits (2-norm, 1e-7), one
+// accumulator / these parts / FP32 multiply-adds of the summed slices: bf16 slices
+// 1.0 / 0.7 / 0.9 at K=8, M=60 (blocks up to 4 wide), 1.0 / 0.7 / 1.0 at K=24, M=200 (10),
+// 3.3 / 0.8 / 1.4 at K=36, M=500 (25); fp16 1.3 / 1.0 / 1.0, 1.2 / 0.9 / 1.2, 2.5 / 1.3 / 1.5.
+// Time of a sigma: 706 -> 734 us at K=54, M=1000 (BF16X2), 7.17 -> 7.29 ms at K=108, M=2000
+// (FP16X2); taking the N tiles one after another keeps z and c in registers.
+template <bool F16, bool SECOND, bool REST, int NT, int NSA, class Frag>
+__device__ __forceinline__ void mma_step(float (&x)[NT][4], bool first, int nj, const uint32_t (&a)[NSA][4],
+                                         Frag&& b) {
+  using P = Pairs<F16>;
+  constexpr int NP = SECOND ? P::N2 : P::N1;
+#pragma unroll
+  for (int j = 0; j < NT; ++j)
+    if (j == 0 || j < nj) {
+      float z[4] = {0.0f, 0.0f, 0.0f, 0.0f}, c[4];
+      mma16<F16>(z, a[0], b(j, 0, 0), b(j, 1, 0));
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        c[e] = REST ? -z[e] : 0.0f;
+        x[j][e] = first ? z[e] : x[j][e] + z[e];
+      }
+      if (REST) mma16<F16>(c, a[0], b(j, 0, 0), b(j, 1, 0));
+#pragma unroll
+      for (int p = 0; p < NP - 1; ++p) {
+        const int as = SECOND ? P::a2(p) : P::a1(p), bs = SECOND ? P::b2(p) : P::b1(p);
+        mma16<F16>(c, a[as], b(j, 0, bs), b(j, 1, bs));
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[j][e] += c[e];
+    }
+}
+
+// The power of two 2^k (and 2^-k) that brings the largest |v| of a row of four lanes
+// into [2^14, 2^15); 1 for a row of zeros or of numbers past FP32's range
+__device__ __forceinline__ void row_scale(float m, float& up, float& down) {
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+  const int e = (__float_as_int(m) >> 23) & 0xff;  // |v| < 2^(e - 126)
+  const bool ok = e >= 15 && e <= 240;
+  up = __int_as_float((ok ? 268 - e : 127) << 23);
+  down = __int_as_float((ok ? e - 14 : 127) << 23);
+}
+
 // 8-byte slot of a running sum: a float-float pair while terms are added, an
 // FP64 number when the warps' sums are added
 union Slot {
@@ -137,7 +189,6 @@ template <int D, bool F16>
 __global__ void __launch_bounds__(32 * SmallCfg<D, F16>::NW, SmallCfg<D, F16>::MINB) sigma_small_kernel(SmallDev a) {
   constexpr int NT = SmallCfg<D, F16>::NT, NW = SmallCfg<D, F16>::NW, NSL = F16 ? 2 : 3, TILE = 128 * NSL;
   constexpr int GROUP = 8;           // terms summed in FP32 before each float-float addition
-  using P = Pairs<F16>;
   // running sums, [warp][element of the lane][lane]
   __shared__ Slot acc[NW][NT * 4][32];
   __shared__ int next;
@@ -234,8 +285,6 @@ __global__ void __launch_bounds__(32 * SmallCfg<D, F16>::NW, SmallCfg<D, F16>::M
         cur = tk.in_blk;
       }
       const float sc = (float)tk.scale;
-      // fp16: |X| <= 32 * 2^30 of the scaled operands (2^15 with an identity)
-      const float f = F16 && !idL ? 0x1p-20f : 1.0f, finv = F16 && !idL ? 0x1p20f : 1.0f;
       float x[NT][4];
 #pragma unroll
       for (int j = 0; j < NT; ++j)
@@ -252,11 +301,7 @@ __global__ void __launch_bounds__(32 * SmallCfg<D, F16>::NW, SmallCfg<D, F16>::M
 #pragma unroll
               for (int q = 0; q < 4; ++q) fa[s][q] = trans8(fa[s][q]);
           }
-#pragma unroll
-          for (int p = 0; p < P::N1; ++p)
-#pragma unroll
-            for (int j = 0; j < NT; ++j)
-              if (j < n8) mma16<F16>(x[j], fa[P::a1(p)], fp[2 * ks][j][P::b1(p)], fp[2 * ks + 1][j][P::b1(p)]);
+          mma_step<F16, false, D == 16 && F16>(x, ks == 0, n8, fa, [&](int j, int h, int sl) { return fp[2 * ks + h][j][sl]; });
         }
       } else {  // X = psi (the tile's rows and columns)
 #pragma unroll
@@ -284,6 +329,19 @@ __global__ void __launch_bounds__(32 * SmallCfg<D, F16>::NW, SmallCfg<D, F16>::M
 #pragma unroll
           for (int e = 0; e < 4; ++e) grp[j][e] = fmaf(sc, x[j][e], grp[j][e]);
       } else {  // Y = X R^T
+        // fp16: every row of X on a scale of its own, undone in Y: its elements are
+        // held to 2^-39 of its largest, as the splits hold operands and psi. On one scale
+        // for all (2^-20, from |X| <= 2^35) psi blocks far below max |psi| lost their bits
+        float up[2], down[2] = {1.0f, 1.0f};
+        if (F16) {
+          float mx[2] = {0.0f, 0.0f};
+#pragma unroll
+          for (int j = 0; j < NT; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) mx[e >> 1] = fmaxf(mx[e >> 1], fabsf(x[j][e]));
+#pragma unroll
+          for (int h = 0; h < 2; ++h) row_scale(mx[h], up[h], down[h]);
+        }
         float y[NT][4];
 #pragma unroll
         for (int j = 0; j < NT; ++j)
@@ -305,20 +363,18 @@ __global__ void __launch_bounds__(32 * SmallCfg<D, F16>::NW, SmallCfg<D, F16>::M
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             uint32_t s3[3];
+            const float f = F16 ? up[q & 1] : 1.0f;
             split_pair<F16>(x[2 * ks + (q >> 1)][2 * (q & 1)] * f, x[2 * ks + (q >> 1)][2 * (q & 1) + 1] * f, s3);
 #pragma unroll
             for (int s = 0; s < 3; ++s) fx[s][q] = s3[s];
           }
-#pragma unroll
-          for (int p = 0; p < P::N2; ++p)
-#pragma unroll
-            for (int j = 0; j < NT; ++j)
-              if (j < tn8) mma16<F16>(y[j], fx[P::a2(p)], fr[j][0][P::b2(p)], fr[j][1][P::b2(p)]);
+          mma_step<F16, true, D == 16>(y, ks == 0, tn8, fx, [&](int j, int h, int sl) { return fr[j][h][sl]; });
         }
 #pragma unroll
         for (int j = 0; j < NT; ++j)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) grp[j][e] = fmaf(sc, y[j][e] * finv, grp[j][e]);
+          for (int e = 0; e < 4; ++e)
+            grp[j][e] = fmaf(sc, F16 ? y[j][e] * down[e >> 1] : y[j][e], grp[j][e]);
       }
       if (++ng == GROUP) {
         flush_group();
