@@ -275,29 +275,22 @@ __global__ void scale_kernel(double* __restrict__ x, const double* __restrict__ 
     x[e] *= s;
 }
 
-// Eigenpairs of the symmetric part of the k x k matrix H (row-major, leading
-// dimension ldh) by cyclic Jacobi in round-robin order (Brent-Luk): each
+// Eigenpairs of the symmetric k x k matrix A (shared memory; overwritten) in the
+// basis Q by cyclic Jacobi in round-robin order (Brent-Luk): each
 // round rotates up to 16 disjoint index pairs at once. Four warps share the
 // work (the FP64 rate of one SM sub-partition would otherwise bound it):
 // pair i's rotation is computed by warp i % 4, and every thread applies the
-// rotations of its warp's pairs to its row (and its column). w ascending,
-// Y columns = vectors (Y row-major k x ldh). k <= 32; 128 threads.
+// rotations of its warp's pairs to its row (and its column). w = values + shift
+// ascending, Y columns = vectors Q v (Y row-major k x ldh). k <= 32; 128 threads,
+// which see A and Q (a barrier since they were written).
 constexpr int EIGH_WARPS = 4;
-__device__ void jacobi_eigh(const double* __restrict__ H, int k, int ldh, double* __restrict__ w,
+__device__ void jacobi_eigh(double (*A)[33], double (*Q)[33], int k, int ldh, double shift, double* __restrict__ w,
                             double* __restrict__ Y) {
-  __shared__ double A[32][33];
-  __shared__ double Q[32][33];
   __shared__ double cs[16], sn[16];
   __shared__ int pp[16], qq[16];
   __shared__ double red[2][EIGH_WARPS];
   __shared__ int stop;
   const int tid = threadIdx.x, r = tid & 31, wid = tid >> 5;
-  for (int e = tid; e < k * k; e += blockDim.x) {
-    const int i = e / k, c = e % k;
-    A[i][c] = 0.5 * (H[i * ldh + c] + H[c * ldh + i]);
-    Q[i][c] = i == c ? 1.0 : 0.0;
-  }
-  __syncthreads();
   const int kp = k + (k & 1);            // players, one dummy when k is odd
   const int npairs = kp / 2;
   for (int sweep = 0; sweep < 60 && k > 1; ++sweep) {
@@ -387,14 +380,21 @@ __device__ void jacobi_eigh(const double* __restrict__ H, int k, int ldh, double
       const double u = A[j][j];
       rank += (u < v) || (u == v && j < tid);
     }
-    w[rank] = v;
+    w[rank] = v + shift;
     for (int rr = 0; rr < k; ++rr) Y[rr * ldh + rank] = Q[rr][tid];
   }
 }
 
 __global__ void __launch_bounds__(32 * EIGH_WARPS)
 eigh_full_kernel(const double* __restrict__ H, int k, int ldh, double* __restrict__ w, double* __restrict__ Y) {
-  jacobi_eigh(H, k, ldh, w, Y);
+  __shared__ double A[32][33], Q[32][33];
+  for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
+    const int i = e / k, c = e % k;
+    A[i][c] = 0.5 * (H[i * ldh + c] + H[c * ldh + i]);
+    Q[i][c] = i == c ? 1.0 : 0.0;
+  }
+  __syncthreads();
+  jacobi_eigh(A, Q, k, ldh, 0.0, w, Y);
 }
 
 // Lowest eigenpair of the symmetric part of the k x k matrix H (k <= 32):
@@ -404,27 +404,35 @@ eigh_full_kernel(const double* __restrict__ H, int k, int ldh, double* __restric
 // two barriers per round), warm-started from the previous call's vectors in Yf,
 // and the lowest pair is then refined in FP64: with residual r = H y - theta y,
 // y -= sum_i q_i (q_i . r) / (lambda_i - theta) over the other FP32
-// eigenvectors, which multiplies its error by about 1e-6 per step. Where the
-// lowest two values are closer than FP32 can tell apart, or the residual does
-// not reach FP64 rounding in a few steps, the FP64 Jacobi above decides.
+// eigenvectors, which multiplies its error by about 1e-6 per step, until |r| <=
+// 1e-15 |H|_F, the bound the FP64 Jacobi stops at. Where the lowest two values are
+// closer than FP32 can tell apart, or the residual does not reach it in a few
+// steps, the FP64 Jacobi above decides.
+//
+// All of it on H - H[0][0]: the scale that FP32 and the bounds see is then the
+// spread of the projected spectrum, not a constant in the Hamiltonian (at -88 Ha
+// any gap below 1.8 mHa used to go to the FP64 Jacobi).
 // Per call at K=16, M=150: 40 us (FP64 Jacobi of the whole spectrum: 224 us).
 __global__ void __launch_bounds__(32 * EIGH_WARPS)
 eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restrict__ w, double* __restrict__ Y,
                    float* __restrict__ Yf, int k0) {
   __shared__ double Hs[32][33];
   __shared__ float A[32][33], Q[32][33], T[32][33];
-  __shared__ float cs[16], sn[16];
+  __shared__ float sn[16], th[16];
   __shared__ int pp[16], qq[16];
   __shared__ double part[EIGH_WARPS][32], yv[32], rv[32];
   __shared__ float coef[32], redf[2][EIGH_WARPS];
   __shared__ int state;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nt = 32 * EIGH_WARPS;
   const int kp = k + (k & 1), npairs = kp / 2;  // odd k: one empty row and column
+  const double shift = H[0];
   double mx = 0.0;
   for (int e = tid; e < kp * kp; e += nt) {
     const int i = e / kp, c = e - i * kp;
-    const double h = (i < k && c < k) ? 0.5 * (H[i * ldh + c] + H[c * ldh + i]) : 0.0;
+    double h = 0.0;
+    if (i < k && c < k) h = i == c ? H[i * (ldh + 1)] - shift : 0.5 * (H[i * ldh + c] + H[c * ldh + i]);
     Hs[i][c] = h;
+    Q[i][c] = (i < k0 && c < k0) ? Yf[i * 32 + c] : (i == c ? 1.0f : 0.0f);
     mx = fmax(mx, fabs(h));
   }
   for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -432,11 +440,30 @@ eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restr
   __syncthreads();
   mx = fmax(fmax(part[0][0], part[1][0]), fmax(part[2][0], part[3][0]));
   const int ex = mx > 0.0 ? ilogb(mx) : 0;
-  const double sc = ldexp(1.0, -ex);  // FP32 works on H / 2^ex
+  const double sc = ldexp(1.0, -ex);  // FP32 works on the shifted H / 2^ex
+  // Every fourth call Q <- Q (3 - Q^T Q) / 2 (2.5 us): Q is then orthonormal to 1e-6 or so
+  // whatever the number of calls (8e-5 was seen after 32 calls), below the gap of 2e-5 that the selection asks for
+  const bool again = k0 > 0 && k0 % 4 == 0;
+  if (again) {
+    for (int e = tid; e < kp * kp; e += nt) {
+      const int i = e / kp, c = e - i * kp;
+      float s = 0.0f;
+      for (int j = 0; j < kp; ++j) s = fmaf(Q[j][i], Q[j][c], s);
+      T[i][c] = s;
+    }
+    __syncthreads();
+    for (int e = tid; e < kp * kp; e += nt) {
+      const int i = e / kp, c = e - i * kp;
+      float s = 0.0f;
+      for (int j = 0; j < kp; ++j) s = fmaf(Q[i][j], (j == c ? 1.0f : 0.0f) - T[j][c], s);
+      A[i][c] = fmaf(0.5f, s, Q[i][c]);
+    }
+    __syncthreads();
+  }
   for (int e = tid; e < kp * kp; e += nt) {
     const int i = e / kp, c = e - i * kp;
+    if (again) Q[i][c] = A[i][c];
     A[i][c] = (float)(Hs[i][c] * sc);
-    Q[i][c] = (i < k0 && c < k0) ? Yf[i * 32 + c] : (i == c ? 1.0f : 0.0f);
   }
   __syncthreads();
   if (k0 > 0) {  // A <- Q^T A Q
@@ -467,6 +494,7 @@ eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restr
     bi[u] = i;
     bj[u] = i + x;
   }
+  float fro2 = 0.0f;  // |shifted H|_F^2 / 2^(2 ex)
   for (int sweep = 0; sweep < 10 && k > 1; ++sweep) {
     float off = 0.0f, tot = 0.0f;
     for (int e = tid; e < kp * kp; e += nt) {
@@ -486,6 +514,7 @@ eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restr
     __syncthreads();
     off = redf[0][0] + redf[0][1] + redf[0][2] + redf[0][3];
     tot = redf[1][0] + redf[1][1] + redf[1][2] + redf[1][3];
+    fro2 = tot;
     if (!(off > 1e-11f * tot)) break;
     for (int round = 0; round < kp - 1; ++round) {
       if (tid < npairs) {
@@ -493,27 +522,36 @@ eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restr
         int p = player(tid), q = player(kp - 1 - tid);
         if (p > q) { const int t = p; p = q; q = t; }
         const float apq = A[p][q];
-        float c = 1.0f, sv = 0.0f;
+        // sine and tan(angle / 2): with them a rotation by a small angle is orthogonal to
+        // rounding, where a cosine of FP32 is not
+        float sv = 0.0f, tau = 0.0f;
         if (apq != 0.0f) {
           const float z = (A[q][q] - A[p][p]) / (2.0f * apq), az = fabsf(z);
           const float t = (z >= 0.0f ? 1.0f : -1.0f) * (az > 1e8f ? 0.5f / az : 1.0f / (az + sqrtf(1.0f + az * az)));
-          c = rsqrtf(1.0f + t * t);
+          const float c = rsqrtf(1.0f + t * t);
           sv = t * c;
+          tau = __fdividef(sv, 1.0f + c);
         }
-        cs[tid] = c;
         sn[tid] = sv;
+        th[tid] = tau;
         pp[tid] = p;
         qq[tid] = q;
       }
       __syncthreads();
+      auto rotate = [](float s, float tau, float& x, float& y) {  // x' = c x - s y, y' = s x + c y
+        const float u = fmaf(tau, x, y), v = fmaf(-tau, y, x);
+        x = fmaf(-s, u, x);
+        y = fmaf(s, v, y);
+      };
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         if (tid + u * nt < nblocks) {  // A block (pairs i, j) <- J_i^T block J_j
           const int i = bi[u], j = bj[u], p = pp[i], q = qq[i], r = pp[j], s = qq[j];
-          const float ci = cs[i], si = sn[i], cj = cs[j], sj = sn[j];
-          const float a = A[p][r], b = A[p][s], c = A[q][r], d = A[q][s];
-          const float a1 = cj * a - sj * b, b1 = sj * a + cj * b, c1 = cj * c - sj * d, d1 = sj * c + cj * d;
-          float a2 = ci * a1 - si * c1, b2 = ci * b1 - si * d1, c2 = si * a1 + ci * c1, d2 = si * b1 + ci * d1;
+          float a2 = A[p][r], b2 = A[p][s], c2 = A[q][r], d2 = A[q][s];
+          rotate(sn[j], th[j], a2, b2);
+          rotate(sn[j], th[j], c2, d2);
+          rotate(sn[i], th[i], a2, c2);
+          rotate(sn[i], th[i], b2, d2);
           if (i == j) b2 = c2 = 0.0f;
           A[p][r] = a2;
           A[r][p] = a2;
@@ -527,9 +565,10 @@ eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restr
       }
       for (int e = tid; e < kp * npairs; e += nt) {
         const int i = e / npairs, j = e - i * npairs, p = pp[j], q = qq[j];
-        const float x = Q[i][p], y = Q[i][q];
-        Q[i][p] = cs[j] * x - sn[j] * y;
-        Q[i][q] = sn[j] * x + cs[j] * y;
+        float x = Q[i][p], y = Q[i][q];
+        rotate(sn[j], th[j], x, y);
+        Q[i][p] = x;
+        Q[i][q] = y;
       }
       __syncthreads();
     }
@@ -573,7 +612,7 @@ eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restr
       const double rr = warp_sum(r * r);
       rv[lane] = r;
       if (lane == 0) {
-        const double lim = 1e-15 * (double)k * mx;  // rounding of the residual itself
+        const double lim = 1e-15 * ((double)sqrtf(fro2) / sc);
         state = rr <= lim * lim * yy ? 2 : (step < 6 && rr == rr ? 1 : 0);
       }
       part[0][lane] = theta;
@@ -607,14 +646,21 @@ eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restr
   __syncthreads();
   for (int e = tid; e < k * k; e += nt) Yf[(e / k) * 32 + e % k] = Q[e / k][e % k];
   if (!ok) {
-    jacobi_eigh(H, k, ldh, w, Y);
+    __shared__ double Ad[32][33], Qd[32][33];
+    for (int e = tid; e < k * k; e += nt) {
+      const int i = e / k, c = e % k;
+      Ad[i][c] = Hs[i][c];
+      Qd[i][c] = i == c ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    jacobi_eigh(Ad, Qd, k, ldh, shift, w, Y);
     return;
   }
   if (wid == 0) {
     const double y = yv[lane];
     const double yy = warp_sum(y * y);
     if (lane < k) Y[lane * ldh] = y / sqrt(yy);
-    if (lane == 0) w[0] = theta;
+    if (lane == 0) w[0] = theta + shift;
   }
 }
 
