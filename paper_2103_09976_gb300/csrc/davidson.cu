@@ -407,7 +407,7 @@ eigh_full_kernel(const double* __restrict__ H, int k, int ldh, double* __restric
 // eigenvectors, which multiplies its error by about 1e-6 per step, until |r| <=
 // 1e-15 |H|_F, the bound the FP64 Jacobi stops at. Where the lowest two values are
 // closer than FP32 can tell apart, or the residual does not reach it in a few
-// steps, the FP64 Jacobi above decides.
+// steps, the FP64 Jacobi above decides, started from these vectors.
 //
 // All of it on H - H[0][0]: the scale that FP32 and the bounds see is then the
 // spread of the projected spectrum, not a constant in the Hamiltonian (at -88 Ha
@@ -646,14 +646,42 @@ eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restr
   __syncthreads();
   for (int e = tid; e < k * k; e += nt) Yf[(e / k) * 32 + e % k] = Q[e / k][e % k];
   if (!ok) {
+    // FP64 Jacobi from the FP32 vectors: orthonormal in FP64 after two steps Q <- Q (3 -
+    // Q^T Q) / 2 (1e-6, 1e-12, 1e-24), they leave it two sweeps instead of nine (596 us at
+    // 32 vectors, 1284 from the identity, 1087 by eigh_full_kernel)
     __shared__ double Ad[32][33], Qd[32][33];
+    auto product = [&](double (*X)[33], bool xt, double (*Z)[33], double (*out)[33]) {  // out = X Z or X^T Z
+      for (int e = tid; e < k * k; e += nt) {
+        const int i = e / k, c = e - i * k;
+        double s = 0.0;
+        for (int j = 0; j < k; ++j) s = fma(xt ? X[j][i] : X[i][j], Z[j][c], s);
+        out[i][c] = s;
+      }
+      __syncthreads();
+    };
+    for (int e = tid; e < k * k; e += nt) Qd[e / k][e % k] = (double)Q[e / k][e % k];
+    __syncthreads();
+    for (int step = 0; step < 2; ++step) {
+      product(Qd, true, Qd, Ad);
+      for (int e = tid; e < k * k; e += nt) Ad[e / k][e % k] = (e / k == e % k ? 1.5 : 0.0) - 0.5 * Ad[e / k][e % k];
+      __syncthreads();
+      product(Qd, false, Ad, Hs);
+      for (int e = tid; e < k * k; e += nt) Qd[e / k][e % k] = Hs[e / k][e % k];
+      __syncthreads();
+    }
     for (int e = tid; e < k * k; e += nt) {
-      const int i = e / k, c = e % k;
-      Ad[i][c] = Hs[i][c];
-      Qd[i][c] = i == c ? 1.0 : 0.0;
+      const int i = e / k, c = e - i * k;
+      Hs[i][c] = i == c ? H[i * (ldh + 1)] - shift : 0.5 * (H[i * ldh + c] + H[c * ldh + i]);
     }
     __syncthreads();
-    jacobi_eigh(Ad, Qd, k, ldh, shift, w, Y);
+    product(Hs, false, Qd, Ad);
+    product(Qd, true, Ad, Hs);
+    for (int e = tid; e < k * k; e += nt) {
+      const int i = e / k, c = e - i * k;
+      if (c < i) Hs[i][c] = Hs[c][i] = 0.5 * (Hs[i][c] + Hs[c][i]);
+    }
+    __syncthreads();
+    jacobi_eigh(Hs, Qd, k, ldh, shift, w, Y);
     return;
   }
   if (wid == 0) {

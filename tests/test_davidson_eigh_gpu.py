@@ -56,3 +56,8 @@ def test_time_does_not_depend_on_a_constant(run, gap):
     _, (plain, _) = run(0.0, gap)
     _, (shifted, _) = run(-1e4, gap)
     assert shifted <= 1.5 * plain, (plain, shifted)
+
+
+def test_close_pairs_start_the_fp64_jacobi_from_the_fp32_vectors(run):
+    _, (lowest, full) = run(0.0, 1e-12)
+    assert lowest <= 0.7 * full, (lowest, full)
