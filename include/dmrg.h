@@ -252,7 +252,8 @@ dmrg_status dmrg_sigma_noalloc(dmrg_ctx* ctx, int site, const double* psi, doubl
  * item split and largest-first order of the persistent kernel's work items,
  * Sec. II.D-E collapsed into one list) on a seeded psi, keeps the fastest
  * and reports it. Mixed precision (BF16X3 / BF16X2 / FP16X2): times the
- * tensor-core path for {4, 8, 16, 32} items per SM x {1, 4, 16} x 2^20
+ * tensor-core path with the setting in force (the default below, or an earlier
+ * call's choice) and with {4, 8, 16, 32} items per SM x {1, 4, 16} x 2^20
  * multiply-adds of fixed cost per unit of stacked terms (how each output
  * tile's units are split into work items and ordered, largest first) and
  * reports the choice in items_per_sm and per_task_cost; then, unless

@@ -152,6 +152,12 @@ static void prepare_tc_plan(Context& c, Problem& p) {
   ++p.tc_plan_gen;
 }
 
+// Items per SM of the tensor-core plan, the tuned number or the one by the units.
+static int tc_items_reported(const Context& c, const Problem& p) {
+  if (p.tc_items_per_sm > 0) return p.tc_items_per_sm;
+  return p.tc_plan_ready ? std::max(1, p.tc.want_items / c.n_sm) : 16;
+}
+
 // Split jobs: every stored block in store order, then the identity blocks of
 // the left and of the right sectors (the order of the plan's split-block
 // indices).
@@ -823,9 +829,7 @@ dmrg_status dmrg_get_sigma_info(dmrg_ctx* ctx, int site, dmrg_sigma_info* info) 
     info->op_elements = p.L.elements + p.R.elements;
     info->op_bytes_read = p.wl.bytes_ops;
     info->psi_size = p.psi_size;
-    info->tc_items_per_sm = p.tc_items_per_sm > 0 ? p.tc_items_per_sm
-                            : p.tc_plan_ready      ? std::max(1, p.tc.want_items / ctx->c.n_sm)
-                                                   : 16;
+    info->tc_items_per_sm = tc_items_reported(ctx->c, p);
     info->tc_producers = ctx->c.opts.tc_producers > 0 ? ctx->c.opts.tc_producers
                                                        : p.tc_producers[ctx->c.opts.sigma_prec == DMRG_FP16X2 ? 1 : 0];
     info->tc_unit_cost = p.tc_unit_cost;
@@ -859,12 +863,9 @@ dmrg_status dmrg_autotune(dmrg_ctx* ctx, int site, int* items_per_sm, double* pe
     DMRG_CUDA(cudaEventCreate(&e1));
     if (c.opts.sigma_prec != DMRG_FP64) {
       // tensor-core path: items per SM of the persistent kernel (the split
-      // of each output tile's units into items, largest first)
+      // of each output tile's units into items, largest first) x fixed unit
+      // cost of that split
       if (!tc_ready_for(p, c.opts.sigma_prec)) prepare_tc(c, p);
-      // items per SM x fixed unit cost (in multiply-adds: 1 / 4 / 16 MMAs of
-      // 128 x 128 x 64) of the item split
-      const int cand[4] = {4, 8, 16, 32};
-      const double ucand[3] = {128.0 * 128 * 64, 4 * 128.0 * 128 * 64, 16 * 128.0 * 128 * 64};
       const int g = c.opts.sigma_prec == DMRG_FP16X2 ? 1 : 0;
       double best = 1e300;
       int bi = p.tc_items_per_sm;
@@ -880,19 +881,18 @@ dmrg_status dmrg_autotune(dmrg_ctx* ctx, int site, int* items_per_sm, double* pe
         return ms;
       };
       try {
-        for (double uc : ucand)
-          for (int wi : cand) {
-            p.tc_items_per_sm = wi;
-            p.tc_unit_cost = uc;
-            prepare_tc_plan(c, p);
-            prepare_tc(c, p);  // FP16X2: records of the new plan
-            const float ms = time_one();
-            if (ms < best) {
-              best = ms;
-              bi = wi;
-              bu = uc;
-            }
+        for (const TcSetting& s : tc_settings({bi, bu})) {
+          p.tc_items_per_sm = s.items_per_sm;
+          p.tc_unit_cost = s.unit_cost;
+          prepare_tc_plan(c, p);
+          prepare_tc(c, p);  // FP16X2: records of the new plan
+          const float ms = time_one();
+          if (ms < best) {
+            best = ms;
+            bi = s.items_per_sm;
+            bu = s.unit_cost;
           }
+        }
         p.tc_items_per_sm = bi;
         p.tc_unit_cost = bu;
         prepare_tc_plan(c, p);
@@ -916,7 +916,7 @@ dmrg_status dmrg_autotune(dmrg_ctx* ctx, int site, int* items_per_sm, double* pe
       cudaEventDestroy(e0);
       cudaEventDestroy(e1);
       check_device_error(c, p);
-      if (items_per_sm) *items_per_sm = bi;
+      if (items_per_sm) *items_per_sm = tc_items_reported(c, p);
       if (per_task_cost) *per_task_cost = bu;
       if (best_ms) *best_ms = best;
       return;

@@ -436,6 +436,13 @@ namespace dmrg {
 static inline int ceil8(int x) { return (x + 7) / 8; }
 static inline int up16(int x) { return (x + 15) & ~15; }
 
+std::vector<TcSetting> tc_settings(const TcSetting& now) {
+  std::vector<TcSetting> v{now};
+  for (double mmas : {1.0, 4.0, 16.0})
+    for (int items : {4, 8, 16, 32}) v.push_back({items, mmas * (128.0 * 128 * 64)});
+  return v;
+}
+
 void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const OpSet& R,
                    const WorkList& wl, TcPlan& plan, const TcShape& shape) {
   plan = TcPlan();

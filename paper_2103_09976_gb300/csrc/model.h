@@ -384,6 +384,14 @@ struct TcShape {
   int n_sm = 152;           // SMs that share the small-class items
   int small_max = TC_SMALL_MAX;  // widest blocks of the small classes (TC_SMALL_MAX or TC_MEDIUM_MAX)
 };
+// Settings that the autotuner times: `now` (items per SM 0: by the number of
+// units) first, so that a tuned plan is never one that timed slower than the
+// plan it replaces, then 4 to 32 items per SM by 1, 4 and 16 MMAs of 128 x 128 x 64.
+struct TcSetting {
+  int items_per_sm;
+  double unit_cost;
+};
+std::vector<TcSetting> tc_settings(const TcSetting& now);
 void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const OpSet& R,
                    const WorkList& wl, TcPlan& plan, const TcShape& shape);
 

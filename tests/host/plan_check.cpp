@@ -424,6 +424,14 @@ int main(int argc, char** argv) {
     }
   }
 
+  // the autotuner times the setting in force before any other, and each of these once
+  const std::vector<TcSetting> tune = tc_settings({0, 1048576.0});
+  if (tune.size() != 13 || tune[0].items_per_sm != 0 || tune[0].unit_cost != 1048576.0) fail("settings of the autotuner");
+  for (size_t a = 0; a < tune.size(); ++a)
+    for (size_t b = 0; b < a; ++b)
+      if (tune[a].items_per_sm == tune[b].items_per_sm && tune[a].unit_cost == tune[b].unit_cost)
+        fail("setting of the autotuner twice");
+
   // bytes the FP64 kernel requests per sigma: for every (item, task) the
   // output tile's rows of the left block, the psi block and the tile's
   // columns of the right block (identities are not read)
