@@ -128,12 +128,15 @@ void prepare_worklist(Context& c, Problem& p) {
 
 static_assert(sizeof(TcItem) == sizeof(Item), "reduction reads TcItem as Item");
 
+static TcShape tc_shape(const Context& c, const Problem& p) {
+  return TcShape{c.n_sm * p.tc_items_per_sm, p.tc_unit_cost, c.n_sm, TC_MEDIUM_MAX};
+}
+
 // Work records of the tensor-core path for the problem's tuning (the split
 // operator store is unchanged by it).
 static void prepare_tc_plan(Context& c, Problem& p) {
   cudaStream_t st = c.stream;
-  build_tc_plan(p.blocks, p.L, p.R, p.wl, p.tc,
-                TcShape{c.n_sm * p.tc_items_per_sm, p.tc_unit_cost, c.n_sm, TC_MEDIUM_MAX});
+  build_tc_plan(p.blocks, p.L, p.R, p.wl, p.tc, tc_shape(c, p));
   p.d_tc_recs.upload(p.tc.recs, st);
   p.d_tc_items.upload(p.tc.items, st);
   p.d_tc_small.upload(p.tc.small, st);
@@ -155,7 +158,8 @@ static void prepare_tc_plan(Context& c, Problem& p) {
 // Items per SM of the tensor-core plan, the tuned number or the one by the units.
 static int tc_items_reported(const Context& c, const Problem& p) {
   if (p.tc_items_per_sm > 0) return p.tc_items_per_sm;
-  return p.tc_plan_ready ? std::max(1, p.tc.want_items / c.n_sm) : 16;
+  const int want = p.tc_plan_ready ? p.tc.want_items : tc_want_items(p.blocks, p.wl, tc_shape(c, p));
+  return std::max(1, want / c.n_sm);
 }
 
 // Split jobs: every stored block in store order, then the identity blocks of

@@ -436,6 +436,62 @@ namespace dmrg {
 static inline int ceil8(int x) { return (x + 7) / 8; }
 static inline int up16(int x) { return (x + 15) & ~15; }
 
+namespace {
+
+// Size classes of the plan: which terms leave the tensor cores, and how many
+// items the units of the others are split into.
+struct Classes {
+  int small_max;
+  long long n_small[3] = {0, 0, 0};  // terms per small class
+  int want_items = 0;
+  // terms of an (output block, psi block) pair: -1 tensor cores, 0 all blocks <= TC_SMALL_MID,
+  // 1 <= TC_SMALL_MAX, 2 <= TC_MEDIUM_MAX
+  int of(const PsiBlock& ob, const PsiBlock& ib) const {
+    const int wmax = std::max(std::max(ob.mL, ob.mR), std::max(ib.mL, ib.mR));
+    return wmax > small_max ? -1 : wmax <= TC_SMALL_MID ? 0 : wmax <= TC_SMALL_MAX ? 1 : 2;
+  }
+};
+
+Classes size_classes(const std::vector<PsiBlock>& blocks, const WorkList& wl, const TcShape& shape) {
+  Classes cl;
+  cl.small_max = shape.small_max;
+  for (size_t b = 0; b < blocks.size(); ++b)
+    for (int t = wl.out_start[b]; t < wl.out_start[b + 1]; ++t) {
+      const int cls = cl.of(blocks[b], blocks[wl.tasks[t].in_blk]);
+      if (cls >= 0) ++cl.n_small[cls];
+    }
+  // the <= 64 class needs enough terms to fill the GPU by itself; fewer join the
+  // tensor cores' items, which run anyway (at K=16, M=150 a kernel of their own
+  // takes 35 us and their partial tiles 18 us of the reduction, and the
+  // tensor-core kernel is 17 us faster without them)
+  constexpr int MEDIUM_TERMS_PER_SM = 64;
+  if (cl.n_small[2] < (long long)MEDIUM_TERMS_PER_SM * shape.n_sm) cl.small_max = std::min(cl.small_max, TC_SMALL_MAX);
+  double n_units = 0;
+  for (size_t b = 0; b < blocks.size(); ++b) {
+    const PsiBlock& ob = blocks[b];
+    long long n = 0;
+    for (int t = wl.out_start[b]; t < wl.out_start[b + 1]; ++t) n += cl.of(ob, blocks[wl.tasks[t].in_blk]) < 0;
+    for (int r0 = 0; r0 < ob.mL; r0 += 128)
+      n_units += (double)n * ((ob.mR + 127) / 128) / std::max(1, 16 / ((std::min(128, ob.mL - r0) + 7) / 8));
+  }
+  // Items: an even finish wants many per SM, but each costs a partial tile
+  // written and reduced and a start. 16 per SM where they hold 40 units or more,
+  // at least 2. Kernel per sigma with 4 / 8 / 16 / 32 per SM (three producers):
+  // 23.8 / 19.8 / 18.7 / 18.6 ms at K=76, M=4000, 5.6 / 4.7 / 4.6 / 4.6 ms at K=108,
+  // M=2000 (reduction 0.03 / 0.05 / 0.10 / 0.19 ms); solves at K=16, M=150: 313 us per
+  // product with 4, 298 with 2, 301 with 1.
+  cl.want_items = shape.want_items > 0
+                      ? shape.want_items
+                      : (int)std::min(16.0 * shape.n_sm, std::max(2.0 * shape.n_sm, n_units / 40));
+  return cl;
+}
+
+}  // namespace
+
+int tc_want_items(const std::vector<PsiBlock>& blocks, const WorkList& wl, const TcShape& shape) {
+  return size_classes(blocks, wl, shape).want_items;
+}
+
 std::vector<TcSetting> tc_settings(const TcSetting& now) {
   std::vector<TcSetting> v{now};
   for (double mmas : {1.0, 4.0, 16.0})
@@ -568,29 +624,8 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
     return s1 + G * s2;
   };
   const double unit_overhead = shape.unit_cost;  // fixed cost of a unit in the item split
-  double total = 0, n_units = 0;
-  // size class of the terms of (output block, psi block): -1 tensor cores, 0 all blocks <= TC_SMALL_MID,
-  // 1 <= TC_SMALL_MAX, 2 <= TC_MEDIUM_MAX
-  int small_max = shape.small_max;
-  auto small_class = [&](const PsiBlock& ob, int in_blk) {
-    const PsiBlock& ib = blocks[in_blk];
-    const int wmax = std::max(std::max(ob.mL, ob.mR), std::max(ib.mL, ib.mR));
-    return wmax > small_max ? -1 : wmax <= TC_SMALL_MID ? 0 : wmax <= TC_SMALL_MAX ? 1 : 2;
-  };
-  long long n_small[3] = {0, 0, 0};  // terms per small class
-  for (size_t b = 0; b < nblk; ++b) {
-    const PsiBlock& ob = blocks[b];
-    for (int t = wl.out_start[b]; t < wl.out_start[b + 1]; ++t) {
-      const int cls = small_class(ob, base[t].in_blk);
-      if (cls >= 0) ++n_small[cls];
-    }
-  }
-  // the <= 64 class needs enough terms to fill the GPU by itself; fewer join the
-  // tensor cores' items, which run anyway (at K=16, M=150 a kernel of their own
-  // takes 35 us and their partial tiles 18 us of the reduction, and the
-  // tensor-core kernel is 17 us faster without them)
-  constexpr int MEDIUM_TERMS_PER_SM = 64;
-  if (n_small[2] < (long long)MEDIUM_TERMS_PER_SM * shape.n_sm) small_max = std::min(small_max, TC_SMALL_MAX);
+  const Classes cl = size_classes(blocks, wl, shape);
+  double total = 0;
   for (size_t b = 0; b < nblk; ++b) {
     const PsiBlock& ob = blocks[b];
     for (int r0 = 0; r0 < ob.mL; r0 += 128)
@@ -598,22 +633,13 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
         const int tm = std::min(128, ob.mL - r0), tn = std::min(128, ob.mR - c0);
         const int G = std::max(1, 16 / ceil8(tm));
         for (int t = wl.out_start[b]; t < wl.out_start[b + 1]; ++t) {
-          if (small_class(ob, base[t].in_blk) >= 0) continue;  // not part of the tensor-core items
+          if (cl.of(ob, blocks[base[t].in_blk]) >= 0) continue;  // not part of the tensor-core items
           const TcPsiBlock& ib = plan.psi[base[t].in_blk];
           total += unit_macs(1, tn, ib.m, ib.n) / G + unit_overhead / G;
-          n_units += 1.0 / G;
         }
       }
   }
-  // Items: an even finish wants many per SM, but each costs a partial tile
-  // written and reduced and a start. 16 per SM where they hold 40 units or more,
-  // at least 2. Kernel per sigma with 4 / 8 / 16 / 32 per SM (three producers):
-  // 23.8 / 19.8 / 18.7 / 18.6 ms at K=76, M=4000, 5.6 / 4.7 / 4.6 / 4.6 ms at K=108,
-  // M=2000 (reduction 0.03 / 0.05 / 0.10 / 0.19 ms); solves at K=16, M=150: 313 us per
-  // product with 4, 298 with 2, 301 with 1.
-  plan.want_items = shape.want_items > 0
-                        ? shape.want_items
-                        : (int)std::min(16.0 * shape.n_sm, std::max(2.0 * shape.n_sm, n_units / 40));
+  plan.want_items = cl.want_items;
   const double target = total / plan.want_items;
 
   struct Unit {  // one unit: positions [t0, t1) of its part's sorted task order
@@ -638,9 +664,9 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
   // The <= 64 class (12 warps, one CTA per SM) holds one psi block per item in
   // shared memory: 6 items per SM.
   int small_item[3];
-  small_item[0] = (int)std::min<long long>(512, std::max<long long>(32, n_small[0] / (shape.n_sm * 14)));
-  small_item[1] = (int)std::min<long long>(512, std::max<long long>(16, n_small[1] / (shape.n_sm * 8)));
-  small_item[2] = (int)std::min<long long>(512, std::max<long long>(1, n_small[2] / (shape.n_sm * 6)));
+  small_item[0] = (int)std::min<long long>(512, std::max<long long>(32, cl.n_small[0] / (shape.n_sm * 14)));
+  small_item[1] = (int)std::min<long long>(512, std::max<long long>(16, cl.n_small[1] / (shape.n_sm * 8)));
+  small_item[2] = (int)std::min<long long>(512, std::max<long long>(1, cl.n_small[2] / (shape.n_sm * 6)));
   std::vector<Part> parts(nparts);
   in_parallel([&](int j) {
     Part& P = parts[j];
@@ -682,7 +708,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
             while (e < kend && base[P.order[e]].in_blk == h.in_blk && (base[P.order[e]].flags & 3) == (h.flags & 3)) ++e;
             const TcPsiBlock& ib = plan.psi[h.in_blk];
             // small class: the whole output block (one tile) and the psi block are small
-            const int cls = small_class(ob, h.in_blk);
+            const int cls = cl.of(ob, blocks[h.in_blk]);
             if (cls >= 0) {
               for (int q = k; q < e; ++q) {
                 const Base& x = base[P.order[q]];

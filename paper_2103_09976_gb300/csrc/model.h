@@ -384,6 +384,8 @@ struct TcShape {
   int n_sm = 152;           // SMs that share the small-class items
   int small_max = TC_SMALL_MAX;  // widest blocks of the small classes (TC_SMALL_MAX or TC_MEDIUM_MAX)
 };
+// Kind-0 items that a plan of this shape aims at (TcPlan::want_items), without building it.
+int tc_want_items(const std::vector<PsiBlock>& blocks, const WorkList& wl, const TcShape& shape);
 // Settings that the autotuner times: `now` (items per SM 0: by the number of
 // units) first, so that a tuned plan is never one that timed slower than the
 // plan it replaces, then 4 to 32 items per SM by 1, 4 and 16 MMAs of 128 x 128 x 64.

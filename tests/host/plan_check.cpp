@@ -58,6 +58,17 @@ int main(int argc, char** argv) {
   if (argc > 7 && std::string(argv[7]) == "medium") shape.small_max = TC_MEDIUM_MAX;
   build_tc_plan(blocks, oL, oR, wl, plan, shape);
 
+  // items the plan aims at, with and without the plan: fixed, and by the number of units
+  if (plan.want_items != shape.want_items) fail("items asked for");
+  {
+    TcShape by_units = shape;
+    by_units.want_items = 0;
+    TcPlan q;
+    build_tc_plan(blocks, oL, oR, wl, q, by_units);
+    if (q.want_items != tc_want_items(blocks, wl, by_units)) fail("items with and without the plan");
+    if (q.want_items < 2 * by_units.n_sm || q.want_items > 16 * by_units.n_sm) fail("items by the number of units");
+  }
+
   // (0) FP64 work list: groups tile every output block into 32 x 256 tiles;
   //     the items of a group split the block's task range in order; slots
   //     are consecutive; the schedule is a permutation

@@ -24,6 +24,7 @@ def test_small_plan_takes_two_items_per_sm():
             capi.dmrg_load_synthetic(ctx, 4, 8, 4, 0, left, right, 5)
             n = capi.dmrg_psi_layout(ctx)["size"]
             x, y = random_unit_vector(n, 6), np.full(n, np.nan)
+            assert capi.dmrg_get_sigma_info(ctx)["tc_items_per_sm"] == 2   # what the plan will take
             capi.dmrg_sigma(ctx, -1, x, y)
             info = capi.dmrg_get_sigma_info(ctx)
         finally:
