@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <exception>
 #include <functional>
 #include <numeric>
 #include <thread>
@@ -234,6 +235,31 @@ static int resolve(const OpDesc& op, const Basis& b, int qin, bool trans, const 
   return qout;
 }
 
+// fn(0) .. fn(n - 1), a thread each. Parts whose thread cannot be started run
+// on this one; an exception of a part comes out here, after all have ended.
+static void run_parts(int n, const std::function<void(int)>& fn) {
+  std::vector<std::exception_ptr> err(n);
+  auto part = [&](int j) {
+    try {
+      fn(j);
+    } catch (...) {
+      err[j] = std::current_exception();
+    }
+  };
+  std::vector<std::thread> pool;
+  pool.reserve(n);
+  int here = 1;  // parts from this one on, and part 0, run on this thread
+  try {
+    for (; here < n; ++here) pool.emplace_back(part, here);
+  } catch (...) {  // no thread to be had, or no memory for one
+  }
+  part(0);
+  for (int j = here; j < n; ++j) part(j);
+  for (std::thread& t : pool) t.join();
+  for (const std::exception_ptr& e : err)
+    if (e) std::rethrow_exception(e);
+}
+
 void build_tasks(const std::vector<PsiBlock>& blocks, const OpSet& L, const OpSet& R,
                  const std::vector<Term>& terms, WorkList& wl) {
   // output block index by left sector
@@ -306,13 +332,7 @@ void build_tasks(const std::vector<PsiBlock>& blocks, const OpSet& L, const OpSe
     th_flops[th] = flops;
     th_bytes[th] = bytes;
   };
-  if (nth == 1) {
-    work(0);
-  } else {
-    std::vector<std::thread> pool;
-    for (int th = 0; th < nth; ++th) pool.emplace_back(work, th);
-    for (auto& x : pool) x.join();
-  }
+  run_parts(nth, work);
   double flops = 0, bytes = 0;
   for (int th = 0; th < nth; ++th) {
     flops += th_flops[th];
@@ -564,18 +584,9 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
                          wl.out_start.begin());
     bstart[j] = std::max(bstart[j], bstart[j - 1]);
   }
-  auto in_parallel = [&](const std::function<void(int)>& fn) {
-    if (nparts == 1) {
-      fn(0);
-      return;
-    }
-    std::vector<std::thread> pool;
-    for (int j = 0; j < nparts; ++j) pool.emplace_back(fn, j);
-    for (auto& x : pool) x.join();
-  };
   std::vector<Base> base(wl.tasks.size());
   std::vector<char> bad(nparts, 0);
-  in_parallel([&](int j) {
+  run_parts(nparts, [&](int j) {
     for (int t = wl.out_start[bstart[j]]; t < wl.out_start[bstart[j + 1]]; ++t) {
       const Task& k = wl.tasks[t];
       const PsiBlock& in = blocks[k.in_blk];
@@ -668,7 +679,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
   small_item[1] = (int)std::min<long long>(512, std::max<long long>(16, cl.n_small[1] / (shape.n_sm * 8)));
   small_item[2] = (int)std::min<long long>(512, std::max<long long>(1, cl.n_small[2] / (shape.n_sm * 6)));
   std::vector<Part> parts(nparts);
-  in_parallel([&](int j) {
+  run_parts(nparts, [&](int j) {
     Part& P = parts[j];
     std::vector<unsigned long long> keys;
     for (size_t b = bstart[j]; b < bstart[j + 1]; ++b) {
@@ -798,7 +809,7 @@ void build_tc_plan(const std::vector<PsiBlock>& blocks, const OpSet& L, const Op
   plan.small_blk.resize(2 * SM[nparts]);
   plan.n_units = 0;
   std::vector<double> icost(I[nparts]);
-  in_parallel([&](int j) {
+  run_parts(nparts, [&](int j) {
     const Part& P = parts[j];
     std::copy(P.small.begin(), P.small.end(), plan.small.begin() + SM[j]);
     std::copy(P.small_blk.begin(), P.small_blk.end(), plan.small_blk.begin() + 2 * SM[j]);
