@@ -6,7 +6,9 @@
 // dedicated work list (see sweep.cpp).
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "kernels.h"
 
@@ -913,6 +915,36 @@ bool svd_cluster_fits(int d, int m) {
   const int npairs = (d + 1) / 2, ppc = (npairs + SVD_CLUSTER - 1) / SVD_CLUSTER;
   return d >= 1 && d <= 32 * SVD_REG && m <= 32 * SVD_REG && ppc <= SVD_CLUSTER_WARPS &&
          (size_t)ppc * 4 * (m + d + 1) * sizeof(double) <= SVD_CLUSTER_SMEM;
+}
+
+SvdShape plan_svd_blocks(const std::vector<SvdDims>& dims, bool clusters, std::vector<SvdBlock>& sb) {
+  SvdShape s;
+  s.nb = (int)dims.size();
+  sb.resize(dims.size());
+  std::vector<int> cl;  // blocks of the cluster kernel
+  for (int b = 0; b < s.nb; ++b) {
+    const int d = dims[b].d, m = dims[b].m, dp = d + (d & 1);
+    const bool fits = clusters && svd_cluster_fits(d, m);
+    sb[b] = {dims[b].psi_off, s.q_elems, s.w_elems, s.work_elems, s.work_elems + (long long)d * m, d, m,
+             s.grid_pairs, dp / 2, dp - 1, fits ? 1 : 0, 0, 0};
+    if (fits) {
+      const int ppc = (dp / 2 + SVD_CLUSTER - 1) / SVD_CLUSTER;
+      s.cluster_warps = std::max(s.cluster_warps, ppc);
+      s.cluster_smem = std::max(s.cluster_smem, (int)(ppc * 4 * (m + d + 1) * sizeof(double)));
+      cl.push_back(b);
+    } else {
+      s.grid_pairs += dp / 2;
+      s.grid_rounds = std::max(s.grid_rounds, dp - 1);
+    }
+    s.max_d = std::max(s.max_d, d);
+    s.work_elems += (long long)d * m + (long long)d * d;
+    s.q_elems += (long long)d * d;
+    s.w_elems += d;
+  }
+  std::stable_sort(cl.begin(), cl.end(), [&](int a, int b) { return sb[a].d > sb[b].d; });  // the longest first
+  for (size_t i = 0; i < cl.size(); ++i) sb[i].order = cl[i];
+  s.n_cluster = (int)cl.size();
+  return s;
 }
 
 void launch_svd_blocks(const double* psi, const SvdBlock* sb, const SvdShape& shape, double* Q, double* w, double* work,

@@ -163,9 +163,9 @@ struct BlockingDev {
   int left;                     // 1: block x site, 0: site x block
   int* err;                     // set to 1 on an inconsistent term
 };
-struct GramBlock {      // one psi block for decimation / one block to orthonormalise
-  long long psi_off, g_off, w_off;
-  int d, m;             // Gram dimension and contracted dimension (or d x m columns)
+struct GramBlock {      // a block to orthonormalise
+  long long g_off;
+  int d, m;             // m columns of length d
 };
 struct TakeBlock {      // dst (d x k) = first k columns of Q (d x d)
   long long q_off, dst_off;
@@ -190,11 +190,12 @@ void launch_bgemm(const double* A, const double* B, double* C, const GJob* jobs,
 void launch_opcomb(const double* src, const long long* xoff, const double* coef, const CombClass* cls, int ncls,
                    int ntiles, double* dst, cudaStream_t st);
 // Per psi block: singular vectors of its d-dimensional side (rows when left,
-// columns otherwise) and squared singular values, by one-sided Jacobi over
-// the whole GPU (one cooperative launch for all blocks): Q (d x d row-major,
+// columns otherwise) and squared singular values, by one-sided Jacobi (a
+// cluster of CTAs per block, or one cooperative launch for the blocks that no
+// cluster holds): Q (d x d row-major,
 // columns = vectors) and w (d values), by descending singular value. Work
 // space: 64 doubles, then A (d x m) and V (d x d) of every block at a_off /
-// v_off. max_d_hint >= every d (shared memory of the final sort).
+// v_off.
 struct SvdBlock {
   long long psi_off, q_off, w_off, a_off, v_off;
   int d, m, pair0, npairs, rounds;
@@ -211,7 +212,14 @@ struct SvdShape {
   int nb = 0, max_d = 1;
   int grid_pairs = 0, grid_rounds = 0;                    // of the grid-wide kernel's blocks
   int n_cluster = 0, cluster_warps = 1, cluster_smem = 0;  // blocks, warps and shared memory of a CTA
+  long long q_elems = 0, w_elems = 0, work_elems = 64;    // doubles of Q, w and the work space
 };
+struct SvdDims {  // a psi block: offset, dimension of the side whose vectors are wanted, the other one
+  long long psi_off;
+  int d, m;
+};
+// Offsets and kernels of all blocks; clusters = false: every block on the grid-wide kernel.
+SvdShape plan_svd_blocks(const std::vector<SvdDims>& dims, bool clusters, std::vector<SvdBlock>& sb);
 void launch_svd_blocks(const double* psi, const SvdBlock* sb, const SvdShape& shape, double* Q, double* w, double* work,
                        bool left, int n_sm, cudaStream_t st);
 void launch_orthonormalize(double* store, const GramBlock* gb, int nb, cudaStream_t st);

@@ -383,50 +383,27 @@ struct Decim {
 void decimate(Context& c, Problem& p, const Enlarged& E, const double* psi, int M, bool forward, Decim& D) {
   cudaStream_t st = c.stream;
   const int nb = (int)p.blocks.size();
-  std::vector<GramBlock> gb(nb);   // Q / w offsets and the two dimensions of every block
-  std::vector<SvdBlock> sb(nb);
-  long long goff = 0, woff = 0, aoff = 64;
-  SvdShape shape;
-  shape.nb = nb;
-  std::vector<int> cl;  // blocks of the cluster kernel
+  std::vector<SvdDims> dims(nb);
   for (int b = 0; b < nb; ++b) {
     const PsiBlock& pb = p.blocks[b];
-    const int d = forward ? pb.mL : pb.mR, m = forward ? pb.mR : pb.mL;
-    gb[b] = {pb.off, goff, woff, d, m};
-    const int dp = d + (d & 1);
-    const bool fits = svd_cluster_fits(d, m);
-    sb[b] = {pb.off, goff, woff, aoff, aoff + (long long)d * m, d, m, shape.grid_pairs, dp / 2, dp - 1, fits ? 1 : 0, 0, 0};
-    if (fits) {
-      const int ppc = (dp / 2 + SVD_CLUSTER - 1) / SVD_CLUSTER;
-      shape.cluster_warps = std::max(shape.cluster_warps, ppc);
-      shape.cluster_smem = std::max(shape.cluster_smem, (int)(ppc * 4 * (m + d + 1) * sizeof(double)));
-      cl.push_back(b);
-    } else {
-      shape.grid_pairs += dp / 2;
-      shape.grid_rounds = std::max(shape.grid_rounds, dp - 1);
-    }
-    shape.max_d = std::max(shape.max_d, d);
-    aoff += (long long)d * m + (long long)d * d;
-    goff += (long long)d * d;
-    woff += d;
+    dims[b] = {pb.off, forward ? pb.mL : pb.mR, forward ? pb.mR : pb.mL};
   }
-  std::stable_sort(cl.begin(), cl.end(), [&](int a, int b) { return sb[a].d > sb[b].d; });
-  for (size_t i = 0; i < cl.size(); ++i) sb[i].order = cl[i];
-  shape.n_cluster = (int)cl.size();
+  std::vector<SvdBlock> svd;
+  const SvdShape shape = plan_svd_blocks(dims, true, svd);
   DevBuf dsb, Q, W, work;
-  dsb.upload(sb, st);
-  Q.alloc(std::max<long long>(1, goff) * sizeof(double));
-  W.alloc(std::max<long long>(1, woff) * sizeof(double));
-  work.alloc((size_t)aoff * sizeof(double));
+  dsb.upload(svd, st);
+  Q.alloc(std::max<long long>(1, shape.q_elems) * sizeof(double));
+  W.alloc(std::max<long long>(1, shape.w_elems) * sizeof(double));
+  work.alloc((size_t)shape.work_elems * sizeof(double));
   {
     ProfScope ps(c.prof, 3, st);
     launch_svd_blocks(psi, dsb.as<SvdBlock>(), shape, Q.as<double>(), W.as<double>(), work.as<double>(), forward,
                       c.n_sm, st);
   }
   DMRG_CUDA(cudaGetLastError());
-  std::vector<double> w(woff);
+  std::vector<double> w(shape.w_elems);
   unsigned int flags[16] = {};
-  DMRG_CUDA(cudaMemcpyAsync(w.data(), W.p, woff * sizeof(double), cudaMemcpyDeviceToHost, st));
+  DMRG_CUDA(cudaMemcpyAsync(w.data(), W.p, w.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   DMRG_CUDA(cudaMemcpyAsync(flags, work.p, sizeof(flags), cudaMemcpyDeviceToHost, st));
   DMRG_CUDA(cudaStreamSynchronize(st));
   if (flags[SVD_LOST]) throw Error(DMRG_ECUDA, "decimation: a wait of the SVD kernel ran out");
@@ -435,7 +412,7 @@ void decimate(Context& c, Problem& p, const Enlarged& E, const double* psi, int 
   for (int b = 0; b < nb; ++b) {
     const PsiBlock& pb = p.blocks[b];
     const int r = std::min(pb.mL, pb.mR);
-    for (int i = 0; i < r; ++i) sv[b].push_back(std::sqrt(std::max(0.0, w[gb[b].w_off + i])));
+    for (int i = 0; i < r; ++i) sv[b].push_back(std::sqrt(std::max(0.0, w[svd[b].w_off + i])));
     qLs[b] = p.L.basis.q[pb.qL];
   }
   const std::vector<int> kept = select_kept(sv, qLs, M, c.opts.keep_one_per_q != 0, &D.discarded);
@@ -457,8 +434,8 @@ void decimate(Context& c, Problem& p, const Enlarged& E, const double* psi, int 
     D.nb.dim.push_back(kept[b]);
     D.esec_of_new.push_back(forward ? p.blocks[b].qL : p.blocks[b].qR);
     D.uoff.push_back(uo);
-    tb.push_back({gb[b].g_off, uo, gb[b].d, kept[b]});
-    uo += (long long)gb[b].d * kept[b];
+    tb.push_back({svd[b].q_off, uo, svd[b].d, kept[b]});
+    uo += (long long)svd[b].d * kept[b];
   }
   D.nb.finish();
   (void)E;
@@ -599,7 +576,7 @@ void sweep_build_blocks(Context& c, const double* t, const double* v, int K, int
       Dm.nb.dim.push_back(m[a]);
       Dm.esec_of_new.push_back(comp[a]);
       Dm.uoff.push_back(uo);
-      gb.push_back({0, uo, 0, d, m[a]});
+      gb.push_back({uo, d, m[a]});
       uo += (long long)d * m[a];
     }
     Dm.nb.finish();

@@ -59,32 +59,18 @@ int main(int argc, char** argv) {
   CK(cudaMalloc(&dwork, (64 + no + nq) * 8));
   CK(cudaMalloc(&dsb, nb * sizeof(SvdBlock)));
   CK(cudaMemcpy(dpsi, psi.data(), no * 8, cudaMemcpyHostToDevice));
+  std::vector<SvdDims> dims(nb);
+  for (int b = 0; b < nb; ++b) dims[b] = {off[b], D[b], M[b]};
   std::vector<double> W[2], Q(nq);
   std::vector<int> cls(nb);
   for (int run = 1; run >= 0; --run) {  // 1: all grid-wide, 0: as the rule picks
-    std::vector<SvdBlock> sb(nb);
-    std::vector<int> cl;
-    SvdShape sh;
-    sh.nb = nb;
-    for (int b = 0; b < nb; ++b) {
-      const int d = D[b], m = M[b], dp = d + (d & 1);
-      const bool fits = run == 0 && svd_cluster_fits(d, m);
-      sb[b] = {off[b], qoff[b], woff[b], 64 + off[b] + qoff[b], 64 + off[b] + qoff[b] + (long long)d * m,
-               d, m, sh.grid_pairs, dp / 2, dp - 1, fits ? 1 : 0, 0, 0};
-      cls[b] = fits;
-      if (fits) {
-        const int ppc = (dp / 2 + SVD_CLUSTER - 1) / SVD_CLUSTER;
-        sh.cluster_warps = std::max(sh.cluster_warps, ppc);
-        sh.cluster_smem = std::max(sh.cluster_smem, (int)(ppc * 4 * (m + d + 1) * sizeof(double)));
-        cl.push_back(b);
-      } else {
-        sh.grid_pairs += dp / 2;
-        sh.grid_rounds = std::max(sh.grid_rounds, dp - 1);
-      }
-      sh.max_d = std::max(sh.max_d, d);
+    std::vector<SvdBlock> sb;
+    const SvdShape sh = plan_svd_blocks(dims, run == 0, sb);
+    if (sh.q_elems != nq || sh.w_elems != nw || sh.work_elems != 64 + no + nq) {
+      fprintf(stderr, "sizes of the plan\n");
+      return 1;
     }
-    for (size_t i = 0; i < cl.size(); ++i) sb[i].order = cl[i];
-    sh.n_cluster = (int)cl.size();
+    for (int b = 0; b < nb; ++b) cls[b] = sb[b].cluster;
     CK(cudaMemcpy(dsb, sb.data(), nb * sizeof(SvdBlock), cudaMemcpyHostToDevice));
     launch_svd_blocks(dpsi, dsb, sh, dQ, dw, dwork, left, n_sm, 0);
     CK(cudaGetLastError());
