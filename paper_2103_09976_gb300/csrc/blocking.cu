@@ -7,9 +7,11 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <string>
 #include <type_traits>
 #include <vector>
 
+#include "../../include/dmrg.h"
 #include "kernels.h"
 
 namespace dmrg {
@@ -917,6 +919,37 @@ bool svd_cluster_fits(int d, int m) {
          (size_t)ppc * 4 * (m + d + 1) * sizeof(double) <= SVD_CLUSTER_SMEM;
 }
 
+// Launch of n clusters; the kernel's attributes are set on the way.
+static cudaLaunchConfig_t cluster_config(int n, int warps, int smem, cudaStream_t st, cudaLaunchAttribute& at) {
+  set_max_dynamic_smem((const void*)svd_cluster_kernel, (int)SVD_CLUSTER_SMEM);
+  const cudaError_t e = cudaFuncSetAttribute((const void*)svd_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) throw Error(DMRG_ECUDA, std::string("cudaFuncSetAttribute(cluster size): ") + cudaGetErrorString(e));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)n * SVD_CLUSTER);
+  cfg.blockDim = dim3(32u * warps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = SVD_CLUSTER;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+bool svd_clusters_launch() {
+  int n = 0;
+  try {
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = cluster_config(1, SVD_CLUSTER_WARPS, (int)SVD_CLUSTER_SMEM, nullptr, at);
+    if (cudaOccupancyMaxActiveClusters(&n, svd_cluster_kernel, &cfg) != cudaSuccess) n = 0;
+  } catch (const Error&) {
+  }
+  if (n <= 0) cudaGetLastError();  // the answer, not an error of the caller's
+  return n > 0;
+}
+
 SvdShape plan_svd_blocks(const std::vector<SvdDims>& dims, bool clusters, std::vector<SvdBlock>& sb) {
   SvdShape s;
   s.nb = (int)dims.size();
@@ -955,21 +988,8 @@ void launch_svd_blocks(const double* psi, const SvdBlock* sb, const SvdShape& sh
   if (sig_bytes > 48 * 1024) set_max_dynamic_smem((const void*)svd_finish_kernel, (int)sig_bytes);
   if (cudaMemsetAsync(work, 0, 64, st) != cudaSuccess) return;  // the flags of both kernels; the caller's cudaGetLastError reports it
   if (shape.n_cluster > 0) {
-    set_max_dynamic_smem((const void*)svd_cluster_kernel, (int)SVD_CLUSTER_SMEM);
-    if (cudaFuncSetAttribute((const void*)svd_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-        cudaSuccess)
-      return;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)shape.n_cluster * SVD_CLUSTER);
-    cfg.blockDim = dim3(32u * shape.cluster_warps);
-    cfg.dynamicSmemBytes = shape.cluster_smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = SVD_CLUSTER;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute at;
+    cudaLaunchConfig_t cfg = cluster_config(shape.n_cluster, shape.cluster_warps, shape.cluster_smem, st, at);
     if (cudaLaunchKernelEx(&cfg, svd_cluster_kernel, sb, psi, work, left ? 1 : 0) != cudaSuccess) return;
   }
   if (total_pairs > 0 && max_rounds > 0) {

@@ -208,6 +208,9 @@ constexpr int SVD_CLUSTER_WARPS = 16;             // most warps, one pair each, 
 constexpr size_t SVD_CLUSTER_SMEM = 220 * 1024;   // most shared memory of a CTA
 constexpr int SVD_LOST = 8;  // 32-bit word of the work area: not zero when a wait of the cluster kernel ran out
 bool svd_cluster_fits(int d, int m);
+// Whether a cluster of the largest kind can be placed on the current device: a
+// GPU shared out in parts may have no SVD_CLUSTER SMs that form one.
+bool svd_clusters_launch();
 struct SvdShape {
   int nb = 0, max_d = 1;
   int grid_pairs = 0, grid_rounds = 0;                    // of the grid-wide kernel's blocks

@@ -389,7 +389,7 @@ void decimate(Context& c, Problem& p, const Enlarged& E, const double* psi, int 
     dims[b] = {pb.off, forward ? pb.mL : pb.mR, forward ? pb.mR : pb.mL};
   }
   std::vector<SvdBlock> svd;
-  const SvdShape shape = plan_svd_blocks(dims, true, svd);
+  const SvdShape shape = plan_svd_blocks(dims, svd_clusters_launch(), svd);
   DevBuf dsb, Q, W, work;
   dsb.upload(svd, st);
   Q.alloc(std::max<long long>(1, shape.q_elems) * sizeof(double));

@@ -59,6 +59,10 @@ int main(int argc, char** argv) {
   CK(cudaMalloc(&dwork, (64 + no + nq) * 8));
   CK(cudaMalloc(&dsb, nb * sizeof(SvdBlock)));
   CK(cudaMemcpy(dpsi, psi.data(), no * 8, cudaMemcpyHostToDevice));
+  if (!svd_clusters_launch()) {
+    fprintf(stderr, "no cluster can be placed\n");
+    return 1;
+  }
   std::vector<SvdDims> dims(nb);
   for (int b = 0; b < nb; ++b) dims[b] = {off[b], D[b], M[b]};
   std::vector<double> W[2], Q(nq);
