@@ -915,7 +915,8 @@ namespace dmrg {
 
 bool svd_cluster_fits(int d, int m) {
   const int npairs = (d + 1) / 2, ppc = (npairs + SVD_CLUSTER - 1) / SVD_CLUSTER;
-  return d >= 1 && d <= 32 * SVD_REG && m <= 32 * SVD_REG && ppc <= SVD_CLUSTER_WARPS &&
+  static_assert((32 * SVD_REG / 2 + SVD_CLUSTER - 1) / SVD_CLUSTER == SVD_CLUSTER_WARPS, "a warp for every pair of a CTA");
+  return d >= 1 && d <= 32 * SVD_REG && m <= 32 * SVD_REG &&
          (size_t)ppc * 4 * (m + d + 1) * sizeof(double) <= SVD_CLUSTER_SMEM;
 }
 

@@ -204,7 +204,7 @@ struct SvdBlock {
   int pad;
 };
 constexpr int SVD_CLUSTER = 16;                   // CTAs of a cluster
-constexpr int SVD_CLUSTER_WARPS = 16;             // most warps, one pair each, of a CTA
+constexpr int SVD_CLUSTER_WARPS = 8;              // most warps, one pair each, of a CTA (256 columns over 16 CTAs)
 constexpr size_t SVD_CLUSTER_SMEM = 220 * 1024;   // most shared memory of a CTA
 constexpr int SVD_LOST = 8;  // 32-bit word of the work area: not zero when a wait of the cluster kernel ran out
 bool svd_cluster_fits(int d, int m);
