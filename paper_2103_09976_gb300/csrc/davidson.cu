@@ -142,16 +142,6 @@ __global__ void __launch_bounds__(DT) dots_kernel(DotSet a, DotSet b, long long 
   if (threadIdx.x < k) d.out[(long long)threadIdx.x * d.stride] = s;
 }
 
-// 1 / d for a preconditioner: FP32 start and two Newton steps (within an ulp
-// or two), plain division outside FP32's range
-__device__ __forceinline__ double fast_rcp(double d) {
-  const double a = fabs(d);
-  if (!(a > 1e-30 && a < 1e30)) return 1.0 / d;
-  double r = (double)(1.0f / (float)d);
-  r = fma(r, fma(-d, r, 1.0), r);
-  return fma(r, fma(-d, r, 1.0), r);
-}
-
 // One pass over the subspace after the projected eigenproblem: Ritz vector
 // x = sum_i y_i V_i and ax = sum_i y_i AV_i, residual r = ax - theta x,
 // preconditioned direction t = r / clamp(theta - diag), r . r, and the
@@ -185,7 +175,7 @@ ritz_kernel(const double* __restrict__ V, const double* __restrict__ AV, long lo
     rr = fma(re, re, rr);
     double den = th - diag[e];
     if (fabs(den) < 1e-8) den = den < 0.0 ? -1e-8 : 1e-8;
-    const double te = re * fast_rcp(den);
+    const double te = re / den;
     t[e] = te;
 #pragma unroll
     for (int i = 0; i < KB; ++i)
