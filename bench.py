@@ -68,14 +68,12 @@ def config(M, prec="fp64"):
             "l2": "inputs larger than L2 (operator store >> 129 MB), no flush"}
 
 
-# DRAM bytes per sigma at M=2000, from ncu captures of the small case M=800
-# scaled by the bytes each kernel requests (counted with the kernels' own
-# formulas by tests/host/plan_check.cpp) at both sizes:
-# profiles/sigma_f64_middle_bond_m800_dram.md, sigma_mixed_middle_bond_m800_dram.md.
-F64_TRAFFIC_M2000 = 70.0e9
-MIXED_TRAFFIC_M2000 = {"bf16x3": 32.4e9, "bf16x2": 32.4e9, "fp16x2": 20.6e9}
-TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum at M=800 (small case) per requested byte, "
-                  "times the requested bytes at M=2000")
+# DRAM bytes of one sigma's product kernels at M=2000 with the default work
+# split, counted by ncu in a single pass: profiles/sigma_middle_bond_m2000_dram.md.
+F64_TRAFFIC_M2000 = 61.0e9
+MIXED_TRAFFIC_M2000 = {"bf16x3": 27.5e9, "bf16x2": 27.4e9, "fp16x2": 18.1e9}
+TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one sigma at M=2000, default split "
+                  "(profiles/sigma_middle_bond_m2000_dram.md)")
 
 # ------------------------------------------------------------------ clocks
 class Clocks:
@@ -414,7 +412,7 @@ def main():
                        "roofline": {"bound": "hbm", "achieved": alg_bytes / kern / 1e9, "peak": hbm,
                                     "unit": "GB/s", "frac": alg_bytes / kern / 1e9 / hbm, "traffic": traffic,
                                     "traffic_source": TRAFFIC_SOURCE if traffic else None,
-                                    "kernel": "sigma_small_kernel + sigma_tc_kernel (one sigma)",
+                                    "kernel": "sigma_small_kernel + sigma_medium_kernel + sigma_tc_kernel (one sigma)",
                                     "peak_source": "MEASURED_PEAKS.json hbm_gbs",
                                     "tensor_tflops_issued": nprod * flops / kern / 1e12,
                                     "tensor_frac_of_bf16_peak": nprod * flops / kern / 1e12 / bf16}}
@@ -435,7 +433,7 @@ def main():
            "roofline": {"bound": "alu", "achieved": achieved, "peak": peak64, "unit": "TFLOP/s",
                         "frac": achieved / peak64,
                         "traffic": F64_TRAFFIC_M2000 if args.M == 2000 else None,
-                        "traffic_source": TRAFFIC_SOURCE + " (profiles/sigma_f64_middle_bond_m800_dram.md)",
+                        "traffic_source": TRAFFIC_SOURCE if args.M == 2000 else None,
                         "kernel": "sigma_f64_kernel",
                         "peak_source": "cuBLAS DGEMM 4096^3 measured in this run (no FP64 entry in MEASURED_PEAKS.json); "
                                        "cross-check: measured bf16 x nominal FP64/bf16 ratio = "

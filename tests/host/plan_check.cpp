@@ -444,33 +444,48 @@ int main(int argc, char** argv) {
         fail("setting of the autotuner twice");
 
   // bytes the FP64 kernel requests per sigma: for every (item, task) the
-  // output tile's rows of the left block, the psi block and the tile's
-  // columns of the right block (identities are not read)
+  // output tile's rows of the left block, and, for every row slice of the tile (16
+  // rows up to 128 columns, 8 rows of wider tiles; one warp each), the psi block
+  // and the tile's columns of the right block (identities are not read)
   double f64_req = 0.0;
-  for (const Item& it : wl.items)
+  for (const Item& it : wl.items) {
+    const int rows = it.ncols <= 128 ? 16 : 8, slices = (it.nrows + rows - 1) / rows;
     for (int t = it.t_begin; t < it.t_end; ++t) {
       const Task& k = wl.tasks[t];
       const PsiBlock& ib = blocks[k.in_blk];
-      f64_req += 8.0 * ((k.aoff >= 0 ? (double)it.nrows * ib.mL : 0.0) + (double)ib.mL * ib.mR +
-                        (k.boff >= 0 ? (double)it.ncols * ib.mR : 0.0));
+      f64_req += 8.0 * ((k.aoff >= 0 ? (double)it.nrows * ib.mL + (double)slices * ib.mL * ib.mR
+                                     : (double)it.nrows * ib.mR) +
+                        (k.boff >= 0 ? (double)slices * it.ncols * ib.mR : 0.0));
     }
-  // tile positions the small-class kernels read per sigma: each term's left
-  // and right blocks, and its psi block once per warp and run of terms of
-  // one psi block (warps take every 8th (<= 16 class) or 4th term)
-  long long small_tiles = 0;
+  }
+  // tile positions the small-class kernels read per sigma. Kinds 1 and 2: four
+  // warps, each 16 rows of its terms (two warps share a term of more rows): the
+  // rows' tiles of the left block (of psi where that is the identity), the right
+  // block, and psi when the warp's psi block changes. Kind 3: psi once per item,
+  // both blocks of a term once.
+  long long small_tiles = 0, medium_tiles = 0;
   for (const TcItem& it : plan.items) {
+    const int tm8 = (it.nrows + 7) / 8, tn8 = (it.ncols + 7) / 8;
+    if (it.kind == 3) {
+      const TcPsiBlock& pb = plan.psi[plan.small[it.r_begin].in_blk];
+      const int m8 = (pb.m + 7) / 8, n8 = (pb.n + 7) / 8;
+      medium_tiles += (long long)pb.R8 * pb.C8;
+      for (int k = it.r_begin; k < it.r_end; ++k)
+        medium_tiles += (plan.small[k].a_tile >= 0 ? tm8 * m8 : 0) + (plan.small[k].b_tile >= 0 ? tn8 * n8 : 0);
+    }
     if (it.kind != 1 && it.kind != 2) continue;
-    const int nw = it.kind == 2 ? 8 : 4;
-    for (int w = 0; w < nw; ++w) {
+    const int n_rows = it.nrows > 16 ? 2 : 1;
+    for (int w = 0; w < 4; ++w) {
+      const int rows = std::min(2, tm8 - 2 * (w % n_rows));
       int cur = -1;
-      for (int k = it.r_begin + w; k < it.r_end; k += nw) {
+      for (int k = it.r_begin + w / n_rows; k < it.r_end; k += 4 / n_rows) {
         const SmallTerm& x = plan.small[k];
         const TcPsiBlock& pb = plan.psi[x.in_blk];
-        const int m = pb.m, n = pb.n, tm = it.nrows, tn = it.ncols;
-        if (x.in_blk != cur) small_tiles += (long long)pb.R8 * pb.C8;
+        const int m8 = (pb.m + 7) / 8, n8 = (pb.n + 7) / 8;
+        if (x.in_blk != cur) small_tiles += (long long)m8 * n8;
         cur = x.in_blk;
-        if (x.a_tile >= 0) small_tiles += (long long)((tm + 7) / 8) * ((m + 7) / 8);
-        if (x.b_tile >= 0) small_tiles += (long long)((tn + 7) / 8) * ((n + 7) / 8);
+        small_tiles += x.a_tile >= 0 ? rows * m8 : std::min(rows, m8 - 2 * (w % n_rows)) * n8;
+        if (x.b_tile >= 0) small_tiles += (long long)tn8 * n8;
       }
     }
   }
@@ -478,10 +493,12 @@ int main(int argc, char** argv) {
               "\"plan_tasks\": %lld, \"units\": %lld, \"items\": %zu, \"mma_s1\": %lld, \"mma_s2\": %lld, "
               "\"stages\": %lld, \"medium_items\": %d, \"op_elements\": %lld, \"f64_request_bytes\": %.17g, "
               "\"tc_copy_bytes_bf16\": %lld, \"tc_copy_bytes_fp16\": %lld, \"small_read_bytes_bf16\": %lld, "
-              "\"small_read_bytes_fp16\": %lld, \"layout\": [",
+              "\"small_read_bytes_fp16\": %lld, \"medium_copy_bytes_bf16\": %lld, \"medium_copy_bytes_fp16\": %lld, "
+              "\"layout\": [",
               size, blocks.size(), terms.size(), wl.tasks.size(), wl.flops, plan.n_terms, plan.n_units,
               plan.items.size(), mma_s1, mma_s2, stages, plan.n_medium, (long long)(oL.elements + oR.elements), f64_req,
-              copy_tiles[0] * 384, copy_tiles[1] * 256, small_tiles * 384, small_tiles * 256);
+              copy_tiles[0] * 384, copy_tiles[1] * 256, small_tiles * 384, small_tiles * 256, medium_tiles * 384,
+              medium_tiles * 256);
   for (size_t b = 0; b < blocks.size(); ++b) {
     const PsiBlock& pb = blocks[b];
     std::printf("%s[%d, %d, %d, %d, %d, %d, %lld]", b ? ", " : "", L.q[pb.qL].n, L.q[pb.qL].s, R.q[pb.qR].n,
