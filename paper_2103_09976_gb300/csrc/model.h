@@ -348,7 +348,7 @@ struct TcPlan {
   long long scratch_elems = 0;
   int max_tile = 0;                     // elements of the largest group's tile
   std::vector<TcUnitRec, NoInit<TcUnitRec>> recs;  // kind-0 item i: records [items[i].r_begin, items[i].r_end)
-  std::vector<SmallTerm> small;         // kind-1/2 item i: terms [items[i].r_begin, items[i].r_end)
+  std::vector<SmallTerm> small;         // item i of kind 1, 2 or 3: terms [items[i].r_begin, items[i].r_end)
   // per record and term slot (record * TC_MAX_G + q): split-block indices of
   // the left and right blocks (stored blocks in store order, then the
   // identity blocks of the left and right sectors); -1 for unused slots

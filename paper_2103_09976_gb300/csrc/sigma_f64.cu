@@ -417,7 +417,7 @@ void launch_sigma_f64(const SigmaDev& a, int n_sm, cudaStream_t st) {
 void launch_reduce(const SigmaDev& a, cudaStream_t st) {
   if (a.n_groups < 1 || a.max_tile < 1) return;
   // a CTA per run of elements until that fills the GPU many times over (a
-  // transformation has one group per operator block, 1e5 and more)
+  // plan has one group per output tile: a few for small bonds, thousands for large ones)
   int ny = (a.max_tile + RED_THREADS - 1) / RED_THREADS;
   ny = std::min(ny, std::max(1, 152 * 64 / a.n_groups));
   const dim3 grid((unsigned)a.n_groups, (unsigned)ny);

@@ -1,5 +1,5 @@
 """GPU parity of the mixed-precision sigma (bf16-slice products on tcgen05,
-small classes on the CUDA cores) against the CPU oracle and against the FP64
+small classes on warp-level matrix instructions) against the CPU oracle and against the FP64
 GPU path, through the C ABI.
 
 Tolerances follow from the arithmetic. BF16X3 represents every operand to
@@ -43,7 +43,7 @@ def _oracle_full(left, right, nL, n, Q, seed, x):
 
 @pytest.mark.parametrize("prec", [2, 1, 3])
 @pytest.mark.parametrize("M,nsp,ntot,seed", [
-    (24, 3, 6, 1),        # tiny blocks: every class on the CUDA cores
+    (24, 3, 6, 1),        # tiny blocks: every class on warp-level instructions
     (120, 4, 8, 2),
     (1200, 3, 6, 3),      # blocks up to 107: several stage-1 stages, two 64-column halves
     (4000, 3, 6, 4),      # blocks up to 355: several 128-row / 128-column tiles, 3 psi chunks
