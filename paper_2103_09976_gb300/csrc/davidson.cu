@@ -402,7 +402,7 @@ eigh_full_kernel(const double* __restrict__ H, int k, int ldh, double* __restric
 // All of it on H - H[0][0]: the scale that FP32 and the bounds see is then the
 // spread of the projected spectrum, not a constant in the Hamiltonian (at -88 Ha
 // any gap below 1.8 mHa used to go to the FP64 Jacobi).
-// Per call at K=16, M=150: 40 us (FP64 Jacobi of the whole spectrum: 224 us).
+// Per call at K=16, M=150: 43 us (FP64 Jacobi of the whole spectrum: 224 us).
 __global__ void __launch_bounds__(32 * EIGH_WARPS)
 eigh_lowest_kernel(const double* __restrict__ H, int k, int ldh, double* __restrict__ w, double* __restrict__ Y,
                    float* __restrict__ Yf, int k0) {

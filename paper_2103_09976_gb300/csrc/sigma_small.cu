@@ -20,19 +20,19 @@
 // on the summed slices or less (mma_step). The fp16 split (hi + lo) takes all four
 // products in the first product and, with X as three fp16 slices, five in the second
 // (lo x the third slice, below 2^-33, is left out); every row of X is scaled so that
-// its largest element fills the range of fp16 (row_scale). The bf16 split (hi + mid +
+// its largest element fills the range of fp16 (row_scales). The bf16 split (hi + mid +
 // lo) takes the six products above 2^-24 in both, X as three bf16 slices; what is left
 // out is below 2^-25. Terms of a warp are summed in FP32 over groups of 8, groups in
 // float-float (48 bits), warps in FP64 in warp order, so the result does not depend on
 // scheduling.
 //
 // Bound by instruction issue (<= 16: 65% of issue slots) and load latency (<= 32:
-// 12-16 warps per SM of 128-159 registers); a term of 16 x 16 blocks reads 2-3 KB
+// 12-16 warps per SM of 128-162 registers); a term of 16 x 16 blocks reads 2-3 KB
 // for 18-24 matrix instructions. So a warp takes 16 rows (a term of more rows is
 // shared by two), CTAs are 4 warps, items come from a counter, the next term's
 // record is loaded a term ahead and its L and R before psi and the first product.
 // Both kernels per sigma, against FP32 multiply-adds from shared memory: 1.63 ->
-// 0.96 ms at K=108, M=2000 (FP16X2), 0.74 -> 0.40 ms at K=54, M=1000 (BF16X2), 63
+// 0.92 ms at K=108, M=2000 (FP16X2), 0.74 -> 0.39 ms at K=54, M=1000 (BF16X2), 63
 // -> 46 us at K=24, M=250.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -131,51 +131,75 @@ struct Pairs<false> {  // hl, mm, lh, hm, mh, hh
 // b(j, h, s): slice s of K tile h. The matrix instruction adds with truncation
 // (measured: operands aligned to the largest exponent with two extra bits, the
 // result cut to 24), so a sum left to it shrinks by up to a unit in the last place
-// an instruction, always in one direction. Hence hi x hi of every K step goes to a
-// fresh accumulator z, the other products to c, and FP32 additions, which round to
-// nearest, join them. REST: c starts with hi x hi on top of -z, which gives what was
-// cut off (to a quarter unit); the <= 16 class needs it, where FP32 multiply-adds
-// round a few times only. Relative error of sigma against 64 bits (2-norm, 1e-7), one
-// accumulator / these parts / FP32 multiply-adds of the summed slices: bf16 slices
-// 1.0 / 0.7 / 0.9 at K=8, M=60 (blocks up to 4 wide), 1.0 / 0.7 / 1.0 at K=24, M=200 (10),
-// 3.3 / 0.8 / 1.4 at K=36, M=500 (25); fp16 1.3 / 1.0 / 1.0, 1.2 / 0.9 / 1.2, 2.5 / 1.3 / 1.5.
-// Time of a sigma: 706 -> 734 us at K=54, M=1000 (BF16X2), 7.17 -> 7.29 ms at K=108, M=2000
-// (FP16X2); taking the N tiles one after another keeps z and c in registers.
+// an instruction, always in one direction. Hence every K step has its own
+// accumulator z, corrections first and hi x hi last, one cut at full size, and FP32
+// additions, which round to nearest, join the steps. REST: z starts with hi x
+// hi on top of its own negative, which gives what was cut off (to a quarter unit); the
+// <= 16 class needs it, where FP32 multiply-adds round a few times only. Relative
+// error of sigma against 64 bits (2-norm, 1e-7), one accumulator / these parts / FP32
+// multiply-adds of the summed slices: bf16 slices 1.0 / 0.8 / 0.9 at K=8, M=60 (blocks up to 4
+// wide), 1.0 / 0.8 / 1.0 at K=24, M=200 (10), 3.3 / 1.1 / 1.4 at K=36, M=500 (25); fp16 1.3 / 1.0 /
+// 1.0, 1.2 / 0.9 / 1.2, 2.5 / 1.2 / 1.5. Time of a sigma, one accumulator and one scale for
+// all X -> this: 806 -> 812 us at K=54, M=1000 (BF16X2), 7.45 -> 7.56 ms at K=108, M=2000 (FP16X2),
+// launched without a graph.
 template <bool F16, bool SECOND, bool REST, int NT, int NSA, class Frag>
 __device__ __forceinline__ void mma_step(float (&x)[NT][4], bool first, int nj, const uint32_t (&a)[NSA][4],
                                          Frag&& b) {
   using P = Pairs<F16>;
   constexpr int NP = SECOND ? P::N2 : P::N1;
+  if (!REST) {
+    float z[NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) z[j][e] = 0.0f;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      const int as = SECOND ? P::a2(p) : P::a1(p), bs = SECOND ? P::b2(p) : P::b1(p);
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+        if (j < nj) mma16<F16>(z[j], a[as], b(j, 0, bs), b(j, 1, bs));
+    }
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[j][e] = first ? z[j][e] : x[j][e] + z[j][e];
+    return;
+  }
 #pragma unroll
   for (int j = 0; j < NT; ++j)
     if (j == 0 || j < nj) {
-      float z[4] = {0.0f, 0.0f, 0.0f, 0.0f}, c[4];
+      float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};
       mma16<F16>(z, a[0], b(j, 0, 0), b(j, 1, 0));
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        c[e] = REST ? -z[e] : 0.0f;
         x[j][e] = first ? z[e] : x[j][e] + z[e];
+        z[e] = -z[e];
       }
-      if (REST) mma16<F16>(c, a[0], b(j, 0, 0), b(j, 1, 0));
+      mma16<F16>(z, a[0], b(j, 0, 0), b(j, 1, 0));
 #pragma unroll
       for (int p = 0; p < NP - 1; ++p) {
         const int as = SECOND ? P::a2(p) : P::a1(p), bs = SECOND ? P::b2(p) : P::b1(p);
-        mma16<F16>(c, a[as], b(j, 0, bs), b(j, 1, bs));
+        mma16<F16>(z, a[as], b(j, 0, bs), b(j, 1, bs));
       }
 #pragma unroll
-      for (int e = 0; e < 4; ++e) x[j][e] += c[e];
+      for (int e = 0; e < 4; ++e) x[j][e] += z[e];
     }
 }
 
-// The power of two 2^k (and 2^-k) that brings the largest |v| of a row of four lanes
-// into [2^14, 2^15); 1 for a row of zeros or of numbers past FP32's range
-__device__ __forceinline__ void row_scale(float m, float& up, float& down) {
-  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-  const int e = (__float_as_int(m) >> 23) & 0xff;  // |v| < 2^(e - 126)
-  const bool ok = e >= 15 && e <= 240;
-  up = __int_as_float((ok ? 268 - e : 127) << 23);
-  down = __int_as_float((ok ? e - 14 : 127) << 23);
+// Powers of two 2^k (and 2^-k) that bring the largest |v| of each of the two rows of
+// four lanes into [2^14, 2^15) (as near as FP32's exponents allow). Only the
+// exponents matter, so both rows' go through the two shuffles in one word.
+__device__ __forceinline__ void row_scales(float m0, float m1, float (&up)[2], float (&down)[2]) {
+  unsigned m = __float_as_uint(m0) >> 23 | (__float_as_uint(m1) >> 23) << 16;
+  m = __vmaxu2(m, __shfl_xor_sync(0xffffffffu, m, 1));
+  m = __vmaxu2(m, __shfl_xor_sync(0xffffffffu, m, 2));
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const unsigned e = min(max((m >> (16 * h)) & 0xff, 15u), 240u) << 23;  // |v| < 2^(e - 126)
+    up[h] = __uint_as_float((268u << 23) - e);
+    down[h] = __uint_as_float(e - (14u << 23));
+  }
 }
 
 // 8-byte slot of a running sum: a float-float pair while terms are added, an
@@ -339,8 +363,7 @@ __global__ void __launch_bounds__(32 * SmallCfg<D, F16>::NW, SmallCfg<D, F16>::M
           for (int j = 0; j < NT; ++j)
 #pragma unroll
             for (int e = 0; e < 4; ++e) mx[e >> 1] = fmaxf(mx[e >> 1], fabsf(x[j][e]));
-#pragma unroll
-          for (int h = 0; h < 2; ++h) row_scale(mx[h], up[h], down[h]);
+          row_scales(mx[0], mx[1], up, down);
         }
         float y[NT][4];
 #pragma unroll
