@@ -205,9 +205,9 @@ typedef struct {
   long long op_elements;
   double op_bytes_read;
   long long psi_size;
-  /* tensor-core plan setting at this site for the context's precision
-     (after the plan is built by a mixed-precision sigma or dmrg_autotune;
-     defaults before): items per SM, producer warps, unit cost */
+  /* tensor-core plan setting at this site for the context's precision:
+     items per SM (of the plan that a mixed-precision sigma builds, or that
+     dmrg_autotune chose), producer warps, unit cost */
   int tc_items_per_sm;
   int tc_producers;
   double tc_unit_cost;
