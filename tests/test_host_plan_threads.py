@@ -1,5 +1,5 @@
 """Task and plan construction where no thread can be started: the same lists,
-built on the calling thread. The checker runs with a thread stack (its stack
+built on the calling thread. The program runs with a thread stack (its stack
 limit) larger than the address space it may use."""
 
 import json
